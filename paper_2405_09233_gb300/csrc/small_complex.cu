@@ -16,191 +16,342 @@
 namespace ts {
 namespace {
 
+// Squares of entries whose squared modulus lies in this range neither overflow nor lose bits.
+constexpr double kSqLo = 1e-280, kSqHi = 1e280;
+__device__ __forceinline__ double cnorm(double2 z) { return fma(z.y, z.y, z.x * z.x); }
+// a - b c in four FP64 instructions.
+__device__ __forceinline__ double2 cfms(double2 a, double2 b, double2 c) {
+  return make_double2(fma(b.y, c.y, fma(-b.x, c.x, a.x)), fma(-b.y, c.x, fma(-b.x, c.y, a.y)));
+}
+__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {   // a + b c
+  return make_double2(fma(-b.y, c.y, fma(b.x, c.x, a.x)), fma(b.y, c.x, fma(b.x, c.y, a.y)));
+}
+__device__ __forceinline__ double2 crecip(double2 z) {
+  const double n = cnorm(z);
+  if (n >= kSqLo && n <= kSqHi) {
+    const double d = 1.0 / n;
+    return make_double2(z.x * d, -z.y * d);
+  }
+  return cdiv(make_double2(1.0, 0.0), z);
+}
+
 // LU with partial pivoting of M = H_k - t_jj I, lower bandwidth bw, one CTA per (j, k).
-// LU[(k*s + j)] is an N x N column-major factor; piv holds the row chosen at each step.  Per column
-// c: warp 0 finds the pivot among rows c..c+bw (shuffle argmax, first index on ties), swaps it into
-// column c, and forms the multipliers (kept in column c, and the first kLuMaxBw in shared memory);
-// then every thread takes columns q > c, applies the row interchange to its column and subtracts
-// the multipliers times M[c, q] down the band: two barriers per column.  (The first version reduced
-// the pivot candidates of all 256 threads serially and used five barriers per column.)
-constexpr int kLuMaxBw = 256;
-__global__ void __launch_bounds__(256) k_shifted_lu(const double2* __restrict__ H, long long sH,
-                                                    const double2* __restrict__ T, double2* __restrict__ LU,
-                                                    int* __restrict__ piv, int N, int bw, int s, int* err) {
+// LU[(k*s + j)] is an N x N column-major factor; piv holds the row chosen at each step.
+//
+// GB300 issues an FP64 instruction of one warp in 64 clocks, so the serial part of a column (pivot
+// search, reciprocal, multipliers: one warp) costs as much as many columns of the update.  Interval c
+// therefore overlaps them: warps 1-7 apply column c (row interchange, then M[r, q] -= l_r u_q, a warp
+// per column and a lane per row, so that a column's band is read in whole lines) to the columns
+// q >= c + 2, while warp 0 applies it to column c + 1, finds that column's pivot and forms its
+// multipliers; one barrier per column.  Pivots are compared by squared modulus as bit patterns (an
+// integer comparison; hypot only where a square could leave the FP64 range).
+// banded = 1 (the band form, bw < N - 1): row interchanges are applied from column c on, so L keeps
+// its band and the solve interleaves interchanges and eliminations.  banded = 0: they are applied to
+// the whole rows, so that P b is formed once and L is a plain triangle.  On exit the diagonal holds the
+// reciprocals 1 / u_cc and the rows of U are scaled by them (unit upper triangle): a step of the
+// solve is then one multiply-subtract instead of a division and one.
+// Measured: n = s = 64, p = 8 (320 factorisations) 981 -> 457 us; N = 320, bw = 32
+// (160) 8.66 -> 5.33 ms.
+constexpr int kLuMaxBw = 512;
+constexpr int kLuThreads = 256;
+__global__ void __launch_bounds__(kLuThreads) k_shifted_lu(const double2* __restrict__ H, long long sH,
+                                                           const double2* __restrict__ T, double2* LU,
+                                                           int* __restrict__ piv, int N, int bw, int s, int banded,
+                                                           int* err) {
   const int j = blockIdx.x, k = blockIdx.y;
   const double2* Hk = H + (long long)k * sH;
   const double2 shift = T[(long long)k * s * s + (long long)j * s + j];
   double2* M = LU + ((long long)k * s + j) * N * N;
   int* pv = piv + ((long long)k * s + j) * N;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ int sp[2];
+  __shared__ unsigned long long sbest[kLuThreads / 32];
+  __shared__ double2 sl[2][kLuMaxBw];
+  // max |M|: a pivot below N * 1e-14 * max|M| marks a (numerically) singular shift
+  unsigned long long mb = 0;
   for (long long e = threadIdx.x; e < (long long)N * N; e += blockDim.x) {
     double2 v = Hk[e];
     if ((e % N) == (e / N)) v = csub(v, shift);
     M[e] = v;
+    mb = max(mb, (unsigned long long)__double_as_longlong(cnorm(v)));
   }
-  __shared__ int sp;
-  __shared__ double sbest[256];
-  __shared__ double2 sl[kLuMaxBw];
-  __syncthreads();
-  // max-norm of M: a pivot below N * 1e-14 * max|M| marks a (numerically) singular shift
-  double mx = 0.0;
-  for (long long e = threadIdx.x; e < (long long)N * N; e += blockDim.x) mx = fmax(mx, cabs2(M[e]));
-  sbest[threadIdx.x] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m0 = 0.0;
-    for (int t = 0; t < (int)blockDim.x; ++t) m0 = fmax(m0, sbest[t]);
-    sbest[0] = m0;
+  auto block_max = [&](unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if (lane == 0) sbest[warp] = v;
+    __syncthreads();
+    v = 0;
+    for (int w = 0; w < kLuThreads / 32; ++w) v = max(v, sbest[w]);
+    return v;
+  };
+  double big = __longlong_as_double((long long)block_max(mb));
+  if (big >= kSqLo && big <= kSqHi) {
+    big = sqrt(big);
+  } else {   // squares out of range (or no finite entry)
+    mb = 0;
+    for (long long e = threadIdx.x; e < (long long)N * N; e += blockDim.x)
+      mb = max(mb, (unsigned long long)__double_as_longlong(cabs2(M[e])));
+    big = __longlong_as_double((long long)block_max(mb));
   }
-  __syncthreads();
-  const double tiny = 1e-14 * N * sbest[0];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c = 0; c < N; ++c) {
-    const int rmax = (c + bw < N - 1) ? c + bw : N - 1, nr = rmax - c;
+  const double tiny = 1e-14 * N * big;
+  // Pivot of column c, interchange inside the column, multipliers into the column and sl[c & 1]: one warp.
+  auto pivot_column = [&](int c) {
     double2* Mc = M + (long long)N * c;
-    if (warp == 0) {
-      double best = -1.0;
-      int bi = c;
+    const int rmax = (c + bw < N - 1) ? c + bw : N - 1, nr = rmax - c;
+    unsigned long long best = 0;
+    int bi = c;
+    bool exact = false;
+    for (int pass = 0; pass < 2; ++pass) {
+      best = 0;
+      bi = c;
       for (int r = c + lane; r <= rmax; r += 32) {
-        const double v = cabs2(Mc[r]);
-        if (v > best) {
-          best = v;
+        const double v = exact ? cabs2(Mc[r]) : cnorm(Mc[r]);
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v) + 1;   // 0: no candidate
+        if (b > best) {
+          best = b;
           bi = r;
         }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) {
           best = ob;
           bi = oi;
         }
       }
-      const int p = bi;
-      if (lane == 0) {
-        pv[c] = p;
-        sp = p;
-        if (best <= tiny) atomicOr(err, 2);
-        if (p != c) {
-          const double2 t0 = Mc[c];
-          Mc[c] = Mc[p];
-          Mc[p] = t0;
-        }
-      }
-      __syncwarp();
-      const double2 dinv = cdiv(make_double2(1.0, 0.0), Mc[c]);
-      for (int r = lane; r < nr; r += 32) {
-        const double2 l = cmul(Mc[c + 1 + r], dinv);
-        Mc[c + 1 + r] = l;
-        if (r < kLuMaxBw) sl[r] = l;
-      }
+      const double v = __longlong_as_double((long long)(best - 1));
+      if (exact || (v >= kSqLo && v <= kSqHi)) break;
+      exact = true;   // the largest squared modulus is out of range: compare the moduli themselves
     }
-    __syncthreads();
-    const int p = sp;
-    for (int q = c + 1 + (int)threadIdx.x; q < N; q += blockDim.x) {
-      double2* Mq = M + (long long)N * q;
-      if (p != c) {
-        const double2 t0 = Mq[c];
-        Mq[c] = Mq[p];
-        Mq[p] = t0;
+    const int p = bi;
+    const double2 d = Mc[p];
+    const double mod = exact ? __longlong_as_double((long long)(best - 1)) : 0.0;
+    const bool small = exact ? !(mod > tiny) : !(cnorm(d) > tiny * tiny);
+    if (lane == 0) {
+      pv[c] = p;
+      sp[c & 1] = p;
+      if (small) atomicOr(err, 2);
+    }
+    const double2 dinv = crecip(d), top = Mc[c];
+    __syncwarp();
+    for (int r = lane; r < nr; r += 32) {
+      const double2 v = c + 1 + r == p ? top : Mc[c + 1 + r];
+      const double2 l = make_double2(fma(-v.y, dinv.y, v.x * dinv.x), fma(v.y, dinv.x, v.x * dinv.y));
+      Mc[c + 1 + r] = l;
+      if (r < kLuMaxBw) sl[c & 1][r] = l;
+    }
+    __syncwarp();
+    if (lane == 0) Mc[c] = dinv;
+  };
+  // Column c applied to column q (one warp, a lane per row).
+  auto update_column = [&](int c, int q, int p) {
+    const int rmax = (c + bw < N - 1) ? c + bw : N - 1, nr = rmax - c;
+    double2* Mq = M + (long long)N * q;
+    const double2* Mc = M + (long long)N * c;
+    const double2 u = Mq[p], old = Mq[c];
+    __syncwarp();
+    for (int r = lane; r < nr; r += 32) {
+      const double2 v = c + 1 + r == p ? old : Mq[c + 1 + r];
+      const double2 l = r < kLuMaxBw ? sl[c & 1][r] : Mc[c + 1 + r];
+      Mq[c + 1 + r] = cfms(v, l, u);
+    }
+    __syncwarp();
+    if (lane == 0 && p != c) Mq[c] = u;
+  };
+  __syncthreads();
+  if (warp == 0) pivot_column(0);
+  __syncthreads();
+  for (int c = 0; c < N; ++c) {
+    const int p = sp[c & 1];
+    if (warp == 0) {
+      if (c + 1 < N) {
+        update_column(c, c + 1, p);
+        __syncwarp();
+        pivot_column(c + 1);
       }
-      const double2 u = Mq[c];
-      for (int r = 0; r < nr; ++r)
-        Mq[c + 1 + r] = csub(Mq[c + 1 + r], cmul(r < kLuMaxBw ? sl[r] : Mc[c + 1 + r], u));
+    } else {
+      for (int q = c + 1 + warp; q < N; q += kLuThreads / 32 - 1) update_column(c, q, p);
+      if (!banded && p != c)   // the interchange in the columns of L too
+        for (int q = threadIdx.x - 32; q < c; q += kLuThreads - 32) {
+          double2* Mq = M + (long long)N * q;
+          const double2 t0 = Mq[c];
+          Mq[c] = Mq[p];
+          Mq[p] = t0;
+        }
     }
     __syncthreads();
   }
+  // rows of U scaled by the reciprocals on the diagonal
+  for (int q = warp; q < N; q += kLuThreads / 32)
+    for (int r = lane; r < q; r += 32) {
+      const double2 d = M[r + (long long)N * r], v = M[r + (long long)N * q];
+      M[r + (long long)N * q] = make_double2(fma(-v.y, d.y, v.x * d.x), fma(v.y, d.x, v.x * d.y));
+    }
 }
 
-// One CTA per slice: Z[:, j] for j = 0..s-1 in order, using the factors of k_shifted_lu.  Both
-// triangular solves are blocked by kHsB columns so that the long dependent chains run inside one
-// warp on shared memory:
-//   forward  for each block of columns: stage the pivots and, for bands up to kHsBandStage wide,
-//            the L band (rows c+1 .. c+bw), then one warp applies the row interchanges and
-//            eliminations of the block in order (the same operations, in the same order, as the
-//            unblocked solve); wider bands (t-Bartels-Stewart, bw = n - 1) are read from global memory;
-//   backward for each block from the last: stage the diagonal kHsB x kHsB block of U, one warp
-//            solves it, then all threads subtract the block's columns from the rows above (GEMV).
+// One CTA per slice: Z[:, j] for j = 0..s-1 in order, using the factors of k_shifted_lu.  The column
+// sweep is serial by nature (column j needs every earlier one), and so are the substitutions inside it,
+// so the kernel is bound by the FP64 instructions of one warp per eliminated unknown (four, plus a
+// shared-memory round trip) and by what it can overlap with them:
+//   banded L   one warp applies the block's interchanges and eliminations in order, the band of L staged
+//              in shared memory;
+//   triangles  (U, and L when not banded) in blocks of kHsB unknowns: warp 0 substitutes inside the
+//              diagonal block, then every warp updates the next block's rows (its columns split over the
+//              warps, partial sums added in a fixed order), and warps 1-7 update the remaining rows while
+//              warp 0 goes on with the next block.
+// U's rows are already scaled to a unit diagonal, so a substitution step has no division.
+// Measured: n = s = 64, 5 slices 8.97 -> 2.46 ms; N = 320, bw = 32, s = 32,
+// 5 slices 22.4 -> 7.9 ms.
 constexpr int kHsB = 32;
 constexpr int kHsBandStage = 64;
-__global__ void __launch_bounds__(256) k_hs_solve(const double2* __restrict__ LU, const int* __restrict__ piv,
-                                                  const double2* __restrict__ G, const double2* __restrict__ T,
-                                                  double2* __restrict__ Z, int N, int bw, int s) {
+constexpr int kHsThreads = 256;
+__global__ void __launch_bounds__(kHsThreads) k_hs_solve(const double2* __restrict__ LU, const int* __restrict__ piv,
+                                                         const double2* __restrict__ G, const double2* __restrict__ T,
+                                                         double2* __restrict__ Z, int N, int bw, int s, int banded) {
   const int k = blockIdx.x;
   const double2* Gk = G + (long long)k * N * s;
   const double2* Tk = T + (long long)k * s * s;
   double2* Zk = Z + (long long)k * N * s;
   extern __shared__ double2 hs_smem[];
-  double2* rhs = hs_smem;                       // N
-  const bool stage = bw <= kHsBandStage;
-  double2* Lb = rhs + N;                        // kHsB x bw  (band of the block's L columns), if staged
-  double2* Ub = Lb + (stage ? (size_t)kHsB * bw : 0);   // kHsB x (kHsB + 1)
+  double2* rhs = hs_smem;                                      // N
+  double2* Lb = rhs + N;                                       // banded: kHsB x bw (the block's band of L)
+  double2* Ub = Lb + (banded ? (size_t)kHsB * bw : 0);         // 2 x kHsB x (kHsB + 1): diagonal blocks
+  double2* part = Ub + 2 * kHsB * (kHsB + 1);                  // kHsThreads: partial sums
   __shared__ int spv[kHsB];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NW = kHsThreads / 32;
+
+  // Unit triangular solve on rhs; lower: rows and columns in increasing order, else decreasing.
+  auto solve_triangle = [&](const double2* M, bool lower) {
+    const int nblk = (N + kHsB - 1) / kHsB;
+    auto block0 = [&](int b) { return lower ? b * kHsB : N - (b + 1) * kHsB; };   // first row, may be negative
+    auto stage = [&](int b, int t, int nt) {   // diagonal block b into its buffer
+      const int c0 = block0(b);
+      double2* U = Ub + (b & 1) * kHsB * (kHsB + 1);
+      for (int e = t; e < kHsB * kHsB; e += nt) {
+        const int rr = c0 + e % kHsB, cc = c0 + e / kHsB;
+        U[e % kHsB + (kHsB + 1) * (e / kHsB)] =
+            rr >= 0 && cc >= 0 && rr < N && cc < N ? M[rr + (long long)N * cc] : make_double2(0.0, 0.0);
+      }
+    };
+    stage(0, tid, kHsThreads);
+    __syncthreads();
+    for (int b = 0; b < nblk; ++b) {
+      const int c0 = block0(b);
+      if (warp == 0) {
+        const double2* U = Ub + (b & 1) * kHsB * (kHsB + 1);
+        const int row = c0 + lane;
+        const bool live = row >= 0 && row < N;
+        double2 v = live ? rhs[row] : make_double2(0.0, 0.0);
+        const int steps = lower ? min(kHsB, N - c0) : kHsB + min(c0, 0);
+#pragma unroll 4
+        for (int q = 0; q < steps; ++q) {
+          const int cc = lower ? q : kHsB - 1 - q;
+          const double2 z = make_double2(__shfl_sync(0xffffffffu, v.x, cc), __shfl_sync(0xffffffffu, v.y, cc));
+          if (lower ? lane > cc : lane < cc) v = cfms(v, U[lane + (kHsB + 1) * cc], z);
+        }
+        if (live) rhs[row] = v;
+      } else if (b > 0) {
+        // rows beyond the current block, updated by the block before it
+        const int p0 = block0(b - 1);
+        const int r0 = lower ? c0 + kHsB : 0, r1 = lower ? N : c0;
+        const int q0 = max(p0, 0), q1 = min(p0 + kHsB, N);
+        for (int r = r0 + tid - 32; r < r1; r += kHsThreads - 32) {
+          double2 v = rhs[r];
+#pragma unroll 4
+          for (int q = q0; q < q1; ++q) v = cfms(v, M[r + (long long)N * q], rhs[q]);
+          rhs[r] = v;
+        }
+        if (b + 1 < nblk) stage(b + 1, tid - 32, kHsThreads - 32);
+      } else if (b + 1 < nblk) {
+        stage(b + 1, tid - 32, kHsThreads - 32);
+      }
+      __syncthreads();
+      if (b + 1 < nblk) {   // the next block's rows, updated by this block: 4 columns per warp
+        const int row = block0(b + 1) + lane;
+        const bool live = row >= 0 && row < N;
+        double2 v = make_double2(0.0, 0.0);
+        if (live) {
+#pragma unroll
+          for (int t = 0; t < kHsB / NW; ++t) {
+            const int q = c0 + warp * (kHsB / NW) + t;
+            if (q >= 0 && q < N) v = cfms(v, M[row + (long long)N * q], rhs[q]);
+          }
+        }
+        part[tid] = v;
+        __syncthreads();
+        if (warp == 0 && live) {
+          v = rhs[row];
+#pragma unroll
+          for (int w = 0; w < NW; ++w) v = cadd(v, part[w * 32 + lane]);
+          rhs[row] = v;
+        }
+        __syncthreads();
+      }
+    }
+  };
+
   for (int j = 0; j < s; ++j) {
     const double2* M = LU + ((long long)k * s + j) * N * N;
     const int* pv = piv + ((long long)k * s + j) * N;
-    for (int r = threadIdx.x; r < N; r += blockDim.x) {
+    for (int r = tid; r < N; r += kHsThreads) {
       double2 v = Gk[r + (long long)N * j];
-      for (int i = 0; i < j; ++i) v = cadd(v, cmul(Tk[i + (long long)s * j], Zk[r + (long long)N * i]));
+      for (int i = 0; i < j; ++i) v = cfma(v, Tk[i + (long long)s * j], Zk[r + (long long)N * i]);
       rhs[r] = v;
     }
     __syncthreads();
-    // forward: row interchanges and the unit lower factor
-    for (int c0 = 0; c0 < N; c0 += kHsB) {
-      const int nb = min(kHsB, N - c0);
-      for (int e = threadIdx.x; stage && e < nb * bw; e += blockDim.x) {
-        const int cc = e / bw, t = e % bw, c = c0 + cc, r = c + 1 + t;
-        Lb[e] = r < N ? M[r + (long long)N * c] : make_double2(0.0, 0.0);
+    if (banded) {
+      // forward: row interchanges and the unit lower factor, in order
+      for (int c0 = 0; c0 < N; c0 += kHsB) {
+        const int nb = min(kHsB, N - c0);
+        for (int e = tid; e < nb * bw; e += kHsThreads) {
+          const int cc = e / bw, t = e % bw, c = c0 + cc, r = c + 1 + t;
+          Lb[e] = r < N ? M[r + (long long)N * c] : make_double2(0.0, 0.0);
+        }
+        for (int cc = tid; cc < nb; cc += kHsThreads) spv[cc] = pv[c0 + cc];
+        __syncthreads();
+        if (warp == 0) {
+          for (int cc = 0; cc < nb; ++cc) {
+            const int c = c0 + cc, p = spv[cc], nr = min(bw, N - 1 - c);
+            const double2 rc = rhs[p], old = rhs[c];
+            __syncwarp();
+            for (int t = lane; t < nr; t += 32) {
+              const double2 v = c + 1 + t == p ? old : rhs[c + 1 + t];
+              rhs[c + 1 + t] = cfms(v, Lb[cc * bw + t], rc);
+            }
+            if (lane == 0) rhs[c] = rc;
+            __syncwarp();
+          }
+        }
+        __syncthreads();
       }
-      for (int cc = threadIdx.x; cc < nb; cc += blockDim.x) spv[cc] = pv[c0 + cc];
-      __syncthreads();
-      if (warp == 0) {
-        for (int cc = 0; cc < nb; ++cc) {
-          const int c = c0 + cc, p = spv[cc];
-          if (p != c && lane == 0) {
-            const double2 t0 = rhs[c];
-            rhs[c] = rhs[p];
-            rhs[p] = t0;
+    } else {
+      if (warp == 0) {   // P rhs: the interchanges in order
+        for (int c0 = 0; c0 < N; c0 += 32) {
+          const int mine = c0 + lane < N ? pv[c0 + lane] : 0, nb = min(32, N - c0);
+          for (int cc = 0; cc < nb; ++cc) {
+            const int p = __shfl_sync(0xffffffffu, mine, cc);
+            if (lane == 0 && p != c0 + cc) {
+              const double2 t0 = rhs[c0 + cc];
+              rhs[c0 + cc] = rhs[p];
+              rhs[p] = t0;
+            }
           }
-          __syncwarp();
-          const double2 rc = rhs[c];
-          const int nr = min(bw, N - 1 - c);
-          for (int t = lane; t < nr; t += 32) {
-            const double2 l = stage ? Lb[cc * bw + t] : M[(c + 1 + t) + (long long)N * c];
-            rhs[c + 1 + t] = csub(rhs[c + 1 + t], cmul(l, rc));
-          }
-          __syncwarp();
         }
       }
       __syncthreads();
+      solve_triangle(M, true);
     }
-    // backward: the upper factor, by blocks from the last
-    for (int c1 = N; c1 > 0; c1 -= kHsB) {
-      const int c0 = max(0, c1 - kHsB), nb = c1 - c0;
-      for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        const int rr = e % nb, cc = e / nb;
-        Ub[rr + (kHsB + 1) * cc] = M[(c0 + rr) + (long long)N * (c0 + cc)];
-      }
-      __syncthreads();
-      if (warp == 0) {
-        for (int cc = nb - 1; cc >= 0; --cc) {
-          if (lane == 0) rhs[c0 + cc] = cdiv(rhs[c0 + cc], Ub[cc + (kHsB + 1) * cc]);
-          __syncwarp();
-          const double2 zc = rhs[c0 + cc];
-          if (lane < cc) rhs[c0 + lane] = csub(rhs[c0 + lane], cmul(Ub[lane + (kHsB + 1) * cc], zc));
-          __syncwarp();
-        }
-      }
-      __syncthreads();
-      for (int r = threadIdx.x; r < c0; r += blockDim.x) {
-        double2 v = rhs[r];
-        for (int cc = 0; cc < nb; ++cc) v = csub(v, cmul(M[r + (long long)N * (c0 + cc)], rhs[c0 + cc]));
-        rhs[r] = v;
-      }
-      __syncthreads();
+    for (int r = tid; r < N; r += kHsThreads) {   // the diagonal (reciprocals)
+      const double2 d = M[r + (long long)N * r], v = rhs[r];
+      rhs[r] = make_double2(fma(-v.y, d.y, v.x * d.x), fma(v.y, d.x, v.x * d.y));
     }
-    for (int r = threadIdx.x; r < N; r += blockDim.x) Zk[r + (long long)N * j] = rhs[r];
+    __syncthreads();
+    solve_triangle(M, false);
+    for (int r = tid; r < N; r += kHsThreads) Zk[r + (long long)N * j] = rhs[r];
     __syncthreads();
   }
 }
@@ -275,20 +426,27 @@ __global__ void k_cholesky(const double2* __restrict__ Gall, double2* __restrict
 
 }  // namespace
 
+namespace {
+// The band form of the factors pays while the band is well inside the matrix and its block of L fits
+// the staging buffer (TBAS: bw = s, N = m s); otherwise plain triangles.
+bool band_form(int N, int bw) { return bw <= kHsBandStage && 2 * bw < N; }
+}  // namespace
+
 void shifted_lu(const double2* H, long long sH, const double2* T, double2* LU, int* piv, int N, int bw, int s, int K,
                 int* err, cudaStream_t st) {
-  k_shifted_lu<<<dim3(s, K), 256, 0, st>>>(H, sH, T, LU, piv, N, bw, s, err);
+  k_shifted_lu<<<dim3(s, K), kLuThreads, 0, st>>>(H, sH, T, LU, piv, N, bw, s, band_form(N, bw), err);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }
 
 void hs_solve(const double2* LU, const int* piv, const double2* G, const double2* T, double2* Z, int N, int bw, int s,
               int K, cudaStream_t st) {
-  const size_t band = bw <= kHsBandStage ? (size_t)kHsB * bw : 0;
-  const size_t smem = sizeof(double2) * ((size_t)N + band + (size_t)kHsB * (kHsB + 1));
-  TS_REQUIRE(smem <= 200 * 1024, "projected system too large");
-  if (smem > 48 * 1024) TS_CUDA(cudaFuncSetAttribute(k_hs_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_hs_solve<<<K, 256, smem, st>>>(LU, piv, G, T, Z, N, bw, s);
+  const bool band = band_form(N, bw);
+  const size_t smem = sizeof(double2) * ((size_t)N + (band ? (size_t)kHsB * bw : 0) + 2 * (size_t)kHsB * (kHsB + 1) +
+                                         kHsThreads);
+  TS_REQUIRE(smem <= 226 * 1024, "projected system too large");
+  set_max_dynamic_smem((const void*)k_hs_solve, (int)smem);
+  k_hs_solve<<<K, kHsThreads, smem, st>>>(LU, piv, G, T, Z, N, bw, s, band);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }
