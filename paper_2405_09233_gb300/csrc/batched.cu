@@ -344,14 +344,20 @@ __global__ void __launch_bounds__(kTubes) k_b_irfft(BDev d, const Cplx* __restri
   }
 }
 
+constexpr int kBatchSimtBM = 64;   // rows of a work-list tile of the CUDA-core products
+
 // --- per-slice products over the work list ---------------------------------------------------------
 // TILE 0: every instance has n, s <= kTinyL and the items are 8 x 4 tiles for kTinyThreads
-// (gemm_tiny_tile); otherwise 64 x TILE tiles (TILE = 64, 32 or 16 columns; 4 x TILE/16 outputs per
-// thread) for kGemmNT threads.  Every TILE > 0 sums each output entry's products in the same order
+// (gemm_tiny_tile); otherwise 64 x TILE tiles (TILE = 64, 32 or 16 columns): 256 threads in FP64
+// (gemm_tile_f64), one per 8 x 4 block in FP32 (gemm_tile_f32).  Every TILE > 0 sums each output entry's products in the same order
 // (phase 1's reduction index, then phase 2's), so the column width, which the autotuner picks,
 // changes which CTA forms an entry and how much padding it computes, never the entry's value.
+template <typename Real, int TILE>
+constexpr int b_gemm_threads() {
+  return TILE == 0 ? kTinyThreads : (sizeof(Real) == 8 ? 256 : kBatchSimtBM * TILE / 32);
+}
 template <typename Real, int MASK, int TILE>
-__global__ void __launch_bounds__(kGemmNT, 1) k_b_gemm(BDev d, const int4* __restrict__ items,
+__global__ void __launch_bounds__((b_gemm_threads<Real, TILE>()), 1) k_b_gemm(BDev d, const int4* __restrict__ items,
                                                        const typename CplxOf<Real>::T* __restrict__ Xh,
                                                        typename CplxOf<Real>::T* __restrict__ Yh) {
   using Cplx = typename CplxOf<Real>::T;
@@ -377,7 +383,8 @@ __global__ void __launch_bounds__(kGemmNT, 1) k_b_gemm(BDev d, const int4* __res
   a.Y = Yh + in.offS; a.sY = T; a.ldy = in.n;
   a.M = in.n; a.N = in.s; a.K = in.K; a.nyq = in.nyq; a.sgn2 = -1.0;
   if constexpr (TILE == 0) gemm_tiny_tile<Real>(a, it.y, it.z, it.w);
-  else gemm_tile<Real, kGemmBM, TILE, 4, TILE / 16>(a, it.y, it.z, it.w);
+  else if constexpr (sizeof(Real) == 8) gemm_tile_f64<256, TILE, kBatchSimtBM * TILE / 256>(a, it.y, it.z, it.w);
+  else gemm_tile_f32<kBatchSimtBM, TILE, 1>(a, it.y, it.z, it.w);
 }
 
 // Column widths the autotuner chooses from for the CUDA-core work-list products, and one work list.
@@ -395,11 +402,19 @@ void launch_b_gemm(const SimtList& l, const BDev& d, const void* X, void* Y, cud
   using Cplx = typename CplxOf<Real>::T;
   const Cplx* x = static_cast<const Cplx*>(X);
   Cplx* y = static_cast<Cplx*>(Y);
+  auto run = [&](auto tile) {
+    constexpr int TILE = decltype(tile)::value;
+    int smem = 0;
+    if constexpr (sizeof(Real) == 4 && TILE > 0) {
+      smem = F32Tile<kBatchSimtBM, TILE, 1>::kSmem;
+    }
+    k_b_gemm<Real, MASK, TILE><<<l.count, b_gemm_threads<Real, TILE>(), smem, st>>>(d, l.items, x, y);
+  };
   switch (l.bn) {
-    case 0: k_b_gemm<Real, MASK, 0><<<l.count, kTinyThreads, 0, st>>>(d, l.items, x, y); break;
-    case 64: k_b_gemm<Real, MASK, 64><<<l.count, kGemmNT, 0, st>>>(d, l.items, x, y); break;
-    case 32: k_b_gemm<Real, MASK, 32><<<l.count, kGemmNT, 0, st>>>(d, l.items, x, y); break;
-    case 16: k_b_gemm<Real, MASK, 16><<<l.count, kGemmNT, 0, st>>>(d, l.items, x, y); break;
+    case 0: run(std::integral_constant<int, 0>{}); break;
+    case 64: run(std::integral_constant<int, 64>{}); break;
+    case 32: run(std::integral_constant<int, 32>{}); break;
+    case 16: run(std::integral_constant<int, 16>{}); break;
     default: TS_REQUIRE(false, "batched products: unknown tile width");
   }
   TS_CUDA(cudaGetLastError());
@@ -734,7 +749,7 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
         if (std::find(need.begin(), need.end(), bn) == need.end()) need.push_back(bn);
     }
     for (int bn : need) {
-      const int tbm = bn == 0 ? kTinyBM : kGemmBM, tbn = bn == 0 ? kTinyBN : bn;
+      const int tbm = bn == 0 ? kTinyBM : kBatchSimtBM, tbn = bn == 0 ? kTinyBN : bn;
       std::vector<int4> items;
       for (int i = 0; i < count; ++i) {
         const BInst& b = plan.inst[i];

@@ -10,15 +10,29 @@
 // 3 DFMA per complex multiply-add instead of 4.  The sums ar+ai, br+bi are formed once per
 // shared-memory tile element.  Slices k = 0 and k = p/2 are real (their imaginary parts are
 // exactly zero) and take a single real product.
+#include <type_traits>
 #include "internal.cuh"
 #include "gemm_tile.cuh"
 
 namespace ts {
 namespace {
 
-template <typename Real, int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__(kGemmNT, 1) k_gemm_slices(GemmArgs<typename CplxOf<Real>::T> a) {
-  gemm_tile<Real, BM, BN, TM, TN>(a, blockIdx.z, blockIdx.x * BM, blockIdx.y * BN);
+// Slices in the order of their cost: the complex ones (k = 1 ..), then the real ones (k = 0, k = p/2).
+__device__ __forceinline__ int slice_by_cost(int z, int K, int nyq) {
+  const int kc = K - 1 - (nyq >= 0 ? 1 : 0);
+  return z < kc ? z + 1 : (z == kc ? 0 : nyq);
+}
+
+template <int NT, int BN, int TM>
+__global__ void __launch_bounds__(NT, (TM > 2 ? 3 : 4) * (256 / NT)) k_gemm_f64(ZGemmArgs a, int mt, int nt) {
+  const int per = mt * nt, z = blockIdx.x / per, t = blockIdx.x % per;
+  gemm_tile_f64<NT, BN, TM>(a, slice_by_cost(z, a.K, a.nyq), t % mt * F64Tile<NT, BN, TM>::BM, t / mt * BN);
+}
+
+template <int BM, int BN, int G>
+__global__ void __launch_bounds__((F32Tile<BM, BN, G>::NT), G > 1 ? 3 : 2) k_gemm_f32(CGemmArgs a, int mt, int nt) {
+  const int per = mt * nt, z = blockIdx.x / per, t = blockIdx.x % per;
+  gemm_tile_f32<BM, BN, G>(a, slice_by_cost(z, a.K, a.nyq), t % mt * BM, t / mt * BN);
 }
 
 template <typename Real>
@@ -35,8 +49,76 @@ int sm_count() {
   return cached[dev];
 }
 
-// Otherwise the output tile is the largest of 64, 32, 16 whose grid still covers every SM (a product of a few large
-// tiles would leave most of the FP64 pipes idle); 16 when even that does not.
+// Estimated time of the product on bm x bn tiles, in output entries of a real slice per SM: the padded
+// products (three real ones per complex entry) and `stage` extra operations per staged row or column,
+// spread over the SMs, plus part of one tile for the uneven end of the launch.
+double tile_cost(int M, int N, int K, int nyq, int bm, int bn, double stage, double tail) {
+  const double kr = 1 + (nyq >= 0 ? 1 : 0), kc = K - kr;
+  const double mt = (M + bm - 1) / bm, nt = (N + bn - 1) / bn, area = (double)bm * bn;
+  const double one = 3.0 * area + stage * (bm + bn);   // a complex tile
+  return mt * nt * (kc * one + kr * area) / sm_count() + tail * (kc > 0 ? one : area);
+}
+
+template <int NT, int BN, int TM>
+void launch_f64(const ZGemmArgs& a, cudaStream_t st) {
+  constexpr int BM = F64Tile<NT, BN, TM>::BM;
+  const int mt = (a.M + BM - 1) / BM, nt = (a.N + BN - 1) / BN;
+  const long long blocks = (long long)mt * nt * a.K;
+  TS_REQUIRE((long long)mt * nt <= INT32_MAX && blocks <= INT32_MAX, "slice GEMM grid too large");
+  k_gemm_f64<NT, BN, TM><<<(unsigned)blocks, NT, 0, st>>>(a, mt, nt);
+}
+
+template <int BM, int BN, int G>
+void launch_f32(const CGemmArgs& a, cudaStream_t st) {
+  using Cfg = F32Tile<BM, BN, G>;
+  const int mt = (a.M + BM - 1) / BM, nt = (a.N + BN - 1) / BN;
+  const long long blocks = (long long)mt * nt * a.K;
+  TS_REQUIRE((long long)mt * nt <= INT32_MAX && blocks <= INT32_MAX, "slice GEMM grid too large");
+  k_gemm_f32<BM, BN, G><<<(unsigned)blocks, Cfg::NT, Cfg::kSmem, st>>>(a, mt, nt);
+}
+
+// The cheapest tile by tile_cost.  `stage`, `tail` and `slow` were fitted to launches forced onto every shape:
+//   FP64: at 1024 x 1024 x 16 (no padding, no uneven end) the shapes' rates follow the additions of their
+//   factor sums, 0.96 of the pipe at 32 x 32 down to 0.87 at 32 x 4; the 64-thread 16 x 4 tile runs lower, 0.83.
+//   FP32: 0.56, 0.47 and 0.39 of the FP32 rate for the three shapes at that size (fewer products per
+//   barrier and per read); 512 x 128 x 16 takes 65, 72 and 74 us, 256 x 256 x 8 takes 52, 46 and 41 us.
+template <typename Args>
+struct TileShape {
+  int bm, bn;
+  double stage, tail, slow;
+  void (*run)(const Args&, cudaStream_t);
+};
+template <typename Args, size_t N>
+void launch_cheapest(const TileShape<Args> (&shapes)[N], const Args& a, cudaStream_t st) {
+  const TileShape<Args>* best = nullptr;
+  double cost = 0.0;
+  for (const auto& s : shapes) {
+    const double c = s.slow * tile_cost(a.M, a.N, a.K, a.nyq, s.bm, s.bn, s.stage, s.tail);
+    if (!best || c < cost) {
+      best = &s;
+      cost = c;
+    }
+  }
+  best->run(a, st);
+}
+void launch_tiles(const ZGemmArgs& a, cudaStream_t st) {
+  static const TileShape<ZGemmArgs> shapes[] = {
+      {64, 16, 1.3, 0.6, 1.0, launch_f64<256, 16, 4>}, {32, 32, 1.3, 0.6, 1.0, launch_f64<256, 32, 4>},
+      {128, 8, 1.3, 0.6, 1.0, launch_f64<256, 8, 4>},  {32, 16, 1.3, 0.6, 1.0, launch_f64<256, 16, 2>},
+      {64, 8, 1.3, 0.6, 1.0, launch_f64<256, 8, 2>},   {16, 16, 1.3, 0.6, 1.0, launch_f64<256, 16, 1>},
+      {32, 8, 1.3, 0.6, 1.0, launch_f64<256, 8, 1>},   {64, 4, 1.3, 0.6, 1.0, launch_f64<256, 4, 1>},
+      {16, 8, 1.3, 0.6, 1.0, launch_f64<128, 8, 1>},   {32, 4, 1.3, 0.6, 1.0, launch_f64<128, 4, 1>},
+      {16, 4, 1.8, 0.6, 1.0, launch_f64<64, 4, 1>}};
+  launch_cheapest(shapes, a, st);
+}
+void launch_tiles(const CGemmArgs& a, cudaStream_t st) {
+  static const TileShape<CGemmArgs> shapes[] = {{64, 64, 0.0, 0.4, 1.0, launch_f32<64, 64, 1>},
+                                                {64, 32, 0.0, 0.4, 1.2, launch_f32<64, 32, 2>},
+                                                {32, 32, 0.0, 0.4, 1.4, launch_f32<32, 32, 4>}};
+  launch_cheapest(shapes, a, st);
+}
+
+// Products whose reductions are at most kTinyL long run one 8 x 4 tile per CTA (see gemm_tiny_tile).
 template <typename Real>
 void launch_slices(const GemmArgs<typename CplxOf<Real>::T>& a, cudaStream_t st) {
   if (a.M <= 0 || a.N <= 0 || a.K <= 0) return;
@@ -44,18 +126,9 @@ void launch_slices(const GemmArgs<typename CplxOf<Real>::T>& a, cudaStream_t st)
     dim3 grid((a.M + kTinyBM - 1) / kTinyBM, (a.N + kTinyBN - 1) / kTinyBN, a.K);
     TS_REQUIRE(grid.y <= 65535 && grid.z <= 65535, "slice GEMM grid too large");
     k_gemm_tiny<Real><<<grid, kTinyThreads, 0, st>>>(a);
-    count_launch();
-    TS_CUDA(cudaGetLastError());
-    return;
+  } else {
+    launch_tiles(a, st);
   }
-  const long long sms = sm_count();
-  auto ctas = [&](int t) { return (long long)a.K * ((a.M + t - 1) / t) * ((a.N + t - 1) / t); };
-  const int tile = ctas(64) >= sms ? 64 : (ctas(32) >= sms ? 32 : 16);
-  dim3 grid((a.M + tile - 1) / tile, (a.N + tile - 1) / tile, a.K);
-  TS_REQUIRE(grid.y <= 65535 && grid.z <= 65535, "slice GEMM grid too large");
-  if (tile == 64) k_gemm_slices<Real, 64, 64, 4, 4><<<grid, kGemmNT, 0, st>>>(a);
-  else if (tile == 32) k_gemm_slices<Real, 32, 32, 2, 2><<<grid, kGemmNT, 0, st>>>(a);
-  else k_gemm_slices<Real, 16, 16, 1, 1><<<grid, kGemmNT, 0, st>>>(a);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }
