@@ -377,50 +377,98 @@ __global__ void k_small_gemm(const double2* __restrict__ A, long long sA, int ld
   }
 }
 
-// Cholesky G = R^H R of a Hermitian positive definite s x s matrix per slice (one warp each).
-// R is written upper triangular (zeros below).  A pivot d_j (the squared norm of column j's part
-// orthogonal to the previous columns, when G is a Gram matrix) fails when it is not above
-// max(rel * g_jj, tiny2 * max_k g_jj(k)), the second maximum taken over the Grams of all K slices;
-// rel = tiny2 = 0 asks for d_j > 0 only.  A failed slice stops early (R partly written), sets
+// Cholesky G = R^H R of a Hermitian positive definite s x s matrix per slice and the inverse of R, one CTA
+// each, both in shared memory.  R and Rinv are written upper triangular (zeros below).  A pivot d_j (the
+// squared norm of column j's part orthogonal to the previous columns, when G is a Gram matrix) fails when
+// it is not above max(rel * g_jj, tiny2 * max_k g_jj(k)), the second maximum taken over the Grams of all K
+// slices; rel = tiny2 = 0 asks for d_j > 0 only.  A failed slice stops early (nothing written), sets
 // fail_slice[slice] = 1 (each slice's entry is reset to 0 first) and err bit 4 (err may be NULL).
-__global__ void k_cholesky(const double2* __restrict__ Gall, double2* __restrict__ Rall, int s, int K, double rel,
-                           double tiny2, int* err, int* fail_slice) {
+// What bounds it: the chain of s pivots (a square root, a division) with the FP64 issue of one SM; the
+// right-looking forms leave a rank-one update between pivots, spread over all threads: warp 0 forms a
+// pivot and scales its row, every thread updates.
+// Measured: s = 32, 5 slices 279 (two one-warp kernels on global memory) -> 63 us.
+constexpr int kCholThreads = 256;
+__global__ void __launch_bounds__(kCholThreads) k_cholesky_inverse(const double2* __restrict__ Gall,
+                                                                   double2* __restrict__ Rall,
+                                                                   double2* __restrict__ Xall, int s, int K, double rel,
+                                                                   double tiny2, int* err, int* fail_slice) {
+  extern __shared__ double2 chol_smem[];
+  const int ld = s + 1, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  double2* A = chol_smem;                 // G, then R; (r, c) at r + ld c
+  double2* X = chol_smem + (size_t)s * ld;   // accumulates sum_c R(a, c) X(c, b), then R^-1
+  __shared__ double floor_d[64], inv_d[64];
+  __shared__ int bad;
   const double2* G = Gall + (long long)blockIdx.x * s * s;
-  double2* R = Rall + (long long)blockIdx.x * s * s;
-  const int lane = threadIdx.x & 31;
-  if (fail_slice && lane == 0) fail_slice[blockIdx.x] = 0;
-  for (int e = lane; e < s * s; e += 32) R[e] = make_double2(0.0, 0.0);
-  __syncwarp();
-  for (int j = 0; j < s; ++j) {
-    // r_jj = sqrt(g_jj - sum_{i<j} |r_ij|^2)
-    const double gjj = G[j + (long long)s * j].x;
-    double d = gjj;
-    for (int i = 0; i < j; ++i) {
-      const double2 r = R[i + (long long)s * j];
-      d -= r.x * r.x + r.y * r.y;
-    }
-    double floor_d = rel * gjj;
+  for (int e = tid; e < s * s; e += kCholThreads) {
+    A[e % s + ld * (e / s)] = G[e];
+    X[e % s + ld * (e / s)] = make_double2(0.0, 0.0);
+  }
+  for (int j = tid; j < s; j += kCholThreads) {
+    double f = rel * G[j + (long long)s * j].x;
     if (tiny2 > 0.0) {
       double ref2 = 0.0;
       for (int q = 0; q < K; ++q) ref2 = fmax(ref2, Gall[(long long)q * s * s + j + (long long)s * j].x);
-      floor_d = fmax(floor_d, tiny2 * ref2);
+      f = fmax(f, tiny2 * ref2);
     }
-    if (!(d > floor_d)) {
-      if (lane == 0) {
-        if (err) atomicOr(err, 4);
-        if (fail_slice) fail_slice[blockIdx.x] = 1;
+    floor_d[j] = f;
+  }
+  if (tid == 0) {
+    bad = 0;
+    if (fail_slice) fail_slice[blockIdx.x] = 0;
+  }
+  __syncthreads();
+  for (int j = 0; j < s; ++j) {
+    if (warp == 0) {
+      const double d = A[j + ld * j].x;
+      if (!(d > floor_d[j])) {
+        if (lane == 0) {
+          bad = 1;
+          if (err) atomicOr(err, 4);
+          if (fail_slice) fail_slice[blockIdx.x] = 1;
+        }
+      } else {
+        const double rjj = sqrt(d), inv = 1.0 / rjj;
+        __syncwarp();
+        for (int q = j + 1 + lane; q < s; q += 32) A[j + ld * q] = cscale(A[j + ld * q], inv);
+        if (lane == 0) {
+          A[j + ld * j] = make_double2(rjj, 0.0);
+          inv_d[j] = inv;
+        }
       }
-      return;
     }
-    const double rjj = sqrt(d);
-    if (lane == 0) R[j + (long long)s * j] = make_double2(rjj, 0.0);
-    // r_jq = (g_jq - sum_{i<j} conj(r_ij) r_iq) / r_jj for q > j
-    for (int q = j + 1 + lane; q < s; q += 32) {
-      double2 v = G[j + (long long)s * q];
-      for (int i = 0; i < j; ++i) v = csub(v, cmulc(R[i + (long long)s * j], R[i + (long long)s * q]));
-      R[j + (long long)s * q] = cscale(v, 1.0 / rjj);
+    __syncthreads();
+    if (bad) return;
+    // A(p, q) -= conj(R(j, p)) R(j, q), j < p <= q
+    const int m = s - 1 - j;
+    for (int e = tid; e < m * m; e += kCholThreads) {
+      const int p = j + 1 + e % m, q = j + 1 + e / m;
+      if (p <= q) {
+        const double2 u = A[j + ld * p];
+        A[p + ld * q] = cfms(A[p + ld * q], make_double2(u.x, -u.y), A[j + ld * q]);
+      }
     }
-    __syncwarp();
+    __syncthreads();
+  }
+  for (int a = s - 1; a >= 0; --a) {   // row a of R^-1, then its part of the rows above
+    const double inv = inv_d[a];
+    for (int b = a + tid; b < s; b += kCholThreads) {
+      const double2 v = X[a + ld * b];
+      X[a + ld * b] = b == a ? make_double2(inv, 0.0) : make_double2(-v.x * inv, -v.y * inv);
+    }
+    __syncthreads();
+    const int m = s - a;
+    for (int e = tid; e < a * m; e += kCholThreads) {
+      const int r = e % a, b = a + e / a;
+      X[r + ld * b] = cfma(X[r + ld * b], A[r + ld * a], X[a + ld * b]);
+    }
+    __syncthreads();
+  }
+  double2* R = Rall + (long long)blockIdx.x * s * s;
+  double2* Xo = Xall + (long long)blockIdx.x * s * s;
+  for (int e = tid; e < s * s; e += kCholThreads) {
+    const int r = e % s, c = e / s;
+    R[e] = r <= c ? A[r + ld * c] : make_double2(0.0, 0.0);
+    Xo[e] = r <= c ? X[r + ld * c] : make_double2(0.0, 0.0);
   }
 }
 
@@ -462,9 +510,12 @@ void small_gemm(const double2* A, long long sA, int lda, const double2* B, long 
   TS_CUDA(cudaGetLastError());
 }
 
-void cholesky_small(const double2* G, double2* R, int s, int K, double rel, double tiny2, int* err, int* fail_slice,
-                    cudaStream_t st) {
-  k_cholesky<<<K, 32, 0, st>>>(G, R, s, K, rel, tiny2, err, fail_slice);
+void cholesky_inverse(const double2* G, double2* R, double2* Rinv, int s, int K, double rel, double tiny2, int* err,
+                      int* fail_slice, cudaStream_t st) {
+  TS_REQUIRE(s <= 64, "cholesky_inverse: block width above 64");
+  const size_t smem = 2 * sizeof(double2) * (size_t)s * (s + 1);
+  set_max_dynamic_smem((const void*)k_cholesky_inverse, (int)smem);
+  k_cholesky_inverse<<<K, kCholThreads, smem, st>>>(G, R, Rinv, s, K, rel, tiny2, err, fail_slice);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }

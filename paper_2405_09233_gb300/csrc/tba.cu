@@ -47,6 +47,11 @@ __device__ __forceinline__ double slice_weight(int k, int p) {
   return (k == 0 || (p % 2 == 0 && k == p / 2)) ? 1.0 : 2.0;
 }
 
+__device__ __forceinline__ double neg(double v) {   // without an FP64 instruction
+  return __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
+}
+__device__ __forceinline__ float neg(float v) { return -v; }
+
 constexpr int kMaxS = 64;           // block width supported by the row kernels
 
 // C2: double2 (FP64), or float2 for the FP32 inner cycle of mixed-precision TBAS (MODE 0 only).
@@ -76,6 +81,7 @@ template <int MODE, int LT, typename C2>
 __global__ void __launch_bounds__(256) k_sylv_rows(RowsArgsT<C2> a) {
   static_assert(MODE == 0 || sizeof(C2) == 16, "the operator with B_k and the residual run in FP64");
   const int k = blockIdx.y;
+  const bool real = k == 0 || (a.p % 2 == 0 && k == a.p / 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int sp = 32;
   if (LT == 1)
@@ -93,7 +99,31 @@ __global__ void __launch_bounds__(256) k_sylv_rows(RowsArgsT<C2> a) {
 #pragma unroll
     for (int t = 0; t < LT; ++t) acc[t] = C2{0, 0};
     if (live) {
-      if (a.rowptr) {
+      if (real) {   // A_k, V_k and B_k real: one multiply-add of four
+        const int q0 = a.rowptr ? a.rowptr[i] : 0, q1 = a.rowptr ? a.rowptr[i + 1] : a.n;
+        const C2* vk = a.rowptr ? a.vals + (long long)k * a.nnz : a.Ad + (long long)k * a.n * a.n + i;
+        for (int q = q0; q < q1; ++q) {
+          const auto av = a.rowptr ? vk[q].x : vk[(long long)q * a.n].x;
+          const C2* vr = Vk + (long long)(a.rowptr ? a.col[q] : q) * a.s;
+#pragma unroll
+          for (int t = 0; t < LT; ++t) {
+            const int j = jl + 32 * t;
+            if (j < a.s) acc[t].x = fma(av, vr[j].x, acc[t].x);
+          }
+        }
+        if constexpr (MODE >= 1) {
+          const double2* Bk = a.Brow + (long long)k * a.s * a.s;
+          const double2* xr = Vk + (long long)i * a.s;
+          for (int l = 0; l < a.s; ++l) {
+            const double nx = neg(xr[l].x);
+#pragma unroll
+            for (int t = 0; t < LT; ++t) {
+              const int j = jl + 32 * t;
+              if (j < a.s) acc[t].x = fma(nx, Bk[(long long)l * a.s + j].x, acc[t].x);
+            }
+          }
+        }
+      } else if (a.rowptr) {
         const C2* vk = a.vals + (long long)k * a.nnz;
         for (int q = a.rowptr[i]; q < a.rowptr[i + 1]; ++q) {
           const C2 av = vk[q];
@@ -119,7 +149,7 @@ __global__ void __launch_bounds__(256) k_sylv_rows(RowsArgsT<C2> a) {
       if constexpr (MODE >= 1) {
         const double2* Bk = a.Brow + (long long)k * a.s * a.s;
         const double2* xr = Vk + (long long)i * a.s;
-        for (int l = 0; l < a.s; ++l) {
+        for (int l = 0; !real && l < a.s; ++l) {
           const double2 xv = xr[l];
           const double2 nx = make_double2(-xv.x, -xv.y);
 #pragma unroll
@@ -137,8 +167,9 @@ __global__ void __launch_bounds__(256) k_sylv_rows(RowsArgsT<C2> a) {
           const long long o = k * ns + (long long)i * a.s + j;
           if constexpr (MODE == 2) {
             const double2 c = a.C[o];
-            v = make_double2(c.x - v.x, c.y - v.y);
-            local += v.x * v.x + v.y * v.y;
+            v = make_double2(c.x - v.x, real ? 0.0 : c.y - v.y);
+            local = fma(v.x, v.x, local);
+            if (!real) local = fma(v.y, v.y, local);
           }
           a.Out[o] = v;
         }
@@ -151,140 +182,252 @@ __global__ void __launch_bounds__(256) k_sylv_rows(RowsArgsT<C2> a) {
   }
 }
 
-// Partial Gram matrices G_k = V_k^H W_k over row chunks: partials[(k*chunks + c)*s*s + a + s*b].
+// A launch's blocks dealt to the K slices: the real ones (k = 0 and, for even p, k = p/2), whose products
+// are real, get a third of the blocks of a complex one.  Complex slices come first.
+struct SliceParts {
+  int K, nyq;
+  int kc;        // complex slices k = 1 .. kc
+  int nc, nr;    // blocks of a complex / real slice
+  __host__ __device__ int blocks() const { return kc * nc + (K - kc) * nr; }
+  __device__ __forceinline__ void of(int b, int& k, int& part, int& parts) const {
+    if (b < kc * nc) {
+      k = 1 + b / nc;
+      part = b % nc;
+      parts = nc;
+    } else {
+      b -= kc * nc;
+      k = b / nr == 0 ? 0 : nyq;
+      part = b % nr;
+      parts = nr;
+    }
+  }
+  // first block of slice k
+  __device__ __forceinline__ int first(int k) const {
+    return k == 0 ? kc * nc : (k == nyq ? kc * nc + nr : (k - 1) * nc);
+  }
+  __device__ __forceinline__ bool real(int k) const { return k == 0 || k == nyq; }
+  __device__ __forceinline__ int parts(int k) const { return real(k) ? nr : nc; }
+};
+// About `blocks` blocks in all, none with fewer than `min_rows` of the n rows.
+SliceParts slice_parts(int K, int nyq, int n, int blocks, int min_rows) {
+  SliceParts q{K, nyq, K - 1 - (nyq >= 0 ? 1 : 0), 1, 1};
+  const int units = 3 * q.kc + (K - q.kc), most = std::max(1, n / min_rows);
+  q.nc = std::max(1, std::min(most, (int)(3.0 * blocks / units)));
+  q.nr = std::max(1, std::min(most, (int)((double)blocks / units)));
+  return q;
+}
+
+// Partial Gram matrices G_k = V_k^H W_k over row chunks: partials[block * s*s + a + s*b].
 // Gauss's three-multiplication form: with u = conj(v), u w = (T1 - T3) + i (T1 + T2) where
 // T1 = sum w_re (u_re + u_im), T2 = sum u_re (w_im - w_re), T3 = sum u_im (w_re + w_im); the sums
 // of the factors are formed once per entry while staging, so a complex multiply-add costs three
-// DFMA.  Each thread owns a 4 x 4 block of G; min(256 / (s/4)^2, 16) row groups split a staged row
-// batch and are summed in shared memory at the end.
+// FMAs, and one in a real slice.  Each thread owns a 4 x 4 block of G; with HERM (V = W) only the blocks on
+// and above the diagonal are formed.  The threads left over form further groups that split the staged
+// rows and are summed in a fixed order at the end.
+// What bounds it: the FP64 pipe (16 clocks of the SM per warp instruction), so one CTA of eight warps per
+// SM saturates it as long as it never waits: the next rows are in registers while the staged ones are
+// multiplied, staging is double buffered (one barrier per batch), columns are padded to a multiple of
+// 4 only, and blocks are dealt to the slices by their cost.
+// Measured (n = 16384, s = 32, p = 8): 546 -> 357 us, with V = W 214 us; s = 4: 205 -> 34 us.
 // C2 = float2: FP32 inputs and accumulation (the inner cycle of mixed-precision TBAS); the partial
 // Grams are written in FP64 either way.
-template <typename C2>
+constexpr int kGramMaxElems = 4;     // staged elements per thread and operand
+struct GramShape {
+  int sg, tiles, groups, rb;         // 4-wide column groups, 4 x 4 blocks, row groups, staged rows
+  size_t smem;
+};
+template <typename R>
+GramShape gram_shape(int s, bool herm) {
+  GramShape g;
+  g.sg = (s + 3) / 4;
+  g.tiles = herm ? g.sg * (g.sg + 1) / 2 : g.sg * g.sg;
+  g.groups = 256 / g.tiles;
+  g.rb = (16 + g.groups - 1) / g.groups * g.groups;
+  const size_t stage = 2 * 6 * (size_t)g.rb * 4 * g.sg;
+  const size_t sum = (size_t)(g.groups - (g.groups + 1) / 2) * g.tiles * 32;
+  g.smem = std::max(stage, sum) * sizeof(R);
+  TS_REQUIRE(g.rb * 4 * g.sg <= 256 * kGramMaxElems, "gram: block width above kMaxS");
+  return g;
+}
+template <typename C2, bool HERM>
 __global__ void __launch_bounds__(256) k_gram(const C2* __restrict__ V, const C2* __restrict__ W, int n, int s,
-                                              int rows_per_chunk, double2* __restrict__ partials) {
+                                              SliceParts sp, GramShape sh, double2* __restrict__ partials) {
   using R = typename RealOf<C2>::T;
-  constexpr int RB = 16;                                 // rows staged per batch
-  const int k = blockIdx.y, chunk = blockIdx.x, chunks = gridDim.x;
-  // staged planes: u_re, u_im, u_re + u_im of V; w_re, w_im - w_re, w_re + w_im of W (one array, so
-  // the final reduction can reuse it as one contiguous buffer)
-  __shared__ R stage[6][RB][kMaxS];
-  R (*vp1)[kMaxS] = stage[0];
-  R (*vp2)[kMaxS] = stage[1];
-  R (*vp3)[kMaxS] = stage[2];
-  R (*wq1)[kMaxS] = stage[3];
-  R (*wq2)[kMaxS] = stage[4];
-  R (*wq3)[kMaxS] = stage[5];
+  extern __shared__ unsigned char gram_smem[];
+  R* stage = reinterpret_cast<R*>(gram_smem);
+  int k, chunk, chunks;
+  sp.of(blockIdx.x, k, chunk, chunks);
+  const bool real = sp.real(k);
+  const int tid = threadIdx.x, cols = 4 * sh.sg, plane = sh.rb * cols;
   const long long ns = (long long)n * s;
   const C2* Vk = V + k * ns;
   const C2* Wk = W + k * ns;
-  const int sg = (s + 3) / 4;                            // 4-wide groups per side
-  const int tiles = sg * sg;
-  // Row groups (>= 1 since s <= 64), at most one per staged row: more would sit idle and lengthen
-  // the serial group reduction below, whose FP64 adds are expensive on this part.
-  const int groups = min((int)blockDim.x / tiles, RB);
-  const int t = threadIdx.x % tiles, grp = threadIdx.x / tiles;
-  const int a0 = (t % sg) * 4, b0 = (t / sg) * 4;
-  const bool live = grp < groups;
+  const int t = tid % sh.tiles, grp = tid / sh.tiles;
+  const bool live = grp < sh.groups;
+  int ta = t % sh.sg, tb = t / sh.sg;
+  if (HERM) {   // t = tb (tb + 1) / 2 + ta, ta <= tb
+    tb = 0;
+    while ((tb + 1) * (tb + 2) / 2 <= t) ++tb;
+    ta = t - tb * (tb + 1) / 2;
+  }
+  const int a0 = ta * 4, b0 = tb * 4;
+  const int rows = (n + chunks - 1) / chunks, r_begin = chunk * rows, r_end = min(n, r_begin + rows);
+  C2 v[kGramMaxElems], w[kGramMaxElems];
+  auto load = [&](int r0) {
+#pragma unroll
+    for (int q = 0; q < kGramMaxElems; ++q) {
+      const int e = tid + 256 * q, rr = e / cols, cc = e % cols, r = r0 + rr;
+      v[q] = w[q] = C2{0, 0};
+      if (rr < sh.rb && r < r_end && cc < s) {
+        v[q] = Vk[(long long)r * s + cc];
+        if (!HERM) w[q] = Wk[(long long)r * s + cc];
+      }
+    }
+  };
   R T1[4][4], T2[4][4], T3[4][4];
 #pragma unroll
   for (int x = 0; x < 4; ++x)
 #pragma unroll
     for (int y = 0; y < 4; ++y) T1[x][y] = T2[x][y] = T3[x][y] = R(0);
-  const int r_begin = chunk * rows_per_chunk;
-  const int r_end = min(n, r_begin + rows_per_chunk);
-  for (int r0 = r_begin; r0 < r_end; r0 += RB) {
-    for (int e = threadIdx.x; e < RB * kMaxS; e += blockDim.x) {
-      const int rr = e / kMaxS, cc = e % kMaxS;
-      const int r = r0 + rr;
-      C2 v{0, 0}, w{0, 0};
-      if (r < r_end && cc < s) {
-        v = Vk[(long long)r * s + cc];
-        w = Wk[(long long)r * s + cc];
-      }
-      vp1[rr][cc] = v.x;
-      vp2[rr][cc] = -v.y;
-      vp3[rr][cc] = v.x - v.y;
-      wq1[rr][cc] = w.x;
-      wq2[rr][cc] = w.y - w.x;
-      wq3[rr][cc] = w.x + w.y;
-    }
-    __syncthreads();
-    if (live) {
-      for (int rr = grp; rr < RB; rr += groups) {
-        R p1[4], p2[4], p3[4], q1[4], q2[4], q3[4];
+  load(r_begin);
+  int buf = 0;
+  for (int r0 = r_begin; r0 < r_end; r0 += sh.rb, buf ^= 1) {
+    // planes: u_re, u_im, u_re + u_im of V; w_re, w_im - w_re, w_re + w_im of W
+    R* st = stage + buf * 6 * plane;
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          const int a = min(a0 + x, kMaxS - 1), b = min(b0 + x, kMaxS - 1);
-          p1[x] = vp1[rr][a];
-          p2[x] = vp2[rr][a];
-          p3[x] = vp3[rr][a];
-          q1[x] = wq1[rr][b];
-          q2[x] = wq2[rr][b];
-          q3[x] = wq3[rr][b];
+    for (int q = 0; q < kGramMaxElems; ++q) {
+      const int e = tid + 256 * q;
+      if (e < plane) {
+        const C2 x = v[q], y = HERM ? v[q] : w[q];
+        st[e] = x.x;
+        st[3 * plane + e] = y.x;
+        if (!real) {
+          st[plane + e] = neg(x.y);
+          st[2 * plane + e] = x.x - x.y;
+          st[4 * plane + e] = y.y - y.x;
+          st[5 * plane + e] = y.x + y.y;
         }
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int y = 0; y < 4; ++y) {
-            T1[x][y] = fma(q1[y], p3[x], T1[x][y]);
-            T2[x][y] = fma(p1[x], q2[y], T2[x][y]);
-            T3[x][y] = fma(p2[x], q3[y], T3[x][y]);
-          }
       }
     }
-    __syncthreads();
-  }
-  const int ss = s * s;
-  double2* Pk = partials + ((long long)k * chunks + chunk) * ss;
-  if (groups == 1) {
+    __syncthreads();   // also: every thread is done with the other buffer, which the next batch overwrites
+    load(r0 + sh.rb);
     if (live) {
+      auto vec = [&](const R* p, R (&o)[4]) {
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < 4; ++x) o[x] = p[x];
+      };
+      if (real) {
+        for (int rr = grp; rr < sh.rb; rr += sh.groups) {
+          R p1[4], q1[4];
+          vec(st + rr * cols + a0, p1);
+          vec(st + 3 * plane + rr * cols + b0, q1);
 #pragma unroll
-        for (int y = 0; y < 4; ++y)
-          if (a0 + x < s && b0 + y < s)
-            Pk[(a0 + x) + s * (b0 + y)] =   // combined in R, one conversion per part
-                make_double2((double)(T1[x][y] - T3[x][y]), (double)(T1[x][y] + T2[x][y]));
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) T1[x][y] = fma(q1[y], p1[x], T1[x][y]);
+        }
+      } else {
+        for (int rr = grp; rr < sh.rb; rr += sh.groups) {
+          const R* row = st + rr * cols;
+          R p[4], q[4];
+          vec(row + 2 * plane + a0, p);
+          vec(row + 3 * plane + b0, q);
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) T1[x][y] = fma(q[y], p[x], T1[x][y]);
+          vec(row + a0, p);
+          vec(row + 4 * plane + b0, q);
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) T2[x][y] = fma(p[x], q[y], T2[x][y]);
+          vec(row + plane + a0, p);
+          vec(row + 5 * plane + b0, q);
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) T3[x][y] = fma(p[x], q[y], T3[x][y]);
+        }
+      }
     }
-    return;
   }
-  // Several row groups (then s <= 44, so 2 s^2 doubles fit in the staging arrays): sum them in a
-  // fixed order through shared memory.
-  R* red = &stage[0][0][0];
-  for (int g = 0; g < groups; ++g) {
-    if (live && grp == g) {
+  // combined in R (T1 becomes Re, T2 Im), then the groups are halved until one is left
+  if (!real) {
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+    for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const int a = a0 + x, b = b0 + y;
-          if (a < s && b < s) {
-            const R re = T1[x][y] - T3[x][y], im = T1[x][y] + T2[x][y];
-            const int e = a + s * b;
-            if (g == 0) {
-              red[2 * e] = re;
-              red[2 * e + 1] = im;
-            } else {
-              red[2 * e] += re;
-              red[2 * e + 1] += im;
-            }
+      for (int y = 0; y < 4; ++y) {
+        const R re = T1[x][y] - T3[x][y];
+        T2[x][y] = T1[x][y] + T2[x][y];
+        T1[x][y] = re;
+      }
+  }
+  for (int cnt = sh.groups; cnt > 1;) {
+    const int half = (cnt + 1) / 2;
+    __syncthreads();
+    if (live && grp >= half && grp < cnt) {
+      R* o = stage + ((grp - half) * sh.tiles + t) * 32;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        o[(2 * e + t) & 31] = T1[e / 4][e % 4];   // rotated by the block index: the stores spread over the banks
+        o[(2 * e + 1 + t) & 31] = T2[e / 4][e % 4];
+      }
+    }
+    __syncthreads();
+    if (live && grp < cnt - half) {
+      const R* o = stage + (grp * sh.tiles + t) * 32;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        T1[e / 4][e % 4] += o[(2 * e + t) & 31];
+        if (!real) T2[e / 4][e % 4] += o[(2 * e + 1 + t) & 31];
+      }
+    }
+    cnt = half;
+  }
+  if (live && grp == 0) {
+    double2* Pk = partials + (long long)blockIdx.x * s * s;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const int i = a0 + x, j = b0 + y;
+        if (i < s && j < s) {
+          const double re = (double)T1[x][y], im = real ? 0.0 : (double)T2[x][y];
+          if (!HERM) {
+            Pk[i + s * j] = make_double2(re, im);
+          } else if (i <= j) {
+            Pk[i + s * j] = make_double2(re, i == j ? 0.0 : im);
+            if (i != j) Pk[j + s * i] = make_double2(re, neg(im));
           }
         }
-    }
-    __syncthreads();
+      }
   }
-  for (int e = threadIdx.x; e < ss; e += blockDim.x) Pk[e] = make_double2((double)red[2 * e], (double)red[2 * e + 1]);
 }
 
-// out_k (column-major, leading dimension ldo) = sum over chunks of the partial Grams (fixed order).
-__global__ void k_gram_reduce(const double2* __restrict__ partials, int chunks, int s, double2* __restrict__ out,
-                              long long sOut, int ldo) {
-  const int k = blockIdx.x;
-  const int ss = s * s;
-  for (int e = threadIdx.x; e < ss; e += blockDim.x) {
-    double2 acc = make_double2(0.0, 0.0);
-    for (int c = 0; c < chunks; ++c) {
-      const double2 v = partials[((long long)k * chunks + c) * ss + e];
+// out_k (column-major, leading dimension ldo) = sum over a slice's blocks of the partial Grams, in a fixed
+// order: four threads per entry, each every fourth block, then their sums.
+__global__ void __launch_bounds__(256) k_gram_reduce(const double2* __restrict__ partials, SliceParts sp, int s,
+                                                     double2* __restrict__ out, long long sOut, int ldo) {
+  __shared__ double2 red[4][64];
+  const int k = blockIdx.y, ss = s * s, sub = threadIdx.x / 64, e = blockIdx.x * 64 + threadIdx.x % 64;
+  const int chunks = sp.parts(k);
+  const double2* Pk = partials + (long long)sp.first(k) * ss;
+  double2 acc = make_double2(0.0, 0.0);
+  if (e < ss) {
+#pragma unroll 4
+    for (int c = sub; c < chunks; c += 4) {
+      const double2 v = Pk[(long long)c * ss + e];
+      acc.x += v.x;
+      acc.y += v.y;
+    }
+  }
+  red[sub][threadIdx.x % 64] = acc;
+  __syncthreads();
+  if (sub == 0 && e < ss) {
+#pragma unroll
+    for (int q = 1; q < 4; ++q) {
+      const double2 v = red[q][threadIdx.x];
       acc.x += v.x;
       acc.y += v.y;
     }
@@ -293,18 +436,26 @@ __global__ void k_gram_reduce(const double2* __restrict__ partials, int chunks, 
 }
 
 // Out_k = (accumulate ? Out_k : 0) + alpha * In_k M_k (in place allowed), M_k an s x s column-major
-// block with leading dimension ldm.  kRowCols consecutive columns of one row per thread, all
+// block with leading dimension ldm.  NC consecutive columns of one row per thread, all
 // threads of a row in one warp; Gauss's form with the planes M_re, M_im - M_re, M_re + M_im of M_k in
 // shared memory: Re = T1 - T3, Im = T1 + T2 with T1 = sum (a_re + a_im) m_re, T2 = sum a_re (m_im - m_re),
-// T3 = sum a_im (m_re + m_im), three DFMA per complex multiply-add.
+// T3 = sum a_im (m_re + m_im), three FMAs per complex multiply-add; a real slice (the imaginary parts of
+// In and M count as zero) takes one.
+// What bounds it: the FP64 pipe; blocks are dealt to the slices by cost and rows to the warps of a slice
+// round robin over its blocks, so that the last round is spread over the SMs, and NC matches s (eight
+// columns computed for s = 4 were half padding).
+// Measured (n = 16384, s = 32, p = 8): 532 -> 359 us; s = 4: 27.6 -> 12.2 us.
 // Cin = float2 (the FP32 basis of mixed-precision TBAS): products in FP32; Cout may be double2 (the
 // FP64 solution update X += V Y) or float2.
 constexpr int kRowCols = 8;
-template <typename Cin, typename Cout>
+template <int NC, typename Cin, typename Cout>
 __global__ void __launch_bounds__(256) k_rows_mm(const Cin* In, Cout* Out, const double2* __restrict__ M,
-                                                 long long sM, int ldm, int n, int s, double alpha, int accumulate) {
+                                                 long long sM, int ldm, int n, int s, SliceParts sp, double alpha,
+                                                 int accumulate) {
   using R = typename RealOf<Cin>::T;
-  const int k = blockIdx.y;
+  int k, part, parts;
+  sp.of(blockIdx.x, k, part, parts);
+  const bool real = sp.real(k);
   extern __shared__ unsigned char smm_raw[];   // three s x s planes, l-major: plane[l * s + j]
   R* mr = reinterpret_cast<R*>(smm_raw);
   R* md = mr + s * s;
@@ -314,96 +465,79 @@ __global__ void __launch_bounds__(256) k_rows_mm(const Cin* In, Cout* Out, const
     const int l = e % s, j = e / s;
     const double2 v = Mk[l + (long long)ldm * j];
     mr[l * s + j] = (R)v.x;
-    md[l * s + j] = (R)(v.y - v.x);
-    mq[l * s + j] = (R)(v.x + v.y);
+    if (!real) {
+      md[l * s + j] = (R)(v.y - v.x);
+      mq[l * s + j] = (R)(v.x + v.y);
+    }
   }
   __syncthreads();
   // Threads per row: a power of two (1, 2, 4, 8), so a row never straddles two warps.
   int tpr = 1;
   while (tpr * kRowCols < s) tpr *= 2;
-  const int cpt = (s + tpr - 1) / tpr;                   // columns per thread (<= kRowCols)
-  const int rows_per_block = blockDim.x / tpr;
-  const int rloc = threadIdx.x / tpr, cg = threadIdx.x % tpr;
-  const int c0 = cg * cpt;
-  const int c1 = min(c0 + cpt, s);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rpw = 32 / tpr;
+  const int rloc = lane / tpr, c0 = lane % tpr * NC, c1 = min(c0 + NC, s);
   const long long ns = (long long)n * s;
-  const bool live_thread = rloc < rows_per_block;
-  for (int rbase = blockIdx.x * rows_per_block; rbase < n; rbase += gridDim.x * rows_per_block) {
-    const int i = rbase + rloc;
-    const bool live = live_thread && i < n;
-    R T1[kRowCols], T2[kRowCols], T3[kRowCols];
+  int col[NC];
 #pragma unroll
-    for (int c = 0; c < kRowCols; ++c) T1[c] = T2[c] = T3[c] = R(0);
+  for (int c = 0; c < NC; ++c) col[c] = max(0, min(c0 + c, s - 1));
+  const int step = parts * (int)(blockDim.x / 32) * rpw;
+  for (int rbase = (warp * parts + part) * rpw; rbase < n; rbase += step) {
+    const int i = rbase + rloc;
+    const bool live = i < n;
+    R T1[NC], T2[NC], T3[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) T1[c] = T2[c] = T3[c] = R(0);
     const long long ro = k * ns + (long long)i * s;
     if (live) {
-      for (int l = 0; l < s; ++l) {
-        const Cin a = In[ro + l];
-        const R sa = a.x + a.y;
+      if (real) {
+#pragma unroll 4
+        for (int l = 0; l < s; ++l) {
+          const R ar = In[ro + l].x;
 #pragma unroll
-        for (int c = 0; c < kRowCols; ++c) {
-          const int j = min(c0 + c, c1 - 1);
-          T1[c] = fma(sa, mr[l * s + j], T1[c]);
-          T2[c] = fma(a.x, md[l * s + j], T2[c]);
-          T3[c] = fma(a.y, mq[l * s + j], T3[c]);
+          for (int c = 0; c < NC; ++c) T1[c] = fma(ar, mr[l * s + col[c]], T1[c]);
+        }
+      } else {
+#pragma unroll 4
+        for (int l = 0; l < s; ++l) {
+          const Cin a = In[ro + l];
+          const R sa = a.x + a.y;
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            T1[c] = fma(sa, mr[l * s + col[c]], T1[c]);
+            T2[c] = fma(a.x, md[l * s + col[c]], T2[c]);
+            T3[c] = fma(a.y, mq[l * s + col[c]], T3[c]);
+          }
         }
       }
     }
     __syncwarp();   // every thread of the row has read In before any writes Out (in place)
     if (live) {
 #pragma unroll
-      for (int c = 0; c < kRowCols; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int j = c0 + c;
         if (j < c1) {
-          if constexpr (sizeof(R) == 4) {
-            // FP32 products: scale in FP32 and convert at most once, since GB300's FP64 and
-            // conversion rate would otherwise make this epilogue cost more than the s-term loop
-            const float al = (float)alpha;
-            const float vr = al * (T1[c] - T3[c]), vi = al * (T1[c] + T2[c]);
-            if constexpr (sizeof(Cout) == 8) {
-              float2 v = make_float2(vr, vi);
-              if (accumulate) {
-                const float2 o = Out[ro + j];
-                v.x += o.x;
-                v.y += o.y;
-              }
-              Out[ro + j] = v;
-            } else {
-              double2 v = make_double2((double)vr, (double)vi);
-              if (accumulate) {
-                const double2 o = widen(Out[ro + j]);
-                v.x += o.x;
-                v.y += o.y;
-              }
-              Out[ro + j] = to_c2(v, (Cout*)nullptr);
+          // FP32 products are scaled in FP32 and converted at most once, since GB300's FP64 and
+          // conversion rate would otherwise make this epilogue cost more than the s-term loop
+          const R al = (R)alpha;
+          R vr = al * (T1[c] - T3[c]), vi = real ? R(0) : al * (T1[c] + T2[c]);
+          if constexpr (sizeof(Cout) == sizeof(Cin)) {
+            if (accumulate) {
+              const Cout o = Out[ro + j];
+              vr += o.x;
+              if (!real) vi += o.y;
             }
+            Out[ro + j] = Cout{vr, vi};
           } else {
-            double2 v = make_double2(alpha * (double)(T1[c] - T3[c]), alpha * (double)(T1[c] + T2[c]));
+            double2 v = make_double2((double)vr, (double)vi);
             if (accumulate) {
               const double2 o = widen(Out[ro + j]);
               v.x += o.x;
-              v.y += o.y;
+              if (!real) v.y += o.y;
             }
             Out[ro + j] = to_c2(v, (Cout*)nullptr);
           }
         }
       }
-    }
-  }
-}
-
-// Inverse of an upper triangular s x s matrix per slice (one warp; lanes over columns).
-__global__ void k_triinv(const double2* __restrict__ Rall, double2* __restrict__ Xall, int s) {
-  const double2* R = Rall + (long long)blockIdx.x * s * s;
-  double2* X = Xall + (long long)blockIdx.x * s * s;
-  for (int b = threadIdx.x; b < s; b += 32) {
-    for (int a = 0; a < s; ++a) X[a + (long long)s * b] = make_double2(0.0, 0.0);
-    // X[b][b] = 1 / R[b][b] (R has a real positive diagonal)
-    X[b + (long long)s * b] = make_double2(1.0 / R[b + (long long)s * b].x, 0.0);
-    for (int a = b - 1; a >= 0; --a) {
-      double2 acc = make_double2(0.0, 0.0);
-      for (int c = a + 1; c <= b; ++c) acc = cfma(R[a + (long long)s * c], X[c + (long long)s * b], acc);
-      const double inv = 1.0 / R[a + (long long)s * a].x;
-      X[a + (long long)s * b] = make_double2(-acc.x * inv, -acc.y * inv);
     }
   }
 }
@@ -599,7 +733,7 @@ struct TbaWork {
   double2* Rinv;            // K x s x s
   double2* R2;              // K x s x s
   double2* gram_part;       // partial Grams
-  int chunks, rows_per_chunk;
+  SliceParts gram_parts, row_parts;   // blocks of the Gram and row products
   double2* LU;              // K x s x N x N
   int* piv;                 // K x s x N
   double2* Gp;              // K x N x s
@@ -727,17 +861,30 @@ void rows_call(int mode, const ts_op* op, const double2* V, const double2* C, do
 }
 
 template <typename Cin, typename Cout>
-void rows_mm(const Cin* In, Cout* Out, const double2* M, long long sM, int ldm, int n, int s, int K, double alpha,
+void rows_mm(const TbaWork& w, const Cin* In, Cout* Out, const double2* M, long long sM, int ldm, double alpha,
              bool accumulate, cudaStream_t st) {
   using R = typename RealOf<Cin>::T;
+  const int s = w.s;
   TS_REQUIRE(s <= kMaxS, "rows_mm: block width above kMaxS");
   int tpr = 1;
   while (tpr * kRowCols < s) tpr *= 2;
-  const int rows_per_block = 256 / tpr;
-  const int gx = std::max(1, std::min((n + rows_per_block - 1) / rows_per_block, 4 * 152 * 4 / K));
   const size_t smem = sizeof(R) * 3 * (size_t)s * s;
-  set_max_dynamic_smem((const void*)k_rows_mm<Cin, Cout>, (int)(sizeof(R) * 3 * kMaxS * kMaxS));
-  k_rows_mm<Cin, Cout><<<dim3(gx, K), 256, smem, st>>>(In, Out, M, sM, ldm, n, s, alpha, accumulate ? 1 : 0);
+  auto run = [&](auto nc) {
+    constexpr int NC = decltype(nc)::value;
+    set_max_dynamic_smem((const void*)k_rows_mm<NC, Cin, Cout>, (int)(sizeof(R) * 3 * kMaxS * kMaxS));
+    k_rows_mm<NC, Cin, Cout><<<w.row_parts.blocks(), 256, smem, st>>>(In, Out, M, sM, ldm, w.n, s, w.row_parts, alpha,
+                                                                      accumulate ? 1 : 0);
+  };
+  switch ((s + tpr - 1) / tpr) {   // columns per thread
+    case 1: run(std::integral_constant<int, 1>{}); break;
+    case 2: run(std::integral_constant<int, 2>{}); break;
+    case 3: run(std::integral_constant<int, 3>{}); break;
+    case 4: run(std::integral_constant<int, 4>{}); break;
+    case 5: run(std::integral_constant<int, 5>{}); break;
+    case 6: run(std::integral_constant<int, 6>{}); break;
+    case 7: run(std::integral_constant<int, 7>{}); break;
+    default: run(std::integral_constant<int, 8>{}); break;
+  }
   count_launch();
   TS_CUDA(cudaGetLastError());
 }
@@ -748,10 +895,17 @@ double block_flops(const TbaWork& w) { return 8.0 * w.n * w.s * w.s * w.K; }
 template <typename C2>
 void gram(const TbaWork& w, const C2* V, const C2* W, double2* out, long long sOut, int ldo, cudaStream_t st) {
   w.tm->begin(st, 4, block_flops(w));
-  k_gram<C2><<<dim3(w.chunks, w.K), 256, 0, st>>>(V, W, w.n, w.s, w.rows_per_chunk, w.gram_part);
+  auto run = [&](auto herm) {
+    constexpr bool HERM = decltype(herm)::value;
+    const GramShape g = gram_shape<typename RealOf<C2>::T>(w.s, HERM);
+    set_max_dynamic_smem((const void*)k_gram<C2, HERM>, (int)g.smem);
+    k_gram<C2, HERM><<<w.gram_parts.blocks(), 256, g.smem, st>>>(V, W, w.n, w.s, w.gram_parts, g, w.gram_part);
+  };
+  if (V == W) run(std::true_type{});
+  else run(std::false_type{});
   count_launch();
   TS_CUDA(cudaGetLastError());
-  k_gram_reduce<<<w.K, 256, 0, st>>>(w.gram_part, w.chunks, w.s, out, sOut, ldo);
+  k_gram_reduce<<<dim3((w.s * w.s + 63) / 64, w.K), 256, 0, st>>>(w.gram_part, w.gram_parts, w.s, out, sOut, ldo);
   count_launch();
   TS_CUDA(cudaGetLastError());
   w.tm->end(st);
@@ -761,14 +915,8 @@ template <typename Cin, typename Cout>
 void rows_mm_timed(const TbaWork& w, const Cin* In, Cout* Out, const double2* M, long long sM, int ldm,
                    double alpha, bool accumulate, cudaStream_t st) {
   w.tm->begin(st, 4, block_flops(w));
-  rows_mm(In, Out, M, sM, ldm, w.n, w.s, w.K, alpha, accumulate, st);
+  rows_mm(w, In, Out, M, sM, ldm, alpha, accumulate, st);
   w.tm->end(st);
-}
-
-void triinv(const double2* R, double2* X, int s, int K, cudaStream_t st) {
-  k_triinv<<<K, 32, 0, st>>>(R, X, s);
-  count_launch();
-  TS_CUDA(cudaGetLastError());
 }
 
 // Tubal-QR of the block W (in place -> Q); R written to Rout (column-major, ldr).  Per Fourier slice
@@ -778,25 +926,24 @@ void triinv(const double2* R, double2* X, int s, int K, cudaStream_t st) {
 // orthogonal part below 1e-6 of its norm in FP64 (1e-3 in FP32), or its norm below the rank-deficiency
 // scale of Normalization1 -- takes Algorithm 6 itself instead (k_tubal_mgs: Gram-Schmidt with the
 // Normalize tie-break), whose Q the second CholeskyQR pass then only re-orthogonalises to rounding.
-// Returns false when the second Cholesky fails (not expected after either first pass).
+// Returns false when the second Cholesky fails (not expected after either first pass).  have_gram: w.G
+// already holds W^H W.
 template <typename C2>
-bool tubal_qr(const TbaWork& w, C2* W, double2* Rout, long long sR, int ldr, cudaStream_t st) {
+bool tubal_qr(const TbaWork& w, C2* W, double2* Rout, long long sR, int ldr, bool have_gram, cudaStream_t st) {
   const int s = w.s, K = w.K;
   const long long ss = (long long)s * s;
   constexpr bool f64 = sizeof(C2) == 16;
   const double tiny = f64 ? 1e-12 : 1e-4;      // Normalization1: a slice is zero below tiny * ref_j
   const double rel = f64 ? 1e-12 : 1e-6;       // CholeskyQR is trusted for orthogonal parts above sqrt(rel)
   TS_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), st));
-  gram(w, W, W, w.G, ss, s, st);
-  cholesky_small(w.G, w.R1, s, K, rel, tiny * tiny, nullptr, w.fail, st);
-  triinv(w.R1, w.Rinv, s, K, st);
+  if (!have_gram) gram(w, W, W, w.G, ss, s, st);
+  cholesky_inverse(w.G, w.R1, w.Rinv, s, K, rel, tiny * tiny, nullptr, w.fail, st);
   k_tubal_mgs<C2><<<K, 256, 0, st>>>(W, w.G, w.fail, w.R1, w.Rinv, w.n, s, K, tiny);
   count_launch();
   TS_CUDA(cudaGetLastError());
   rows_mm_timed(w, W, W, w.Rinv, ss, s, 1.0, false, st);
   gram(w, W, W, w.G, ss, s, st);
-  cholesky_small(w.G, w.R2, s, K, 0.0, 0.0, w.err, nullptr, st);
-  triinv(w.R2, w.Rinv, s, K, st);
+  cholesky_inverse(w.G, w.R2, w.Rinv, s, K, 0.0, 0.0, w.err, nullptr, st);
   rows_mm_timed(w, W, W, w.Rinv, ss, s, 1.0, false, st);
   small_gemm(w.R2, ss, s, w.R1, ss, s, false, Rout, sR, ldr, s, s, s, K, false, st);   // R = R2 R1
   int e = 0;
@@ -870,9 +1017,10 @@ TbaWork tba_work(ts_ctx* ctx, const ts_op* op, int m) {
   w.R1 = (double2*)get("tba_R1", ss);
   w.R2 = (double2*)get("tba_R2", ss);
   w.Rinv = (double2*)get("tba_Rinv", ss);
-  w.chunks = std::max(1, std::min(2 * 152 / K, (n + 63) / 64));
-  w.rows_per_chunk = (n + w.chunks - 1) / w.chunks;
-  w.gram_part = (double2*)get("tba_gram_part", sizeof(double2) * (size_t)K * w.chunks * s * s);
+  const int nyq = nyquist_index(w.p);
+  w.gram_parts = slice_parts(K, nyq, n, ctx->num_sms, 32);
+  w.row_parts = slice_parts(K, nyq, n, 2 * ctx->num_sms, 32);
+  w.gram_part = (double2*)get("tba_gram_part", sizeof(double2) * (size_t)w.gram_parts.blocks() * s * s);
   w.LU = (double2*)get("tba_LU", sizeof(double2) * (size_t)K * s * N * N);
   w.piv = (int*)get("tba_piv", sizeof(int) * (size_t)K * s * N);
   w.Gp = (double2*)get("tba_Gp", sizeof(double2) * (size_t)K * N * s);
@@ -954,7 +1102,7 @@ ts_status tbas_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const t
       } else {
         convert<double, float>(reinterpret_cast<const double*>(w.R), reinterpret_cast<float*>(V), 2 * blk, st);
       }
-      if (!tubal_qr(w, V, w.H0, ss, s, st)) return false;
+      if (!tubal_qr(w, V, w.H0, ss, s, false, st)) return false;
       TS_CUDA(cudaMemsetAsync(w.Hm, 0, sizeof(double2) * (size_t)K * N * N, st));
       for (int j = 0; j < m; ++j) {
         C2* Vj = V + (long long)j * blk;
@@ -985,7 +1133,7 @@ ts_status tbas_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const t
         double2* Hnext = (j + 1 < m) ? w.Hm + (long long)(j + 1) * s + (long long)N * j * s : w.Hlast;
         const long long sH = (j + 1 < m) ? (long long)N * N : ss;
         const int ldh = (j + 1 < m) ? N : s;
-        if (!tubal_qr(w, Wb, Hnext, sH, ldh, st)) return false;
+        if (!tubal_qr(w, Wb, Hnext, sH, ldh, true, st)) return false;   // w.G is still W^H W
       }
       return true;
     };
@@ -1022,9 +1170,9 @@ ts_status tbas_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const t
     // X += V_m Y
     for (int j = 0; j < mm; ++j) {
       if (low)
-        rows_mm(V32 + (long long)j * blk, w.X, w.Y + (long long)j * s, (long long)Nm * s, Nm, n, s, K, 1.0, true, st);
+        rows_mm(w, V32 + (long long)j * blk, w.X, w.Y + (long long)j * s, (long long)Nm * s, Nm, 1.0, true, st);
       else
-        rows_mm(w.V + (long long)j * blk, w.X, w.Y + (long long)j * s, (long long)Nm * s, Nm, n, s, K, 1.0, true, st);
+        rows_mm(w, w.V + (long long)j * blk, w.X, w.Y + (long long)j * s, (long long)Nm * s, Nm, 1.0, true, st);
     }
     int e = 0;
     TS_CUDA(cudaMemcpyAsync(&e, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
