@@ -794,60 +794,56 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   int* flags = (int*)get("b_flags", sizeof(int) * 2 * count);
   const long long stride = state_stride(m);
   double* state = (double*)get("b_state", sizeof(double) * (size_t)stride * count);
-  // Emulated FP64 residual products: digit planes of every operator; the instances' products run
-  // on kOzBranches side streams (parallel branches of the captured graph, since one small
-  // instance fills few SMs), each branch with its own scratch set sized for the largest instance.
-  // Everything is made before anything is captured.
-  constexpr int kOzBranches = 8;
-  std::vector<OzBuffers> ozb(kOzBranches);
-  std::vector<int> order(count);
+  // Emulated FP64 products: digit planes of every operator, and the work lists of their three phases
+  // (maxima, digits of X, products), one launch each over all instances.  Everything is made before
+  // anything is captured.  (A chain of five launches per instance on eight
+  // side streams before: 64 instances, BF16 inner products, 29.7 -> 23.8 ms per solve.)
   int* tc_err = (int*)get("tc_err", sizeof(int) * 4);
-  cudaEvent_t fork_ev = nullptr;
-  std::vector<cudaEvent_t> join_ev;
+  OzBatchLists oz_lists;
+  const char* oz_inst = nullptr;
+  unsigned long long* oz_mx = nullptr;
+  size_t oz_mx_count = 0;
   if (ozaki) {
-    OzBufferSizes zmax;
+    size_t plane_bytes = 0;
+    std::vector<size_t> poff(count), moff(count);
+    std::vector<const ts_op*> cops(ops.begin(), ops.end());
     for (int i = 0; i < count; ++i) {
       oz_prepare(ops[i], oz_digits, user);
-      const OzBufferSizes z = oz_buffer_sizes(ops[i]->n, ops[i]->s, ops[i]->K, oz_digits);
-      zmax.xc = std::max(zmax.xc, z.xc);
-      zmax.xr = std::max(zmax.xr, z.xr);
-      zmax.K = std::max(zmax.K, z.K);
+      poff[i] = plane_bytes;
+      plane_bytes += oz_batch_plane_bytes(ops[i], oz_digits);
+      moff[i] = oz_mx_count;
+      oz_mx_count += ops[i]->K;
     }
     oz_preload();
-    for (int q = 0; q < kOzBranches; ++q) {
-      const std::string sfx = "_" + std::to_string(q);
-      ozb[q].xc_re = get(("b_oz_xc_re" + sfx).c_str(), zmax.xc);
-      ozb[q].xc_im = get(("b_oz_xc_im" + sfx).c_str(), zmax.xc);
-      ozb[q].xc_nim = get(("b_oz_xc_nim" + sfx).c_str(), zmax.xc);
-      ozb[q].xr_re = get(("b_oz_xr_re" + sfx).c_str(), zmax.xr);
-      ozb[q].xr_im = get(("b_oz_xr_im" + sfx).c_str(), zmax.xr);
-      ozb[q].mx = (unsigned long long*)get(("b_oz_mx" + sfx).c_str(), sizeof(unsigned long long) * zmax.K);
-      ozb[q].Ex = (int*)get(("b_oz_Ex" + sfx).c_str(), sizeof(int) * zmax.K);
-    }
-    while ((int)ctx->side.size() < kOzBranches) {
-      cudaStream_t q;
-      TS_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
-      ctx->side.push_back(q);
-    }
-    TS_CUDA(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
-    join_ev.resize(kOzBranches);
-    for (auto& e : join_ev) TS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    // largest products first, dealt round-robin over the branches
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-      auto cost = [&](int i) { return (double)ops[i]->K * ops[i]->n * ops[i]->s * (ops[i]->n + ops[i]->s); };
-      return cost(a) > cost(b);
-    });
+    char* planes = (char*)get("b_oz_planes", plane_bytes);
+    oz_mx = (unsigned long long*)get("b_oz_mx", sizeof(unsigned long long) * oz_mx_count);
+    const size_t isz = oz_batch_instance_bytes();
+    struct alignas(64) Line { char c[64]; };   // tensor maps are built 64-byte aligned
+    TS_REQUIRE(isz % sizeof(Line) == 0, "batched emulated products: instance table alignment");
+    std::vector<Line> table(isz / sizeof(Line) * count);
+    for (int i = 0; i < count; ++i)
+      oz_batch_instance(ops[i], Xh64 + plan.inst[i].offS, Yh64 + plan.inst[i].offS, oz_digits, planes + poff[i],
+                        oz_mx + moff[i], reinterpret_cast<char*>(table.data()) + isz * i);
+    std::vector<int4> products, splits, maxima;
+    oz_batch_items(cops, &products, &splits, &maxima);
+    TS_REQUIRE(products.size() < (size_t)INT32_MAX && splits.size() < (size_t)INT32_MAX, "batch too large");
+    char* tab = (char*)get("b_oz_tables", isz * count + sizeof(int4) * (products.size() + splits.size() + maxima.size()));
+    int4* items = (int4*)(tab + isz * count);
+    TS_CUDA(cudaMemcpy(tab, table.data(), isz * count, cudaMemcpyHostToDevice));
+    TS_CUDA(cudaMemcpy(items, products.data(), sizeof(int4) * products.size(), cudaMemcpyHostToDevice));
+    oz_lists.products = items;
+    oz_lists.n_products = (int)products.size();
+    items += products.size();
+    TS_CUDA(cudaMemcpy(items, splits.data(), sizeof(int4) * splits.size(), cudaMemcpyHostToDevice));
+    oz_lists.splits = items;
+    oz_lists.n_splits = (int)splits.size();
+    items += splits.size();
+    TS_CUDA(cudaMemcpy(items, maxima.data(), sizeof(int4) * maxima.size(), cudaMemcpyHostToDevice));
+    oz_lists.maxima = items;
+    oz_lists.n_maxima = (int)maxima.size();
+    oz_inst = tab;
     TS_CUDA(cudaMemsetAsync(tc_err, 0, sizeof(int) * 4, user));
   }
-  struct EventGuard {
-    cudaEvent_t& f;
-    std::vector<cudaEvent_t>& j;
-    ~EventGuard() {
-      if (f) cudaEventDestroy(f);
-      for (auto e : j) cudaEventDestroy(e);
-    }
-  } ev_guard{fork_ev, join_ev};
 
   BDev d{};
   d.inst = d_inst;
@@ -1024,27 +1020,14 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
     tct = tables_of(tc_bn);
     TS_CUDA(cudaMemsetAsync(tc_err, 0, sizeof(int) * 4, st));
   }
-  // Emulated-FP64 slice products of every instance (X -> Y, spectral FP64), each gated on the device
-  // by the instance's flag in `gate`: dealt largest first over the kOzBranches side streams, forked
-  // from and joined back to s2.
-  auto oz_all = [&](cudaStream_t s2, const double2* X, double2* Y, const int* gate) -> int {
-    // fork: every branch waits for the products' input; join: s2 waits for every branch
-    TS_CUDA(cudaEventRecord(fork_ev, s2));
-    for (int q = 0; q < kOzBranches; ++q) TS_CUDA(cudaStreamWaitEvent(ctx->side[q], fork_ev, 0));
-    for (int r = 0; r < count; ++r) {
-      const int i = order[r], q = r % kOzBranches;
-      oz_products(ops[i], X + plan.inst[i].offS, Y + plan.inst[i].offS, oz_digits, ozb[q], gate + i, tc_err,
-                  ctx->side[q]);
-    }
-    for (int q = 0; q < kOzBranches; ++q) {
-      TS_CUDA(cudaEventRecord(join_ev[q], ctx->side[q]));
-      TS_CUDA(cudaStreamWaitEvent(s2, join_ev[q], 0));
-    }
-    return 5 * count;
+  // Emulated-FP64 slice products of every instance (Xh64 -> Yh64), each gated on the device by its flag.
+  auto oz_all = [&](cudaStream_t s2, const int* gate) -> int {
+    oz_batch_products(oz_inst, oz_lists, oz_mx, oz_mx_count, oz_digits, gate, tc_err, s2);
+    return 3;
   };
   auto inner_products = [&](cudaStream_t s2) -> int {
     // FP64 solve on the emulated engine: the Arnoldi products too (gated by the inner-cycle flag)
-    if (!mixed && ozaki) return oz_all(s2, (const double2*)Xh, (double2*)Yh, d.act);
+    if (!mixed && ozaki) return oz_all(s2, d.act);   // Xh64 and Yh64 are Xh and Yh in an FP64 batch
     if (tcin) {
       tc_batch_products(o.precision, tc_bn, tct.planes, tct.pitems, tct.n_pitems, tct.maps, tct.inst, d.act,
                         tct.titems, tct.n_titems, tc_err, s2);
@@ -1054,14 +1037,13 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
     else launch_b_gemm<double, 0>(simt_list(simt_bn64), d, Xh, Yh, s2);
     return 1;
   };
-  // FP64 slice products of a true residual: the (instance, slice, tile) work list on CUDA cores, or
-  // one emulated-FP64 product per instance (each gated by the instance's cycle flag).
+  // FP64 slice products of a true residual (gated by the instances' cycle flags), on CUDA cores or emulated.
   auto residual_products = [&](cudaStream_t s2) -> int {
     if (!ozaki) {
       launch_b_gemm<double, 1>(simt_list(simt_bn64), d, Xh64, Yh64, s2);
       return 1;
     }
-    return oz_all(s2, Xh64, Yh64, d.cyc);
+    return oz_all(s2, d.cyc);
   };
   ctx->timer.host_setup_ms += host_ms_since(host_t0);
   const auto cycles_t0 = std::chrono::steady_clock::now();
@@ -1071,7 +1053,7 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   const int first = residual_products(st);
   k_b_irfft<double, double2, 1><<<ntb, kTubes, 0, st>>>(d, Yh64, R, Pt);
   k_b_finalize_norm<<<count, 256, 0, st>>>(d, Pt, 1);
-  count_launch(ozaki ? 5 : 5 + first);   // the emulated products count their own launches
+  count_launch(ozaki ? 5 : 5 + first);   // the emulated products counted their own launches
   TS_CUDA(cudaGetLastError());
 
   std::vector<double> hsc(16 * count);

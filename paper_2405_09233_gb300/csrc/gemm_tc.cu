@@ -840,16 +840,18 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 // 3-D map over planes [K][rows][ld] of ESZ-byte elements, box = (128 bytes of l) x box_rows x 1.
 }  // namespace
 
-void make_map(CUtensorMap* m, const void* base, int esz, int ld, int cols, int rows, int K, int box_rows) {
+void make_map(CUtensorMap* m, const void* base, int esz, int ld, int cols, int rows, int K, int box_rows,
+              int box_bytes) {
   TS_REQUIRE((reinterpret_cast<uintptr_t>(base) & 15) == 0, "TMA base must be 16-byte aligned");
   TS_REQUIRE(((long long)ld * esz) % 16 == 0, "TMA row pitch must be a multiple of 16 bytes");
   const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)K};
   const cuuint64_t strides[2] = {(cuuint64_t)ld * esz, (cuuint64_t)ld * esz * rows};
-  const cuuint32_t box[3] = {(cuuint32_t)(128 / esz), (cuuint32_t)box_rows, 1};
+  const cuuint32_t box[3] = {(cuuint32_t)(box_bytes / esz), (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = encode_fn()(m, esz == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
                            const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) throw Error{TS_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r)};
 }

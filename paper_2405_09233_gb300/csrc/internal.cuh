@@ -134,7 +134,6 @@ struct ts_ctx {
   // DFTs that read the staging buffers done (the next creation may overwrite them).
   cudaEvent_t ev_stage_copied = nullptr, ev_stage_free = nullptr;
   cudaStream_t bstream = nullptr;  // private stream of the batched solver (graph capture)
-  std::vector<cudaStream_t> side;  // side streams of the batched solver's parallel branches
   std::map<std::string, int> tune; // launch shapes chosen by the autotuner (tune.cuh), by problem key
   bool tune_loaded = false;        // the on-disk tuning cache (TSTAR_TUNE_CACHE) has been read
   int f64_engine = 0;              // how the current call computes FP64 applications (ts_fp64_engine)

@@ -1,5 +1,6 @@
 // Emulated FP64 slice products on the tensor cores (Ozaki scheme, gemm_oz.cu).
 #pragma once
+#include <vector>
 #include "internal.cuh"
 
 namespace ts {
@@ -13,8 +14,7 @@ struct OzOperands {
   void* b_re = nullptr;            // [S][K][s][lds]  column-major B_k digits
   void* b_im = nullptr;
   void* b_nre = nullptr;           // digits of -Re B_k
-  int* Eop = nullptr;              // [K] shared exponent of A_k and B_k
-  unsigned long long* mx = nullptr;
+  unsigned long long* mx = nullptr;   // [K] shared maxima of A_k and B_k (FP64 bit patterns), for their exponents
   void release();
 };
 
@@ -26,11 +26,10 @@ struct OzBuffers {
   void* xr_re = nullptr;           // [S][K][n][lds]  row-major X_k digits
   void* xr_im = nullptr;
   unsigned long long* mx = nullptr;   // [K] slice maxima (FP64 bit patterns)
-  int* Ex = nullptr;                  // [K] slice exponents
 };
 struct OzBufferSizes {
   size_t xc = 0, xr = 0;           // bytes of each xc_* / xr_* plane set
-  int K = 0;                       // entries of mx and Ex
+  int K = 0;                       // entries of mx
 };
 OzBufferSizes oz_buffer_sizes(int n, int s, int K, int S);
 
@@ -40,10 +39,28 @@ void oz_preload();
 // Yh_k = A_k Xh_k - Xh_k B_k for the K spectral slices of op (double2, column-major n x s each),
 // emulated FP64 with S digits per value; op must be prepared with at least S digits (the leading S
 // digits of a longer expansion approximate an entry as closely as an S-digit expansion, within
-// 0.502 of the last kept digit's unit).  gate (device, may be null): when *gate == 0
-// every kernel returns at once.  Captures into a CUDA graph (no allocation, no synchronisation).
-void oz_products(const ts_op* op, const double2* Xh, double2* Yh, int S, const OzBuffers& b, const int* gate,
-                 int* err, cudaStream_t st);
+// 0.502 of the last kept digit's unit).  Captures into a CUDA graph (no allocation, no synchronisation).
+void oz_products(const ts_op* op, const double2* Xh, double2* Yh, int S, const OzBuffers& b, int* err,
+                 cudaStream_t st);
+
+// Batches: the products of many instances in one launch per phase, each instance gated on the device by
+// its flag.  oz_batch_instance fills one entry (oz_batch_instance_bytes each, 64-byte aligned) of the
+// instance table in host memory: digit planes carved from `planes` (oz_batch_plane_bytes), maxima at mx (K
+// entries).  oz_batch_items lists the work of the three phases; the caller copies both to the device.
+struct OzBatchLists {
+  const int4* products = nullptr;
+  const int4* splits = nullptr;
+  const int4* maxima = nullptr;
+  int n_products = 0, n_splits = 0, n_maxima = 0;
+};
+size_t oz_batch_instance_bytes();
+size_t oz_batch_plane_bytes(const ts_op* op, int S);
+void oz_batch_instance(const ts_op* op, const double2* Xh, double2* Yh, int S, void* planes, unsigned long long* mx,
+                       void* out);
+void oz_batch_items(const std::vector<const ts_op*>& ops, std::vector<int4>* products, std::vector<int4>* splits,
+                    std::vector<int4>* maxima);
+void oz_batch_products(const void* inst, const OzBatchLists& l, unsigned long long* mx, size_t mx_count, int S,
+                       const int* gate, int* err, cudaStream_t st);
 // Y = M(X) in FP64 through the emulated product (same contract as apply_f64), with S digits per
 // value; the operator's digit planes are prepared (once) with S_op >= S digits.
 void apply_f64_oz(ts_ctx* ctx, const ts_op* op, const double* X, double* Y, int mode, const double* C,

@@ -57,6 +57,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
   atomicCAS(err, 0, code);
   return false;
 }
+// For a warp that issues MMAs with all its lanes converged (see mma_issue_one): the wait of every lane, and a
+// result the compiler knows to be the same in all of them.  The part after the first look is out of line,
+// so that an unrolled issue loop has a few instructions per wait.
+static __device__ __noinline__ bool mbar_wait_call(uint32_t bar, uint32_t parity, int* err, int code) {
+  return mbar_wait(bar, parity, err, code);
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, int code) {
+  const bool ok = mbar_try(bar, parity) || mbar_wait_call(bar, parity, err, code);
+  return __all_sync(0xffffffffu, ok);
+}
+// A value that is the same in every lane, as one the compiler can keep in a uniform register.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+// True in one lane of the (converged) warp.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r;
+}
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2,
                                             uint32_t bar) {
@@ -91,6 +109,31 @@ __device__ __forceinline__ void mma_issue(uint32_t d_tmem, uint64_t a, uint64_t 
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
   }
+}
+
+// The MMA and the commit as a converged warp issues them: every lane passes here with the same operands, the
+// lane with `one` set (elect_one) executes.  The operands then stay in uniform registers, where the
+// instruction wants them; from inside an `if (lane == 0)` each one is moved there again for every MMA.
+__device__ __forceinline__ void mma_issue_one(uint32_t one, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                              uint32_t acc, int kind_tf32) {
+  if (kind_tf32) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(one));
+  } else {
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(one));
+  }
+}
+__device__ __forceinline__ void mma_commit_one(uint32_t one, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+      "r"(one)
+      : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -130,8 +173,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 }  // namespace tcg
 
 // 3-D TMA map over planes [planes][rows][ld] of esz-byte elements (BF16 for esz 2, FP32 for 4):
-// logical extent cols x rows x planes (elements beyond cols or rows read as zero), box = 128 bytes
-// of the contiguous index x box_rows x 1, 128-byte swizzle.
-void make_map(CUtensorMap* m, const void* base, int esz, int ld, int cols, int rows, int planes, int box_rows);
+// logical extent cols x rows x planes (elements beyond cols or rows read as zero), box = box_bytes (128 or
+// 64) of the contiguous index x box_rows x 1, swizzle of the same width.
+void make_map(CUtensorMap* m, const void* base, int esz, int ld, int cols, int rows, int planes, int box_rows,
+              int box_bytes = 128);
 
 }  // namespace ts
