@@ -56,6 +56,41 @@ struct TcCfg {
   static constexpr int kSubK = 128 / 32;                     // MMA K steps per stage (32 bytes each)
 };
 
+// The MMAs of one stage, issued by a converged warp (mma_issue_one): ax, the A_k X_k product, else -X_k B_k;
+// `first`, the tile's first stage.  One lane inside an `if` needs its operands moved to uniform registers
+// for every MMA, which paced the small products: n = 512, s = 128, p = 16 BF16 10.9 -> 8.9 us, split TF32
+// 40.7 -> 30.4; n = 1000, s = 300, p = 8 split TF32 87.3 -> 79.2; n = 4096, s = 256, p = 32 BF16 380 -> 368
+// (there the operand traffic from L2, 4.2 GB, is the next limit).
+template <int BN, int ESZ>
+__device__ __forceinline__ void tc_stage_mmas(uint32_t one, uint32_t stage, uint32_t d_re, uint32_t d_im, bool real,
+                                              bool ax, bool first, uint32_t idp, uint32_t idn) {
+  using Cfg = TcCfg<BN, ESZ>;
+  const uint32_t sA = warp_uniform(stage);
+  const uint64_t dAr = smem_desc_sw128(sA), dAi = smem_desc_sw128(sA + Cfg::kTileA);
+  const uint64_t dBr = smem_desc_sw128(sA + 2 * Cfg::kTileA);
+  const uint64_t dBi = smem_desc_sw128(sA + 2 * Cfg::kTileA + Cfg::kTileB);
+#pragma unroll
+  for (int kk = 0; kk < Cfg::kSubK; ++kk) {
+    const uint64_t o = (uint64_t)(kk * 2);   // 32 bytes >> 4
+    const uint32_t acc = (first && kk == 0) ? 0u : 1u;
+    if (ax) {
+      mma_issue_one(one, d_re, dAr + o, dBr + o, idp, acc, ESZ == 4);
+      if (!real) {
+        mma_issue_one(one, d_re, dAi + o, dBi + o, idn, 1u, ESZ == 4);
+        mma_issue_one(one, d_im, dAi + o, dBr + o, idp, acc, ESZ == 4);
+        mma_issue_one(one, d_im, dAr + o, dBi + o, idp, 1u, ESZ == 4);
+      }
+    } else {
+      mma_issue_one(one, d_re, dAr + o, dBr + o, idn, 1u, ESZ == 4);
+      if (!real) {
+        mma_issue_one(one, d_re, dAi + o, dBi + o, idp, 1u, ESZ == 4);
+        mma_issue_one(one, d_im, dAr + o, dBi + o, idn, 1u, ESZ == 4);
+        mma_issue_one(one, d_im, dAi + o, dBr + o, idn, 1u, ESZ == 4);
+      }
+    }
+  }
+}
+
 // PARTS = 1: one product per operand pair.  PARTS = 3 (split TF32): every l-block is visited three
 // times, hi*hi, hi*lo and lo*hi, accumulating in the same FP32 TMEM accumulators (FP32-level
 // accuracy on the TF32 tensor pipe).
@@ -139,50 +174,27 @@ __device__ __forceinline__ void tc_sylv_tile(const TcMaps& maps, float2* __restr
         mbar_wait(bar_full + 8 * (it % Cfg::kStages), (uint32_t)(it / Cfg::kStages) & 1u, err, 4, wait_ns);
     }
   } else if (warp == 5) {
-    if (lane == 0) {
-      constexpr int fmt = ESZ == 2 ? 1 : 2;
-      constexpr uint32_t idp = make_idesc(fmt, kTileM, BN, false);
-      constexpr uint32_t idn = make_idesc(fmt, kTileM, BN, true);
-      const uint32_t d_re = tmem, d_im = tmem + BN;
-      bool ok = true;
-      for (int it = 0; it < iters && ok; ++it) {
-        const int slot = it % Cfg::kStages;
-        const uint32_t phase = (uint32_t)(it / Cfg::kStages) & 1u;
-        if (!mbar_wait(bar_full + 8 * slot, phase, err, 2, wait_ns)) {
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sA = base + slot * Cfg::kStage;
-        const uint64_t dAr = smem_desc_sw128(sA), dAi = smem_desc_sw128(sA + Cfg::kTileA);
-        const uint64_t dBr = smem_desc_sw128(sA + 2 * Cfg::kTileA);
-        const uint64_t dBi = smem_desc_sw128(sA + 2 * Cfg::kTileA + Cfg::kTileB);
-#pragma unroll
-        for (int kk = 0; kk < Cfg::kSubK; ++kk) {
-          const uint64_t o = (uint64_t)(kk * 2);   // 32 bytes >> 4
-          const uint32_t first = (it == 0 && kk == 0) ? 0u : 1u;
-          if (it / PARTS < it1) {
-            mma_issue(d_re, dAr + o, dBr + o, idp, first, ESZ == 4);
-            if (!real) {
-              mma_issue(d_re, dAi + o, dBi + o, idn, 1u, ESZ == 4);
-              mma_issue(d_im, dAi + o, dBr + o, idp, first, ESZ == 4);
-              mma_issue(d_im, dAr + o, dBi + o, idp, 1u, ESZ == 4);
-            }
-          } else {
-            mma_issue(d_re, dAr + o, dBr + o, idn, 1u, ESZ == 4);
-            if (!real) {
-              mma_issue(d_re, dAi + o, dBi + o, idp, 1u, ESZ == 4);
-              mma_issue(d_im, dAr + o, dBi + o, idn, 1u, ESZ == 4);
-              mma_issue(d_im, dAi + o, dBr + o, idn, 1u, ESZ == 4);
-            }
-          }
-        }
-        mma_commit(bar_empty + 8 * slot);
+    // All lanes converged, one elected lane executes the MMAs (mma_issue_one).
+    constexpr int fmt = ESZ == 2 ? 1 : 2;
+    constexpr uint32_t idp = make_idesc(fmt, kTileM, BN, false);
+    constexpr uint32_t idn = make_idesc(fmt, kTileM, BN, true);
+    const uint32_t one = elect_one(), d_re = warp_uniform(tmem), d_im = d_re + BN;
+    bool ok = true;
+    for (int it = 0; it < iters && ok; ++it) {
+      const int slot = it % Cfg::kStages;
+      const uint32_t phase = (uint32_t)(it / Cfg::kStages) & 1u;
+      if (!mbar_wait_warp(bar_full + 8 * slot, phase, err, 2, wait_ns)) {
+        ok = false;
+        break;
       }
-      mma_commit(bar_acc);
-      // after an error the MMAs already issued still complete before TMEM is freed
-      if (!ok) mbar_wait(bar_acc, 0u, err, 5, wait_ns);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc_stage_mmas<BN, ESZ>(one, base + slot * Cfg::kStage, d_re, d_im, real, it / PARTS < it1, it == 0, idp, idn);
+      mma_commit_one(one, bar_empty + 8 * slot);
     }
+    mma_commit_one(one, bar_acc);
+    // after an error the MMAs already issued still complete before TMEM is freed
+    if (!ok) mbar_wait(bar_acc, 0u, err, 5, wait_ns);
+    __syncwarp();
   } else {
     // Epilogue: warp w reads TMEM lanes 32w..32w+31 (= output rows i0 + 32w + lane).
     const bool ok = mbar_wait(bar_acc, 0u, err, 3, wait_ns);
@@ -353,69 +365,46 @@ __global__ void __launch_bounds__(192, 1)
         mbar_wait(bar_full + 8 * (int)(u % Cfg::kStages), (uint32_t)(u / Cfg::kStages) & 1u, err, 4);
     }
   } else if (warp == 5) {
-    if (lane == 0) {
-      constexpr int fmt = ESZ == 2 ? 1 : 2;
-      constexpr uint32_t idp = make_idesc(fmt, kTileM, BN, false);
-      constexpr uint32_t idn = make_idesc(fmt, kTileM, BN, true);
-      long long g = 0;
-      int t = 0;   // items multiplied by this CTA
-      bool ok = true;
-      for (int q = blockIdx.x; q < nitems && ok; q += gridDim.x) {
-        const int4 it = items[q];
-        if (!active[it.x]) continue;
-        const BTcInst& b = inst[it.x];
-        const bool real = (it.y == 0) || (it.y == b.nyq);
-        const int it1 = (b.n + Cfg::kElemsK - 1) / Cfg::kElemsK, iters = iters_of(b);
-        const int set = t & 1;
-        // the epilogue has drained this accumulator set's previous item (t - 2)
-        if (t >= 2 && !mbar_wait(bar_acce + 8 * set, (uint32_t)((t >> 1) + 1) & 1u, err, 6)) {
+    constexpr int fmt = ESZ == 2 ? 1 : 2;
+    constexpr uint32_t idp = make_idesc(fmt, kTileM, BN, false);
+    constexpr uint32_t idn = make_idesc(fmt, kTileM, BN, true);
+    const uint32_t one = elect_one(), acc0 = warp_uniform(tmem);
+    long long g = 0;
+    int t = 0;   // items multiplied by this CTA
+    bool ok = true;
+    for (int q = blockIdx.x; q < nitems && ok; q += gridDim.x) {
+      const int4 it = items[q];
+      if (!active[it.x]) continue;
+      const BTcInst& b = inst[it.x];
+      const bool real = (it.y == 0) || (it.y == b.nyq);
+      const int it1 = (b.n + Cfg::kElemsK - 1) / Cfg::kElemsK, iters = iters_of(b);
+      const int set = t & 1;
+      // the epilogue has drained this accumulator set's previous item (t - 2)
+      if (t >= 2 && !mbar_wait_warp(bar_acce + 8 * set, (uint32_t)((t >> 1) + 1) & 1u, err, 6)) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d_re = acc0 + set * Cfg::kTmemCols, d_im = d_re + BN;
+      for (int u = 0; u < iters; ++u, ++g) {
+        const int slot = (int)(g % Cfg::kStages);
+        const uint32_t phase = (uint32_t)(g / Cfg::kStages) & 1u;
+        if (!mbar_wait_warp(bar_full + 8 * slot, phase, err, 2)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d_re = tmem + set * Cfg::kTmemCols, d_im = d_re + BN;
-        for (int u = 0; u < iters; ++u, ++g) {
-          const int slot = (int)(g % Cfg::kStages);
-          const uint32_t phase = (uint32_t)(g / Cfg::kStages) & 1u;
-          if (!mbar_wait(bar_full + 8 * slot, phase, err, 2)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sA = base + slot * Cfg::kStage;
-          const uint64_t dAr = smem_desc_sw128(sA), dAi = smem_desc_sw128(sA + Cfg::kTileA);
-          const uint64_t dBr = smem_desc_sw128(sA + 2 * Cfg::kTileA);
-          const uint64_t dBi = smem_desc_sw128(sA + 2 * Cfg::kTileA + Cfg::kTileB);
-#pragma unroll
-          for (int kk = 0; kk < Cfg::kSubK; ++kk) {
-            const uint64_t o = (uint64_t)(kk * 2);
-            const uint32_t first = (u == 0 && kk == 0) ? 0u : 1u;
-            if (u / PARTS < it1) {
-              mma_issue(d_re, dAr + o, dBr + o, idp, first, ESZ == 4);
-              if (!real) {
-                mma_issue(d_re, dAi + o, dBi + o, idn, 1u, ESZ == 4);
-                mma_issue(d_im, dAi + o, dBr + o, idp, first, ESZ == 4);
-                mma_issue(d_im, dAr + o, dBi + o, idp, 1u, ESZ == 4);
-              }
-            } else {
-              mma_issue(d_re, dAr + o, dBr + o, idn, 1u, ESZ == 4);
-              if (!real) {
-                mma_issue(d_re, dAi + o, dBi + o, idp, 1u, ESZ == 4);
-                mma_issue(d_im, dAr + o, dBi + o, idn, 1u, ESZ == 4);
-                mma_issue(d_im, dAi + o, dBr + o, idn, 1u, ESZ == 4);
-              }
-            }
-          }
-          mma_commit(bar_empty + 8 * slot);
-        }
-        if (!ok) break;
-        mma_commit(bar_accf + 8 * set);
-        ++t;
+        tc_stage_mmas<BN, ESZ>(one, base + slot * Cfg::kStage, d_re, d_im, real, u / PARTS < it1, u == 0, idp, idn);
+        mma_commit_one(one, bar_empty + 8 * slot);
       }
-      // every MMA issued (also on an error path) completes before tensor memory is freed
-      mma_commit(bar_done);
-      mbar_wait(bar_done, 0u, err, 5);
+      if (!ok) break;
+      mma_commit_one(one, bar_accf + 8 * set);
+      ++t;
     }
+    // every MMA issued (also on an error path) completes before tensor memory is freed
+    mma_commit_one(one, bar_done);
+    mbar_wait(bar_done, 0u, err, 5);
+    __syncwarp();
   } else {
     // Epilogue: warp w reads TMEM lanes 32w..32w+31 (= output rows i0 + 32w + lane) of set t & 1.
     int t = 0;

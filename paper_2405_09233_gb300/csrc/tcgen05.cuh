@@ -60,11 +60,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
 // For a warp that issues MMAs with all its lanes converged (see mma_issue_one): the wait of every lane, and a
 // result the compiler knows to be the same in all of them.  The part after the first look is out of line,
 // so that an unrolled issue loop has a few instructions per wait.
-static __device__ __noinline__ bool mbar_wait_call(uint32_t bar, uint32_t parity, int* err, int code) {
-  return mbar_wait(bar, parity, err, code);
+static __device__ __noinline__ bool mbar_wait_call(uint32_t bar, uint32_t parity, int* err, int code,
+                                                   unsigned long long limit_ns = kWaitNs) {
+  return mbar_wait(bar, parity, err, code, limit_ns);
 }
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, int code) {
-  const bool ok = mbar_try(bar, parity) || mbar_wait_call(bar, parity, err, code);
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err, int code,
+                                               unsigned long long limit_ns = kWaitNs) {
+  const bool ok = mbar_try(bar, parity) || mbar_wait_call(bar, parity, err, code, limit_ns);
   return __all_sync(0xffffffffu, ok);
 }
 // A value that is the same in every lane, as one the compiler can keep in a uniform register.
@@ -94,21 +96,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
   d |= (uint64_t)1 << 46;                   // descriptor version
   d |= (uint64_t)2 << 61;                   // 128-byte swizzle
   return d;
-}
-
-__device__ __forceinline__ void mma_issue(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc,
-                                          int kind_tf32) {
-  if (kind_tf32) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
-  } else {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
-  }
 }
 
 // The MMA and the commit as a converged warp issues them: every lane passes here with the same operands, the
