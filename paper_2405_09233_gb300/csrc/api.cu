@@ -389,9 +389,17 @@ void apply_f64(ts_ctx* ctx, const ts_op* op, const double* X, double* Y, int mod
     apply_f64_oz(ctx, op, X, Y, mode, C, partials, S, ctx->oz_digits, st);
     return;
   }
+  KernelTimer& tm = ctx->timer;
+  // One launch where that is the cheaper form; an application in place needs X whole until it is transformed.
+  const int tn = X + T * p <= Y || Y + T * p <= X ? apply_small_tile(n, s, p) : 0;
+  if (tn) {
+    tm.begin(st, 0, gemm_flops(n, s, n, s, K, nyquist_index(p)));
+    apply_small_f64(op, tn, X, Y, mode == IRFFT_RESIDUAL ? C : nullptr, partials, st, gate);
+    tm.end(st);
+    return;
+  }
   double2* Xh = static_cast<double2*>(ctx->ws.get("apply_Xh", sizeof(double2) * (size_t)K * T));
   double2* Yh = static_cast<double2*>(ctx->ws.get("apply_Yh", sizeof(double2) * (size_t)K * T));
-  KernelTimer& tm = ctx->timer;
   tm.begin(st, 1, 8.0 * T * p + 16.0 * K * T);
   rfft_tube<double, double2>(X, Xh, T, p, st, gate);
   tm.end(st);

@@ -40,9 +40,16 @@ struct EngineScope {
 
 // Y = M(X) in FP64 (rfft -> fused per-slice GEMMs -> irfft).  mode IRFFT_RESIDUAL writes
 // Y = C - M(X) and the kRedBlocks partial sums of Y^2 to `partials`.  gate (device, may be null; dense
-// operators on the DFMA engine only): when *gate == 0 the three kernels return at once.
+// operators on the DFMA engine only): when *gate == 0 its kernels return at once.
 void apply_f64(ts_ctx* ctx, const ts_op* op, const double* X, double* Y, int mode, const double* C,
                double* partials, cudaStream_t st, const int* gate = nullptr);
+
+// The same in one launch for small dense equations on the DFMA engine (apply_small.cu).  apply_small_tile:
+// the tile width to run it with, 0 where the three launches are the better form.  X and Y must not overlap;
+// C non-null: the residual form.
+int apply_small_tile(int n, int s, int p);
+void apply_small_f64(const ts_op* op, int tn, const double* X, double* Y, const double* C, double* partials,
+                     cudaStream_t st, const int* gate);
 
 // Yh = A_k Xh_k - Xh_k B_k slice by slice on spectral tensors (K slices of n x s, column-major), on the
 // context's FP64 engine: the operator of the spectral Krylov basis (no mode-3 DFTs).
