@@ -213,10 +213,6 @@ void cgemm_slices_f32(const CGemmArgs& a, cudaStream_t st);
 // ---------------- vector kernels (vec.cu) ----------------
 // All reductions write kRedBlocks partial sums; consumers finalise them in a fixed order.
 template <typename T> void dot_partials(const T* x, const T* y, long long N, double* partials, cudaStream_t st);
-// W -= h * Vi with h = finalize(Pin) (stored to *h_out by block 0); Pout = partials of <Vnext, W>
-// (or of <W, W> when Vnext == nullptr).
-template <typename T> void mgs_pass(T* W, const T* Vi, const T* Vnext, long long N, const double* Pin,
-                                    double* h_out, double* Pout, cudaStream_t st);
 // y = x * (*scale)
 template <typename T, typename U> void scale_dev(const T* x, U* y, long long N, const double* scale, cudaStream_t st);
 // X += sum_{i<k} y[i] * V[i*ldv ...]
@@ -234,23 +230,20 @@ void fill_zero(void* p, size_t bytes, cudaStream_t st);
 struct KrylovState;  // device-resident, see small.cu
 size_t krylov_state_bytes(int m);
 void ks_init(void* state, int m, const double* beta_and_inv, cudaStream_t st);
-// GMRES (method 0) / FOM (method 1) step j: consumes column j of H (rows 0..j written by MGS) and
-// ||W|| from Pnorm partials; writes the estimate and 1/h_{j+1,j} into the state.  Inside a
-// graph-captured cycle, `handle` is the conditional handle of step j + 1, which it sets to 0 when the
-// cycle stops after this step (breakdown, bad step, estimate <= stop[0] or <= stop[1]).
-void ks_step(void* state, int m, int j, int method, const double* Pnorm, cudaStream_t st,
-             cudaGraphConditionalHandle handle = 0, const double* stop = nullptr);
 // Solve for y over the first k columns; result in the state's y array.
-void ks_solve(void* state, int m, int k, int method, cudaStream_t st);
-// Inner step j after W = M(V_j), in one cluster launch for short vectors (arnoldi_small_ok(N)): the MGS sweep
-// against V_0..V_j (writing column j of H), h_{j+1,j} = ||W||, the ks_step update (same handle and
-// stop semantics) and V_{j+1} = W / h_{j+1,j} (always formed; W itself is left as M(V_j)).  The basis
-// vectors are V + i ldv.  gate (device, may be null): the kernel returns at once when *gate == 0,
-// and sets *gate = 0 where ks_step would end a graph-captured cycle (stop must then be given).
-bool arnoldi_small_ok(long long N);
+void ks_solve(void* state, int m, int k, cudaStream_t st);
+// Inner step j of tGMRES (method 0) or tFOM (method 1) after W = M(V_j): the Gram-Schmidt sweep against
+// V_0..V_j (writing column j of H), h_{j+1,j} = ||W||, the column's rotation or elimination with the residual
+// estimate, and V_{j+1} = W / h_{j+1,j} (always formed; W is used up).  The basis vectors are V + i ldv;
+// `scratch` holds arnoldi_scratch_bytes().  Inside a graph-captured cycle, `handle` is the conditional handle
+// of step j + 1, set to 0 when the cycle stops after this step (breakdown, bad step, estimate <= stop[0] or
+// <= stop[1]); gate (device, may be null): the kernels do nothing when *gate == 0, and *gate is set to 0
+// under the same conditions (stop must then be given).
+size_t arnoldi_scratch_bytes();
 template <typename T>
-void arnoldi_small(T* W, T* V, long long ldv, long long N, int j, int m, void* state, int method, cudaStream_t st,
-                   cudaGraphConditionalHandle handle = 0, const double* stop = nullptr, int* gate = nullptr);
+void arnoldi_step(T* W, T* V, long long ldv, long long N, int j, int m, void* state, int method, double* scratch,
+                  cudaStream_t st, cudaGraphConditionalHandle handle = 0, const double* stop = nullptr,
+                  int* gate = nullptr);
 // Device addresses inside the state block.
 double* ks_H(void* state, int m);          // column-major (m+1) x m, H[i + (m+1)*j]
 double* ks_y(void* state, int m);

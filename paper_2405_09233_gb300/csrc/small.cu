@@ -6,15 +6,28 @@
 // receives the j earlier rotations, a new rotation zeroes h_{j+1,j}, and the rotated right-hand
 // side g gives the residual norm |gamma_{j+1}| = |g_{j+1}| without forming y.
 // tFOM (§3.2): H_k y = beta e1 by Gaussian elimination with partial pivoting (a Hessenberg
-// matrix only needs a choice between rows c and c+1 at column c); the estimate is
-// h_{k+1,k} |y_k| (Proposition 3.3).
+// matrix only needs a choice between rows c and c+1 at column c), also one column at a time: the
+// eliminations of the columns before k - 1 do not depend on k, and the last column has none; the estimate
+// is h_{k+1,k} |y_k| (Proposition 3.3), y_k = (right-hand side)_k / (last pivot).
+//
+// The Gram-Schmidt sweep takes kGB basis vectors at a time.  Modified Gram-Schmidt's coefficients against
+// V_b .. V_b+7 solve (I + L) h = d, d_i = <V_i, W> and L the strictly lower part of the block's Gram matrix
+// <V_i, V_l>: h_i = <V_i, W - sum_{l<i} h_l V_l> written out.  So one reduction gives eight coefficients where
+// a sweep vector by vector waits for eight, each behind the other; the Gram row of V_j (at most 7 more inner
+// products) is formed once, in step j, whose last block it completes.  The result is modified Gram-Schmidt's
+// up to rounding: against FP64 MGS, orthogonality and residuals are the same (see the tests).
 #include <algorithm>
 #include "internal.cuh"
 #include "reduce.cuh"
+#include "pack.cuh"
 
 namespace ts {
 namespace {
 
+constexpr int kGB = 8;         // basis vectors per block of the sweep
+constexpr int kMaxM = 256;     // longest restart
+
+// tFOM keeps its eliminated columns in R, the multipliers and row choices in cs and sn, its right-hand side in g.
 struct Layout {
   int m;
   __host__ __device__ size_t H() const { return 0; }
@@ -25,8 +38,8 @@ struct Layout {
   __host__ __device__ size_t y() const { return g() + m + 1; }
   __host__ __device__ size_t est() const { return y() + m; }
   __host__ __device__ size_t beta() const { return est() + 8; }
-  __host__ __device__ size_t lu() const { return beta() + 8; }
-  __host__ __device__ size_t hist() const { return lu() + (size_t)m * m + m; }
+  __host__ __device__ size_t gram() const { return beta() + 8; }   // row i: <V_i, V_l>, l in i's block before i
+  __host__ __device__ size_t hist() const { return gram() + (size_t)(m + 1) * kGB; }
   __host__ __device__ size_t total() const { return hist() + m; }
 };
 
@@ -51,287 +64,666 @@ __global__ void k_ks_init(double* st, int m, const double* beta_in) {
 // est[0] = estimate, est[1] = 1/h_{j+1,j}, est[2] = h_{j+1,j}, est[3] = flags (1 breakdown,
 // 2 singular, 4 non-finite), est[4] = steps taken in this cycle (j + 1), est[8 + j] = estimate of
 // step j.  In a graph-captured cycle, `handle` is the conditional handle of step j + 1 (0 for the
-// last step) and the kernel decides whether the cycle goes on: it sets that handle to 0 on breakdown,
+// last step) and the update decides whether the cycle goes on: it sets that handle to 0 on breakdown,
 // a bad step, an estimate <= stop[0] (the tolerance times ||C||) or <= stop[1] (the inner tolerance
-// of mixed precision, or -1).
-// Columns of the Givens state staged in shared memory (tGMRES, m <= kStageMax): thread 0 then
-// rotates without a chain of dependent global loads (~0.7 us each; ~8 us at j = 10 before).
-constexpr int kStageMax = 256;
+// of mixed precision, or -1).  `gate` is closed under the same conditions (launched-ahead cycles).
+struct StepEnd {
+  cudaGraphConditionalHandle handle;
+  const double* stop;
+  int* gate;
+};
 
-// Step j's update given h_{j+1,j} = hn; called by every thread of the block (one block).
-__device__ void ks_update(double* st, int m, int j, int method, double hn, cudaGraphConditionalHandle handle,
-                          const double* stop, int* gate = nullptr) {
-  __shared__ double s_col[kStageMax + 2], s_cs[kStageMax], s_sn[kStageMax];
+// The column update of step j.  One thread runs it; what it reads is staged in shared memory by all threads
+// first (ks_load), so that it does not wait on a chain of dependent global loads.
+struct KsStage {
+  double cs[kMaxM], sn[kMaxM];
+  double g, diag, sub, beta, stop0, stop1;
+};
+
+__device__ __forceinline__ void ks_load(KsStage& S, const double* st, int m, int j, int method, const StepEnd& end,
+                                        int t, int nt) {
   Layout L{m};
-  double* H = st + L.H();
   const int ld = m + 1;
-  const bool staged = method == 0 && m <= kStageMax;
-  if (staged) {
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) s_col[i] = H[i + ld * j];
-    for (int i = threadIdx.x; i < j; i += blockDim.x) {
-      s_cs[i] = st[L.cs() + i];
-      s_sn[i] = st[L.sn() + i];
-    }
-    __syncthreads();
+  for (int i = t; i < j; i += nt) {
+    S.cs[i] = st[L.cs() + i];
+    S.sn[i] = st[L.sn() + i];
   }
-  if (threadIdx.x != 0) return;
-  H[(j + 1) + ld * j] = hn;
-  const double beta = st[L.beta()];
-  double flags = (hn <= kBreakdownRel * beta) ? 1.0 : 0.0;
+  if (t == nt - 1) S.beta = st[L.beta()];
+  if (t == nt - 2 && end.stop) {
+    S.stop0 = end.stop[0];
+    S.stop1 = end.stop[1];
+  }
+  if (t == nt - 3) S.g = method != 0 && j > 0 ? st[L.g() + j - 1] : st[L.g() + j];
+  if (t == nt - 4 && method != 0 && j > 0) {
+    S.diag = st[L.R() + (j - 1) + (size_t)ld * (j - 1)];
+    S.sub = st[L.H() + j + (size_t)ld * (j - 1)];
+  }
+}
+
+// tFOM: the elimination of column j - 1, which step j's row makes possible.
+__device__ __forceinline__ void ks_pivot(KsStage& S, double* st, int m, int j, int method) {
+  if (method == 0 || j == 0) return;
+  Layout L{m};
+  const double t = S.diag, b = S.sub, rhs = S.g;
+  const bool swap = fabs(b) > fabs(t);
+  const double piv = swap ? b : t, f = piv != 0.0 ? (swap ? t : b) / piv : 0.0;
+  S.cs[j - 1] = f;
+  S.sn[j - 1] = swap ? 1.0 : 0.0;
+  st[L.cs() + j - 1] = f;
+  st[L.sn() + j - 1] = swap ? 1.0 : 0.0;
+  st[L.R() + (j - 1) + (size_t)(m + 1) * (j - 1)] = piv;
+  st[L.g() + j - 1] = swap ? 0.0 : rhs;
+  S.g = swap ? rhs : 0.0 - f * rhs;
+}
+
+// The earlier rotations (tGMRES) or eliminations (tFOM) on entries c0 .. c1 - 1 of column j; t is the entry
+// carried from row to row.
+__device__ __forceinline__ void ks_rotate(const KsStage& S, double* st, int m, int j, int method, int c0, int c1,
+                                          const double* h, double& t) {
+  double* R = st + Layout{m}.R() + (size_t)(m + 1) * j;
+  for (int i = c0; i < c1; ++i) {
+    const double b = h[i - c0];
+    if (i == 0) {
+      t = b;
+      continue;
+    }
+    const double c = S.cs[i - 1], s = S.sn[i - 1];
+    if (method == 0) {
+      R[i - 1] = c * t + s * b;
+      t = c * b - s * t;
+    } else {
+      const double top = s != 0.0 ? b : t, bot = s != 0.0 ? t : b;
+      R[i - 1] = top;
+      t = bot - c * top;
+    }
+  }
+}
+
+// sqrt(x) and its reciprocal.  rsqrt and one correction where x is in the middle of the range: half the
+// FP64 instructions of sqrt and a division.
+__device__ __forceinline__ void root(double x, double& r, double& inv) {
+  if (x > 1e-280 && x < 1e280) {
+    inv = rsqrt(x);
+    r = x * inv;
+    r = fma(0.5 * inv, fma(-r, r, x), r);
+  } else {
+    r = sqrt(x);
+    inv = r > 0.0 ? 1.0 / r : 0.0;
+  }
+}
+
+__device__ __forceinline__ void ks_finish(const KsStage& S, double* st, int m, int j, int method, double t, double hn,
+                                          double inv, const StepEnd& end) {
+  Layout L{m};
+  const int ld = m + 1;
+  double* R = st + L.R() + (size_t)ld * j;
+  st[L.H() + (j + 1) + (size_t)ld * j] = hn;
+  double flags = (hn <= kBreakdownRel * S.beta) ? 1.0 : 0.0;
   double est;
   if (method == 0) {
-    double* R = st + L.R();
-    double* cs = st + L.cs();
-    double* sn = st + L.sn();
-    double* g = st + L.g();
-    double* col = staged ? s_col : R + ld * j;
-    const double* c_cs = staged ? s_cs : cs;
-    const double* c_sn = staged ? s_sn : sn;
-    if (!staged)
-      for (int i = 0; i <= j; ++i) col[i] = H[i + ld * j];
-    col[j + 1] = hn;
-    for (int i = 0; i < j; ++i) {
-      const double a = col[i], b = col[i + 1];
-      col[i] = c_cs[i] * a + c_sn[i] * b;
-      col[i + 1] = -c_sn[i] * a + c_cs[i] * b;
-    }
-    const double a = col[j], b = col[j + 1];
-    const double r = hypot(a, b);
-    double c = 1.0, s = 0.0;
-    if (r > 0.0) {
-      c = a / r;
-      s = b / r;
-    }
-    cs[j] = c;
-    sn[j] = s;
-    col[j] = r;
-    col[j + 1] = 0.0;
-    if (staged)
-      for (int i = 0; i <= j + 1; ++i) R[i + ld * j] = col[i];
-    const double gj = g[j];
-    g[j + 1] = -s * gj;
-    g[j] = c * gj;
-    est = fabs(g[j + 1]);
-  } else {
-    // Gaussian elimination with partial pivoting on H_k (k = j+1), right-hand side beta e1.
-    const int k = j + 1;
-    double* M = st + L.lu();   // k x k, column-major, followed by the right-hand side
-    double* rhs = M + (size_t)m * m;
-    for (int c = 0; c < k; ++c)
-      for (int r = 0; r < k; ++r) M[r + k * c] = (r <= c + 1) ? H[r + ld * c] : 0.0;
-    for (int r = 0; r < k; ++r) rhs[r] = (r == 0) ? beta : 0.0;
-    bool singular = false;
-    for (int c = 0; c < k; ++c) {
-      if (c + 1 < k && fabs(M[c + 1 + k * c]) > fabs(M[c + k * c])) {
-        for (int q = c; q < k; ++q) {
-          const double t = M[c + k * q];
-          M[c + k * q] = M[c + 1 + k * q];
-          M[c + 1 + k * q] = t;
-        }
-        const double t = rhs[c];
-        rhs[c] = rhs[c + 1];
-        rhs[c + 1] = t;
-      }
-      const double piv = M[c + k * c];
-      if (piv == 0.0) {
-        singular = true;
-        break;
-      }
-      if (c + 1 < k) {
-        const double f = M[c + 1 + k * c] / piv;
-        for (int q = c; q < k; ++q) M[c + 1 + k * q] -= f * M[c + k * q];
-        rhs[c + 1] -= f * rhs[c];
-      }
-    }
-    double* y = st + L.y();
-    if (!singular) {
-      for (int r = k - 1; r >= 0; --r) {
-        double v = rhs[r];
-        for (int q = r + 1; q < k; ++q) v -= M[r + k * q] * y[q];
-        y[r] = v / M[r + k * r];
-      }
-      est = hn * fabs(y[k - 1]);
+    double r, ri, c = 1.0, s = 0.0;
+    const double q = fma(t, t, hn * hn);
+    if (q > 1e-280 && q < 1e280) {
+      root(q, r, ri);
+      c = t * ri;
+      s = hn * ri;
     } else {
+      r = hypot(t, hn);
+      if (r > 0.0) {
+        c = t / r;
+        s = hn / r;
+      }
+    }
+    st[L.cs() + j] = c;
+    st[L.sn() + j] = s;
+    R[j] = r;
+    R[j + 1] = 0.0;
+    const double gn = -s * S.g;
+    st[L.g() + j] = c * S.g;
+    st[L.g() + j + 1] = gn;
+    est = fabs(gn);
+  } else {
+    R[j] = t;
+    st[L.g() + j] = S.g;
+    if (t == 0.0) {
       flags += 2.0;
       est = INFINITY;
+    } else {
+      est = hn * fabs(S.g / t);
     }
   }
   if (!isfinite(est) || !isfinite(hn)) flags += 4.0;
   st[L.est()] = est;
-  st[L.est() + 1] = hn > 0.0 ? 1.0 / hn : 0.0;
+  st[L.est() + 1] = inv;
   st[L.est() + 2] = hn;
   st[L.est() + 3] = flags;
   st[L.est() + 4] = j + 1;
   st[L.hist() + j] = est;
-  if (handle || gate) {
-    const bool go = flags == 0.0 && !(est <= stop[0]) && !(est <= stop[1]);
+  if (end.handle || end.gate) {
+    const bool go = flags == 0.0 && !(est <= S.stop0) && !(est <= S.stop1);
     if (!go) {
-      if (handle) cudaGraphSetConditional(handle, 0);
-      if (gate) *gate = 0;
+      if (end.handle) cudaGraphSetConditional(end.handle, 0);
+      if (end.gate) *end.gate = 0;
     }
   }
 }
 
-__global__ void k_ks_step(double* st, int m, int j, int method, const double* Pnorm,
-                          cudaGraphConditionalHandle handle, const double* stop) {
-  const double hn = sqrt(finalize_partials(Pnorm));
-  ks_update(st, m, j, method, hn, handle, stop);
+// One warp: lane r < nb holds d_r on entry and h_r on return; row is the lane's Gram row (l < its own r).
+__device__ __forceinline__ double gs_forward(double d, const double (&row)[kGB - 1], int nb, int lane) {
+#pragma unroll
+  for (int l = 0; l < kGB - 1; ++l) {
+    const double hl = __shfl_sync(0xffffffffu, d, l);
+    if (l + 1 < nb && lane > l && lane < nb) d = fma(-row[l], hl, d);
+  }
+  return d;
 }
 
-// Everything of inner step j after W = M(V_j), for vectors of at most kArnMaxN entries, in one
-// launch of a thread-block cluster of CL <= kArnCL CTAs: the modified Gram-Schmidt sweep
-// h_ij = <V_i, W>, W -= h_ij V_i (i = 0..j, in order), the norm h_{j+1,j} = ||W||, the Givens /
-// Hessenberg update (ks_update, by CTA 0) and V_{j+1} = W / h_{j+1,j}.  CTA c owns a contiguous part
-// of the vectors, kept in registers (W) or loaded one pass ahead (the next V_i).  An inner product
-// is summed per warp (butterfly), every warp's partial is stored into every CTA's shared memory
-// (distributed shared memory), and after one cluster barrier each warp adds all partials in the same
-// fixed order, so every thread of every CTA holds the same value, bit for bit.  GB300's FP64 pipe
-// issues one warp's DFMA in 64 clocks per SM sub-partition, so one CTA spent ~2.3 us per MGS pass at
-// 2304 entries in FP64 issue alone; eight SMs cut that eightfold, and the pass is left with two short
-// reduction trees and the barrier.  Same arithmetic as the multi-block kernels (FP64 sums; an FP32
-// basis sums each thread's products in FP32 first), in a different summation order.  All CTAs pass
-// the same barriers (j is a kernel argument; the gate is read once, before the first barrier, and
-// written by CTA 0 only after the last), the first barrier precedes every remote store and no remote
-// store follows the last one.
+// Everything of inner step j after W = M(V_j), for vectors of at most kArnMaxN entries, in one launch of a
+// thread-block cluster of CL <= kArnCL CTAs: the sweep, h_{j+1,j} = ||W||, the column update (by one thread
+// of CTA 0, a warp that does nothing else, beside the sweep) and V_{j+1} = W / h_{j+1,j}.  CTA c owns a
+// contiguous part of the vectors in shared memory, W for the whole step and the basis one block ahead
+// (cp.async).  Warp q forms the inner products with the block's vector q, stores the sum into every CTA's
+// shared memory, and after one cluster barrier each CTA adds all parts in the same fixed order, so every CTA
+// holds the same coefficients, bit for bit.  All CTAs pass the same barriers (j is a kernel argument; the gate
+// is read once, before the first barrier, and written by CTA 0 only after the last), the first barrier
+// precedes every remote store and no remote store follows the last one.
+//
+// Bound by FP64 issue (64 clocks per warp instruction and sub-partition) and by the reduction's round trip.
+// The 20 steps of a cycle, vector by vector -> by blocks: 2304 FP64 entries 517 -> 260 us, 8000 FP64 931 ->
+// 448, 8000 FP32 861 -> 294.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-constexpr int kArnCL = 8, kArnMaxThreads = 512, kArnMaxN = kArnCL * kArnMaxThreads * 16;
+constexpr int kArnCL = 8, kArnWarps = 8, kArnThreads = 32 * (kArnWarps + 1), kArnMaxN = kArnCL * 1024;
 
 __device__ __forceinline__ void cluster_sync_all() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
-template <typename T, int R>
-__global__ void __launch_bounds__(kArnMaxThreads, 1)
-    k_arnoldi_cluster(T* __restrict__ W, T* __restrict__ V, long long ldv, int N, int j, int m, double* st,
-                      int method, cudaGraphConditionalHandle handle, const double* stop, int* gate) {
-  if (gate && *gate == 0) return;   // launched ahead of a cycle that has already ended (all CTAs alike)
-  __shared__ double slots[2][kArnCL * (kArnMaxThreads / 32)];
+template <typename T>
+__device__ __forceinline__ void cp_async_one(T* dst, const T* src) {
+  if constexpr (sizeof(T) == 8)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kArnThreads, 1)
+    k_arnoldi_cluster(const T* __restrict__ W, T* __restrict__ V, long long ldv, int N, int j, int m, double* st,
+                      int method, StepEnd end) {
+  if (end.gate && *end.gate == 0) return;   // launched ahead of a cycle that has already ended (all CTAs alike)
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double slots[2][kArnCL * 2 * kGB];
+  __shared__ double sh[kGB], sG[kGB * kGB], snorm[2];
+  __shared__ KsStage S;
   uint32_t rank, ncta;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(ncta));
-  const int nt = blockDim.x, nw = nt / 32, t = threadIdx.x, lane = t & 31, wp = t >> 5;
+  const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
   const int Nc = (N + (int)ncta - 1) / (int)ncta, e0 = (int)rank * Nc;
-  auto idx = [&](int r) {   // element of (thread, r), or -1
-    const int q = t + nt * r, e = e0 + q;
-    return (q < Nc && e < N) ? e : -1;
-  };
+  const int cnt = max(0, min(Nc, N - e0));
+  T* w = reinterpret_cast<T*>(smem_raw);
+  T* stage = w + Nc;                        // two blocks of kGB parts
   Layout L{m};
-  double* H = st + L.H();
-  const int ld = m + 1;
-  T w[R], v[R], vn[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int e = idx(r);
-    w[r] = e >= 0 ? W[e] : T(0);
-    v[r] = e >= 0 ? V[e] : T(0);
-  }
-  auto dot = [&](const T (&x)[R]) {
-    if constexpr (sizeof(T) == 4) {
-      float f = 0.f;
-#pragma unroll
-      for (int r = 0; r < R; ++r) f = fmaf(x[r], w[r], f);
-      return (double)f;
-    } else {
-      double acc = 0.0;
-#pragma unroll
-      for (int r = 0; r < R; ++r) acc += x[r] * w[r];
-      return acc;
+  double *H = st + L.H() + (size_t)(m + 1) * j, *G = st + L.gram();
+  const int nblk = j / kGB + 1;
+  auto in_block = [&](int b) { return min(kGB, j + 1 - kGB * b); };
+  auto fetch = [&](int b) {                 // block b's parts, by the sweep's warps
+    if (wp < in_block(b) && wp < kArnWarps) {
+      T* d = stage + (size_t)((b & 1) * kGB + wp) * Nc;
+      const T* v = V + (long long)(kGB * b + wp) * ldv + e0;
+      for (int q = lane; q < cnt; q += 32) cp_async_one(d + q, v + q);
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  double gnext = 0.0;
+  auto fetch_gram = [&](int b) {            // a row of V_j itself is not there yet (and not used)
+    if (t < kGB * kGB && t / kGB < in_block(b) && kGB * b + t / kGB < j) gnext = G[(size_t)(kGB * b) * kGB + t];
+  };
+  for (int q = t; q < cnt; q += kArnThreads) cp_async_one(w + q, W + e0 + q);
+  fetch(0);
+  fetch_gram(0);
+  if (rank == 0) ks_load(S, st, m, j, method, end, t, kArnThreads);
+  cluster_sync_all();   // every CTA of the cluster runs before any remote store
+  const bool ks = rank == 0 && t == 32 * kArnWarps;
+  if (ks) ks_pivot(S, st, m, j, method);
+  double carry = 0.0, nrm = 0.0;
   int buf = 0;
-  auto cluster_sum = [&](double x) {
+  auto store_all = [&](double x, int at, int c) {   // x into slot `at` of CTA c
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_addr(&slots[buf][at])), "r"(c));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(x) : "memory");
+  };
+  for (int b = 0; b < nblk; ++b) {
+    const int nb = in_block(b);
+    const bool last = b + 1 == nblk;
+    if (t < kGB * kGB) sG[t] = gnext;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (!last) {
+      fetch(b + 1);
+      fetch_gram(b + 1);
+    }
+    const T* blk = stage + (size_t)(b & 1) * kGB * Nc;
+    if (wp < nb && wp < kArnWarps) {
+      const T *v = blk + (size_t)wp * Nc, *vj = blk + (size_t)(nb - 1) * Nc;
+      const bool gram = last && wp < nb - 1;
+      double x = 0.0, y = 0.0;
+      if constexpr (sizeof(T) == 8) {
+        for (int q = lane; q < cnt; q += 32) {
+          x = fma(v[q], w[q], x);
+          if (gram) y = fma(v[q], vj[q], y);
+        }
+      } else {
+        for (int q0 = lane; q0 < cnt; q0 += 256) {   // eight products per FP64 addition (pack.cuh)
+          float f = 0.f, g = 0.f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) {
-      const uint32_t local = smem_addr(&slots[buf][(int)rank * nw + wp]);
-      for (uint32_t c = 0; c < ncta; ++c) {
-        uint32_t remote;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(c));
-        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(x) : "memory");
+          for (int u = 0; u < 8; ++u) {
+            const int q = q0 + 32 * u;
+            if (q < cnt) {
+              f = fmaf(v[q], w[q], f);
+              if (gram) g = fmaf(v[q], vj[q], g);
+            }
+          }
+          x += (double)f;
+          if (gram) y += (double)g;
+        }
       }
+      // lanes 0-15 end with the sum of x, lanes 16-31 with that of y
+      const double o = __shfl_xor_sync(0xffffffffu, lane < 16 ? y : x, 16);
+      x = (lane < 16 ? x : y) + o;
+#pragma unroll
+      for (int d = 8; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+      const int c = lane & 15;
+      if (c < (int)ncta && (lane < 16 || gram)) store_all(x, (int)rank * 2 * kGB + (lane >> 4) * kGB + wp, c);
     }
     cluster_sync_all();
-    double y = 0.0;
-    for (int q = lane; q < (int)ncta * nw; q += 32) y += slots[buf][q];
+    if (wp == 0) {
+      const int q = lane & 15;
+      const bool used = q < kGB ? q < nb : (last && q - kGB < nb - 1);
+      double x = 0.0;
+      if (used)
+        for (int c = lane >> 4; c < (int)ncta; c += 2) x += slots[buf][c * 2 * kGB + q];
+      x += __shfl_xor_sync(0xffffffffu, x, 16);
+      double row[kGB - 1];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-    buf ^= 1;
-    return y;
-  };
-  cluster_sync_all();   // every CTA of the cluster runs before any remote store
-  for (int i = 0; i <= j; ++i) {
-    const double part = dot(v);
-    if (i < j) {
-      const T* Vn = V + (long long)(i + 1) * ldv;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int e = idx(r);
-        vn[r] = e >= 0 ? Vn[e] : T(0);
+      for (int l = 0; l < kGB - 1; ++l) {
+        const double gj = __shfl_sync(0xffffffffu, x, kGB + l);
+        row[l] = last && lane == nb - 1 ? gj : sG[(lane & 7) * kGB + l];
+      }
+      if (last && rank == 0 && lane >= kGB && lane < kGB + nb - 1) G[(size_t)j * kGB + lane - kGB] = x;
+      x = gs_forward(x, row, nb, lane);
+      if (lane < nb) {
+        sh[lane] = x;
+        if (rank == 0) H[kGB * b + lane] = x;
       }
     }
-    const double h = cluster_sum(part);
-    if (rank == 0 && t == 0) H[i + ld * j] = h;
-    const T hT = (T)h;
+    __syncthreads();
+    if (wp < kArnWarps) {
+      T h[kGB];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      w[r] = w[r] - hT * v[r];
-      v[r] = vn[r];
+      for (int q = 0; q < kGB; ++q) h[q] = q < nb ? (T)sh[q] : T(0);
+      float f = 0.f;
+      for (int e = t, u = 0; e < cnt; e += 32 * kArnWarps, ++u) {
+        T x = w[e];
+#pragma unroll
+        for (int q = 0; q < kGB; ++q)
+          if (q < nb) x = x - h[q] * blk[(size_t)q * Nc + e];
+        w[e] = x;
+        if (last) {
+          if constexpr (sizeof(T) == 8) {
+            nrm = fma(x, x, nrm);
+          } else {
+            f = fmaf(x, x, f);
+            if ((u & 7) == 7) {
+              nrm += (double)f;
+              f = 0.f;
+            }
+          }
+        }
+      }
+      if (sizeof(T) == 4 && last) nrm += (double)f;
+    } else if (ks) {
+      ks_rotate(S, st, m, j, method, kGB * b, kGB * b + nb, sh, carry);
+    }
+    buf ^= 1;
+  }
+  if (wp < kArnWarps) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, d);
+    if (lane < (int)ncta) store_all(nrm, (int)rank * 2 * kGB + wp, lane);
+  }
+  cluster_sync_all();
+  if (wp == 0) {
+    double x = 0.0;
+    for (int q = lane; q < (int)ncta * kArnWarps; q += 32) x += slots[buf][(q / kArnWarps) * 2 * kGB + q % kArnWarps];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+    double hn, inv;
+    root(x, hn, inv);
+    if (lane == 0) {
+      snorm[0] = hn;
+      snorm[1] = inv;
     }
   }
-  const double hn = sqrt(cluster_sum(dot(w)));
-  if (rank == 0) ks_update(st, m, j, method, hn, handle, stop, gate);
-  const double inv = hn > 0.0 ? 1.0 / hn : 0.0;
-  T* Vj1 = V + (long long)(j + 1) * ldv;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int e = idx(r);
-    if (e >= 0) {
-      if constexpr (sizeof(T) == 4) Vj1[e] = w[r] * (float)inv;
-      else Vj1[e] = w[r] * inv;
-    }
+  __syncthreads();
+  if (wp < kArnWarps) {
+    const T inv = (T)snorm[1];
+    T* Vn = V + (long long)(j + 1) * ldv + e0;
+    for (int e = t; e < cnt; e += 32 * kArnWarps) Vn[e] = w[e] * inv;
+  } else if (ks) {
+    ks_finish(S, st, m, j, method, carry, snorm[0], snorm[1], end);
   }
 }
 
-// tGMRES: back substitution R_k y = g_k.  tFOM: y is already the solution of the last step.
-// R_k and g_k are staged in shared memory first (k <= kSolveStage) so that one thread's substitution
-// does not wait on a global load per term (~29 us at k = 18 before).
-constexpr int kSolveStage = 64;
-__global__ void k_ks_solve(double* st, int m, int k, int method) {
-  if (method != 0) return;
-  __shared__ double sR[kSolveStage * kSolveStage], sg[kSolveStage], sy[kSolveStage];
-  Layout L{m};
-  const int ld = m + 1;
-  const double* R = st + L.R();
-  const double* g = st + L.g();
-  double* y = st + L.y();
-  const bool staged = k <= kSolveStage;
-  if (staged) {
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-      const int r = e % k, q = e / k;
-      sR[r + kSolveStage * q] = R[r + ld * q];
+// Longer vectors: the same step as a chain of launches over the whole chip, one per block of the sweep and
+// two more.  Pass b = -1 forms the first block's inner products; pass b subtracts block b and forms those of
+// block b + 1, or ||W||^2 after the last.  A CTA writes its sums to P[sum][CTA]; the next launch adds them
+// up in every CTA (in the same order, so all have the same coefficients).
+// Bound by memory from about a million entries on (FP32: 16.8M entries, 20 steps move 37.6 GB in 6.4 ms), by
+// round trips below.  The sweeps of a 20-step cycle, against a launch per basis vector (reading W, V_i and
+// V_i+1, writing W) above 65536 entries and one cluster launch per step below: FP64, 61440 entries 1877 ->
+// 542 us, 262144 1534 -> 745, 4.2M 8474 -> 5556; FP32, 1.05M 1944 -> 888, 16.8M 10303 -> 6427.  The line to
+// the cluster form lies where both take the same time (FP64, 8000 entries in the cluster 457 us, 8200 here 451).
+constexpr int kGsBlocks = 152, kGsSums = 2 * kGB;
+
+// v[0..NV-1] summed over the warp: lane's result is sum lane / (32 / NV); NV 4, 8 or 16.
+template <int NV>
+__device__ __forceinline__ double warp_reduce_scatter(double (&v)[NV], int lane) {
+  constexpr int LG = NV == 16 ? 4 : (NV == 8 ? 3 : 2);
+#pragma unroll
+  for (int r = 0; r < LG; ++r) {
+    const bool up = (lane & (16 >> r)) != 0;
+#pragma unroll
+    for (int i = 0; i < NV / 2; ++i) {
+      if (i < (NV >> (r + 1))) {
+        const int o = NV >> (r + 1);
+        const double send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16 >> r);
+      }
     }
-    for (int r = threadIdx.x; r < k; r += blockDim.x) sg[r] = g[r];
-    __syncthreads();
   }
-  if (threadIdx.x != 0) return;
-  if (staged) {
-    for (int r = k - 1; r >= 0; --r) {
-      double v = sg[r];
-      for (int q = r + 1; q < k; ++q) v -= sR[r + kSolveStage * q] * sy[q];
-      sy[r] = v / sR[r + kSolveStage * r];
+  double x = v[0];
+#pragma unroll
+  for (int mask = 16 >> LG; mask > 0; mask >>= 1) x += __shfl_xor_sync(0xffffffffu, x, mask);
+  return x;
+}
+
+// One pack of a vector: four FP32 or two FP64 entries (one 16-byte access), or one entry.
+template <typename T, int PK>
+__device__ __forceinline__ void ld_pack(const T* p, long long e, T (&v)[PK]) {
+  if constexpr (PK == 1) v[0] = p[e];
+  else if constexpr (sizeof(T) == 4) {
+    const float4 q = reinterpret_cast<const float4*>(p)[e];
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else {
+    const double2 q = reinterpret_cast<const double2*>(p)[e];
+    v[0] = q.x; v[1] = q.y;
+  }
+}
+template <typename T, int PK>
+__device__ __forceinline__ void st_pack(T* p, long long e, const T (&v)[PK]) {
+  if constexpr (PK == 1) p[e] = v[0];
+  else if constexpr (sizeof(T) == 4) reinterpret_cast<float4*>(p)[e] = make_float4(v[0], v[1], v[2], v[3]);
+  else reinterpret_cast<double2*>(p)[e] = make_double2(v[0], v[1]);
+}
+
+// VB: the most vectors of a block, 4 (the first steps; twice the packs in flight) or 8.
+template <typename T, int PK, int VB>
+__global__ void __launch_bounds__(512, 1)
+    k_gs_pass(T* __restrict__ W, const T* __restrict__ V, long long ldv, long long NP, int j, int b,
+              const double* __restrict__ Pin, double* __restrict__ Pout, double* st, int m, const int* gate) {
+  if (gate && *gate == 0) return;
+  __shared__ double sd[kGsSums], sh[kGB], red[16][kGsSums];
+  const int t = threadIdx.x, lane = t & 31, wp = t >> 5, nw = blockDim.x >> 5;
+  const int nblk = j / kGB + 1;
+  const int nu = b >= 0 ? min(kGB, j + 1 - kGB * b) : 0;              // vectors subtracted
+  const int nd = b + 1 < nblk ? min(kGB, j + 1 - kGB * (b + 1)) : 0;  // vectors multiplied
+  const bool lastu = b + 1 == nblk, lastd = b + 2 == nblk;
+  T h[VB];
+  if (nu) {
+    Layout L{m};
+    double* G = st + L.gram() + (size_t)(kGB * b) * kGB;
+    double row[kGB - 1];
+    if (wp == 0) {
+#pragma unroll
+      for (int l = 0; l < kGB - 1; ++l)   // rows of earlier steps; V_j's is among the sums
+        row[l] = lane < nu && l < lane && kGB * b + lane < j ? G[lane * kGB + l] : 0.0;
     }
-    for (int r = 0; r < k; ++r) y[r] = sy[r];
+    for (int q = wp; q < kGsSums; q += nw) {
+      if (!(q < kGB ? q < nu : (lastu && q - kGB < nu - 1))) continue;
+      double x = 0.0;
+      for (int c = lane; c < (int)gridDim.x; c += 32) x += Pin[q * kGsBlocks + c];
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+      if (lane == 0) sd[q] = x;
+    }
+    __syncthreads();
+    if (wp == 0) {
+      double x = lane < nu ? sd[lane] : 0.0;
+      if (lastu && lane == nu - 1) {
+#pragma unroll
+        for (int l = 0; l < kGB - 1; ++l) row[l] = l < lane ? sd[kGB + l] : 0.0;
+        if (blockIdx.x == 0) {
+#pragma unroll
+          for (int l = 0; l < kGB - 1; ++l)
+            if (l < lane) G[lane * kGB + l] = row[l];
+        }
+      }
+      x = gs_forward(x, row, nu, lane);
+      if (lane < nu) {
+        sh[lane] = x;
+        if (blockIdx.x == 0) st[L.H() + kGB * b + lane + (size_t)(m + 1) * j] = x;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < VB; ++q) h[q] = q < nu ? (T)sh[q] : T(0);
+  }
+  const T *Vu = V + (long long)(kGB * max(b, 0)) * ldv, *Vd = V + (long long)(kGB * (b + 1)) * ldv;
+  // FP32 vectors: two packs (eight products) are summed in FP32 (pack.cuh), and such sums in pairs of FP32
+  // numbers with the rounding error of every addition kept (Knuth's two-sum), as exact as an FP64 sum here; a
+  // conversion and an FP64 addition per eight products took half of this kernel's time.
+  constexpr int UN = sizeof(T) == 4 ? 2 : 1, GR = VB == 4 ? 2 * UN : 1, NI = VB == 4 ? GR : UN;
+  double acc[2 * VB];
+  float hi[2 * VB], lo[2 * VB], f[2 * VB];
+#pragma unroll
+  for (int q = 0; q < 2 * VB; ++q) {
+    acc[q] = 0.0;
+    hi[q] = lo[q] = f[q] = 0.f;
+  }
+  const auto used = [&](int q) { return q < VB ? q < nd : (lastd && q - VB < nd - 1); };
+  const auto add_dot = [&](const T (&x)[PK], const T (&y)[PK], int q) {
+#pragma unroll
+    for (int c = 0; c < PK; ++c) {
+      if constexpr (sizeof(T) == 8) acc[q] = fma(x[c], y[c], acc[q]);
+      else f[q] = fmaf(x[c], y[c], f[q]);
+    }
+  };
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long p0 = (long long)blockIdx.x * blockDim.x + t; p0 < NP; p0 += NI * stride) {
+#pragma unroll
+    for (int u0 = 0; u0 < NI; u0 += GR) {
+      T w[GR][PK], v[VB][GR][PK];
+      bool in[GR];
+#pragma unroll
+      for (int u = 0; u < GR; ++u) {
+        in[u] = p0 + (u0 + u) * stride < NP;
+#pragma unroll
+        for (int c = 0; c < PK; ++c) w[u][c] = T(0);
+        if (in[u]) ld_pack<T, PK>(W, p0 + (u0 + u) * stride, w[u]);
+      }
+      const auto load = [&](const T* base, int count) {
+#pragma unroll
+        for (int q = 0; q < VB; ++q)
+#pragma unroll
+          for (int u = 0; u < GR; ++u) {
+#pragma unroll
+            for (int c = 0; c < PK; ++c) v[q][u][c] = T(0);
+            if (q < count && in[u]) ld_pack<T, PK>(base + q * ldv, p0 + (u0 + u) * stride, v[q][u]);
+          }
+      };
+      if (nu) {
+        load(Vu, nu);
+#pragma unroll
+        for (int u = 0; u < GR; ++u) {
+#pragma unroll
+          for (int q = 0; q < VB; ++q)
+            if (q < nu) {
+#pragma unroll
+              for (int c = 0; c < PK; ++c) w[u][c] = w[u][c] - h[q] * v[q][u][c];
+            }
+          if (in[u]) st_pack<T, PK>(W, p0 + (u0 + u) * stride, w[u]);
+        }
+      }
+      if (nd) load(Vd, nd);
+#pragma unroll
+      for (int u = 0; u < GR; ++u) {
+        if (nd) {
+          T vj[PK];   // V_j where the block holds it, for its Gram row (again, from L1)
+#pragma unroll
+          for (int c = 0; c < PK; ++c) vj[c] = T(0);
+          if (lastd && nd > 1 && in[u])
+            ld_pack<T, PK>(Vd + (long long)(nd - 1) * ldv, p0 + (u0 + u) * stride, vj);
+#pragma unroll
+          for (int q = 0; q < VB; ++q)
+            if (q < nd) add_dot(v[q][u], w[u], q);
+          if (lastd) {
+#pragma unroll
+            for (int q = 0; q < VB - 1; ++q)
+              if (q < nd - 1) add_dot(v[q][u], vj, VB + q);
+          }
+        } else {
+          add_dot(w[u], w[u], 0);
+        }
+        if constexpr (sizeof(T) == 4) {
+          if ((u0 + u) % UN == UN - 1) {
+            if (nd) {
+#pragma unroll
+              for (int q = 0; q < 2 * VB; ++q)
+                if (used(q)) {
+                  const float sum = hi[q] + f[q], g = sum - hi[q];
+                  lo[q] += (hi[q] - (sum - g)) + (f[q] - g);
+                  hi[q] = sum;
+                  f[q] = 0.f;
+                }
+            } else {
+              acc[0] += (double)f[0];   // no sum of squares beyond FP32's range
+              f[0] = 0.f;
+            }
+          }
+        }
+      }
+    }
+  }
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int q = 0; q < 2 * VB; ++q) acc[q] += (double)hi[q] + (double)lo[q];
+  }
+  if (!nd) {
+    const double tot = block_sum(acc[0]);
+    if (t == 0) Pout[blockIdx.x] = tot;
     return;
   }
-  for (int r = k - 1; r >= 0; --r) {
-    double v = g[r];
-    for (int q = r + 1; q < k; ++q) v -= R[r + ld * q] * y[q];
-    y[r] = v / R[r + ld * r];
+  if (lastd) {
+    const double x = warp_reduce_scatter<2 * VB>(acc, lane);
+    if (lane % (16 / VB) == 0) red[wp][lane / (16 / VB)] = x;
+  } else {
+    double a[VB];
+#pragma unroll
+    for (int q = 0; q < VB; ++q) a[q] = acc[q];
+    const double x = warp_reduce_scatter<VB>(a, lane);
+    if (lane % (32 / VB) == 0) red[wp][lane / (32 / VB)] = x;
   }
+  __syncthreads();
+  if (t < (lastd ? 2 * VB : VB)) {
+    double x = 0.0;
+    for (int q = 0; q < nw; ++q) x += red[q][t];
+    Pout[(t < VB ? t : kGB + t - VB) * kGsBlocks + blockIdx.x] = x;
+  }
+}
+
+// h_{j+1,j} from the last pass's sums, V_{j+1} = W / h_{j+1,j}, and the column update (the last CTA).
+template <typename T, int PK>
+__global__ void __launch_bounds__(512, 1)
+    k_gs_finish(const T* __restrict__ W, T* __restrict__ Vn, long long NP, const double* __restrict__ Pin, int nparts,
+                int j, int m, double* st, int method, StepEnd end) {
+  __shared__ double snorm[2];
+  __shared__ double col[kMaxM];
+  __shared__ KsStage S;
+  const int t = threadIdx.x, lane = t & 31;
+  const bool update = blockIdx.x == gridDim.x - 1;
+  Layout L{m};
+  // Only the CTA that may close the gate looks at it: after the end of a cycle the others form a V_{j+1} that
+  // nothing reads.
+  if (update && end.gate && *end.gate == 0) return;
+  if (update) {
+    ks_load(S, st, m, j, method, end, t, blockDim.x);
+    for (int i = t; i <= j; i += blockDim.x) col[i] = st[L.H() + i + (size_t)(m + 1) * j];
+    __syncthreads();
+  }
+  double carry = 0.0;
+  if (update && t == 32) {
+    ks_pivot(S, st, m, j, method);
+    ks_rotate(S, st, m, j, method, 0, j + 1, col, carry);
+  }
+  if (t < 32) {
+    double x = 0.0, hn, inv;
+    for (int c = lane; c < nparts; c += 32) x += Pin[c];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+    root(x, hn, inv);
+    if (lane == 0) {
+      snorm[0] = hn;
+      snorm[1] = inv;
+    }
+  }
+  __syncthreads();
+  if (update) {
+    if (t == 32) ks_finish(S, st, m, j, method, carry, snorm[0], snorm[1], end);
+    return;
+  }
+  const T inv = (T)snorm[1];
+  const long long stride = (long long)(gridDim.x - 1) * blockDim.x;
+  for (long long p = (long long)blockIdx.x * blockDim.x + t; p < NP; p += stride) {
+    T w[PK];
+    ld_pack<T, PK>(W, p, w);
+#pragma unroll
+    for (int c = 0; c < PK; ++c) w[c] = w[c] * inv;
+    st_pack<T, PK>(Vn, p, w);
+  }
+}
+
+// Back substitution R_k y = g_k (tGMRES: after the rotations; tFOM: after the eliminations).  Thread r keeps
+// row r: each solved entry is broadcast and subtracted by all rows at once, and the diagonal's reciprocals are
+// formed together beforehand (one thread, term by term with a division per row, took 16 us at k = 18).
+// Up to kSolveStage columns come from shared memory.
+constexpr int kSolveStage = 64;
+__global__ void k_ks_solve(double* st, int m, int k) {
+  __shared__ double sR[kSolveStage * kSolveStage], sy[kMaxM];
+  Layout L{m};
+  const int ld = m + 1, t = threadIdx.x;
+  const double* R = st + L.R();
+  const bool staged = k <= kSolveStage;
+  if (staged)
+    for (int e = t; e < k * k; e += blockDim.x) sR[e % k + kSolveStage * (e / k)] = R[e % k + ld * (e / k)];
+  double v = t < k ? st[L.g() + t] : 0.0;
+  const double d = t < k ? R[t + ld * t] : 1.0;
+  // a quotient as a product with the reciprocal, unless the reciprocal is not a normal number
+  const double inv = 1.0 / d;
+  const bool ok = fabs(inv) > 1e-290 && fabs(inv) < 1e290;
+  __syncthreads();
+  for (int c = k - 1; c >= 0; --c) {
+    const double r = t < c ? (staged ? sR[t + kSolveStage * c] : R[t + ld * c]) : 0.0;
+    if (t == c) sy[c] = ok ? v * inv : v / d;
+    __syncthreads();
+    if (t < c) v -= r * sy[c];
+  }
+  if (t < k) st[L.y() + t] = sy[t];
 }
 
 }  // namespace
@@ -350,22 +742,17 @@ void ks_init(void* state, int m, const double* beta_and_inv, cudaStream_t st) {
 
 double* ks_hist(void* s, int m) { return static_cast<double*>(s) + Layout{m}.hist(); }
 
-void ks_step(void* state, int m, int j, int method, const double* Pnorm, cudaStream_t st,
-             cudaGraphConditionalHandle handle, const double* stop) {
-  k_ks_step<<<1, 256, 0, st>>>(static_cast<double*>(state), m, j, method, Pnorm, handle, stop);
-  count_launch();
-  TS_CUDA(cudaGetLastError());
-}
-
-bool arnoldi_small_ok(long long N) { return N >= 1 && N <= kArnMaxN; }
-
-template <typename T, int R>
-void launch_arnoldi_cluster(int cl, int nt, T* W, T* V, long long ldv, int n, int j, int m, double* s, int method,
-                            cudaGraphConditionalHandle handle, const double* stop, int* gate, cudaStream_t st) {
+template <typename T>
+void launch_arnoldi_cluster(const T* W, T* V, long long ldv, int N, int j, int m, double* s, int method,
+                            const StepEnd& end, cudaStream_t st) {
+  // CTAs: one per 64 entries up to kArnCL
+  const int cl = std::min(kArnCL, std::max(1, (N + 63) / 64));
+  const int smem = (int)sizeof(T) * ((N + cl - 1) / cl) * (2 * kGB + 1);
+  if (smem > 32 * 1024) set_max_dynamic_smem(reinterpret_cast<const void*>(&k_arnoldi_cluster<T>), smem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cl, 1, 1);
-  cfg.blockDim = dim3(nt, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3(kArnThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -374,37 +761,56 @@ void launch_arnoldi_cluster(int cl, int nt, T* W, T* V, long long ldv, int n, in
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  TS_CUDA(cudaLaunchKernelEx(&cfg, k_arnoldi_cluster<T, R>, W, V, ldv, n, j, m, s, method, handle, stop, gate));
+  TS_CUDA(cudaLaunchKernelEx(&cfg, k_arnoldi_cluster<T>, W, V, ldv, N, j, m, s, method, end));
+  count_launch();
 }
+
+template <typename T, int PK>
+void launch_gs(T* W, T* V, long long ldv, long long NP, int j, int m, double* s, int method, double* P,
+               const StepEnd& end, cudaStream_t st) {
+  // one CTA per SM while there is work; few warps where it is little (their sums are FP64 work too)
+  const long long per = (NP + kGsBlocks - 1) / kGsBlocks;
+  const int nt = per >= 2048 ? 512 : (per >= 512 ? 256 : 128);
+  const int nb = (int)std::min<long long>(kGsBlocks, (NP + nt - 1) / nt);
+  double* Pb[2] = {P, P + (size_t)kGsSums * kGsBlocks};
+  const int nblk = j / kGB + 1;
+  for (int b = -1; b < nblk; ++b) {
+    if (j < 4)
+      k_gs_pass<T, PK, 4><<<nb, nt, 0, st>>>(W, V, ldv, NP, j, b, Pb[(b + 2) & 1], Pb[(b + 1) & 1], s, m, end.gate);
+    else
+      k_gs_pass<T, PK, 8><<<nb, nt, 0, st>>>(W, V, ldv, NP, j, b, Pb[(b + 2) & 1], Pb[(b + 1) & 1], s, m, end.gate);
+    count_launch();
+  }
+  k_gs_finish<T, PK><<<nb + 1, nt, 0, st>>>(W, V + (long long)(j + 1) * ldv, NP, Pb[nblk & 1], nb, j, m, s, method, end);
+  count_launch();
+}
+
+size_t arnoldi_scratch_bytes() { return sizeof(double) * 2 * kGsSums * kGsBlocks; }
 
 template <typename T>
-void arnoldi_small(T* W, T* V, long long ldv, long long N, int j, int m, void* state, int method, cudaStream_t st,
-                   cudaGraphConditionalHandle handle, const double* stop, int* gate) {
-  TS_REQUIRE(arnoldi_small_ok(N) && j >= 0 && j < m, "arnoldi_small: bad size");
+void arnoldi_step(T* W, T* V, long long ldv, long long N, int j, int m, void* state, int method, double* scratch,
+                  cudaStream_t st, cudaGraphConditionalHandle handle, const double* stop, int* gate) {
+  TS_REQUIRE(N >= 1 && j >= 0 && j < m && m <= kMaxM, "arnoldi_step: bad size");
   double* s = static_cast<double*>(state);
-  const int n = (int)N;
-  // CTAs: one per 64 entries up to kArnCL; threads: the CTA's share in R-element runs, whole warps
-  const int cl = (int)std::min<long long>(kArnCL, std::max<long long>(1, (N + 63) / 64));
-  const long long nc = (N + cl - 1) / cl;
-  auto threads = [&](int R) { return (int)((nc + 32LL * R - 1) / (32LL * R) * 32); };
-  if (nc <= kArnMaxThreads * 2LL)
-    launch_arnoldi_cluster<T, 2>(cl, threads(2), W, V, ldv, n, j, m, s, method, handle, stop, gate, st);
-  else if (nc <= kArnMaxThreads * 4LL)
-    launch_arnoldi_cluster<T, 4>(cl, threads(4), W, V, ldv, n, j, m, s, method, handle, stop, gate, st);
-  else if (nc <= kArnMaxThreads * 8LL)
-    launch_arnoldi_cluster<T, 8>(cl, threads(8), W, V, ldv, n, j, m, s, method, handle, stop, gate, st);
+  const StepEnd end{handle, stop, gate};
+  constexpr int PK = 16 / sizeof(T);
+  const auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  if (N <= kArnMaxN)
+    launch_arnoldi_cluster<T>(W, V, ldv, (int)N, j, m, s, method, end, st);
+  else if (N % PK == 0 && ldv % PK == 0 && aligned(W) && aligned(V))
+    launch_gs<T, PK>(W, V, ldv, N / PK, j, m, s, method, scratch, end, st);
   else
-    launch_arnoldi_cluster<T, 16>(cl, threads(16), W, V, ldv, n, j, m, s, method, handle, stop, gate, st);
-  count_launch();
+    launch_gs<T, 1>(W, V, ldv, N, j, m, s, method, scratch, end, st);
   TS_CUDA(cudaGetLastError());
 }
-template void arnoldi_small<double>(double*, double*, long long, long long, int, int, void*, int, cudaStream_t,
-                                    cudaGraphConditionalHandle, const double*, int*);
-template void arnoldi_small<float>(float*, float*, long long, long long, int, int, void*, int, cudaStream_t,
+template void arnoldi_step<double>(double*, double*, long long, long long, int, int, void*, int, double*, cudaStream_t,
                                    cudaGraphConditionalHandle, const double*, int*);
+template void arnoldi_step<float>(float*, float*, long long, long long, int, int, void*, int, double*, cudaStream_t,
+                                  cudaGraphConditionalHandle, const double*, int*);
 
-void ks_solve(void* state, int m, int k, int method, cudaStream_t st) {
-  k_ks_solve<<<1, 256, 0, st>>>(static_cast<double*>(state), m, k, method);
+void ks_solve(void* state, int m, int k, cudaStream_t st) {
+  TS_REQUIRE(k >= 1 && k <= kMaxM, "ks_solve: bad size");
+  k_ks_solve<<<1, (k + 31) / 32 * 32, 0, st>>>(static_cast<double*>(state), m, k);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }

@@ -7,10 +7,9 @@
 //             V_{j+1} = W / h_{j+1,j}.  Then y, X += V_k (*) y, and the true residual.
 // The host reads 4 doubles per inner step (estimate, 1/h, h, flags) to decide whether to stop --
 // except for small problems, which are bound by launch latency and by that look at every step.
-// Vectors of at most 65536 entries run everything after W = M(V_j) in one launch (arnoldi_small, a
-// thread-block cluster), and
-// on the FP64 DFMA engine (real basis, dense operator) a cycle's steps are launched ahead in chunks
-// behind a device gate that the step ending the cycle closes, so the host looks once per chunk.
+// With vectors of at most kAheadMaxN entries on the FP64 DFMA engine (real basis, dense operator) a cycle's
+// steps are launched ahead in chunks behind a device gate that the step ending the cycle closes, so the host
+// looks once per chunk.
 // Other problems of at most kGraphCycleMaxN unknowns run, from their second cycle on, each restart
 // cycle as one CUDA graph in which step j is the body of a conditional (IF) node (step j + 1's node
 // nested inside it) and the step's Givens / Hessenberg kernel switches the remaining steps off on the
@@ -39,6 +38,9 @@ namespace {
 // graphs (unless the environment sets TSTAR_NO_GRAPH_CYCLE=1, or statistics are being collected:
 // event timing is not allowed inside the conditional bodies).
 constexpr long long kGraphCycleMaxN = 1ll << 20;
+
+// Vectors of at most this many entries may have a cycle's steps launched ahead.
+constexpr long long kAheadMaxN = 65536;
 
 // One restart cycle (Algorithm 2 up to m steps) as an executable graph: a prologue (Givens state
 // reset, V_1 = R / ||R||), then m conditional (IF) nodes, node j holding inner step j and, nested at
@@ -107,9 +109,8 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
   double2* Rh = spectral ? static_cast<double2*>(ctx->ws.get("krylov_Rh", sizeof(double2) * (size_t)op->K * Ts))
                          : nullptr;
   double* R = static_cast<double*>(ctx->ws.get("krylov_R", sizeof(double) * (size_t)N));
-  double* P = static_cast<double*>(ctx->ws.get("krylov_P", sizeof(double) * 3 * kRedBlocks));
-  double* Pp[2] = {P, P + kRedBlocks};
-  double* P2 = P + 2 * kRedBlocks;
+  double* P2 = static_cast<double*>(ctx->ws.get("krylov_P", sizeof(double) * kRedBlocks));
+  double* Pgs = static_cast<double*>(ctx->ws.get("krylov_gs", arnoldi_scratch_bytes()));
   double* sc = static_cast<double*>(ctx->ws.get("krylov_scalars", sizeof(double) * 64));
   ctx->host_scalars[13] = 1.0;
   TS_CUDA(cudaMemcpyAsync(sc + 12, ctx->host_scalars + 13, sizeof(double), cudaMemcpyHostToDevice, st));
@@ -179,21 +180,19 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
   }
   if (res <= o.tol * normC) return finish(TS_OK);
 
-  // Inner step j of a cycle: W = M(V_j), the MGS sweep (fused with the next dot), the Givens /
-  // Hessenberg update (which, inside a graph, also decides whether the cycle goes on), and
-  // V_{j+1} = W / h_{j+1,j} when `scale_next` (the graph always forms it; unused after the last step).
+  // Inner step j of a cycle: W = M(V_j) and the rest of the step (arnoldi_step, which inside a graph and
+  // behind the gate also decides whether the cycle goes on).
   double* stop_dev = sc + 8;   // [tol ||C||, inner threshold or -1] for the graph's stopping test
-  const bool small_steps = arnoldi_small_ok(Nb);   // the post-apply part of a step is one launch
   // Small FP64 problems on the DFMA engine: a cycle's steps are launched ahead, kAheadChunk at a
   // time, without waiting for each step's estimate; a step that ends the cycle closes a device gate
   // and the kernels of the steps launched after it return at once.  (Each step of such a problem
   // is a few short kernels; the host round trip per step had cost about as much as they do.)
   const char* no_ahead = std::getenv("TSTAR_NO_LAUNCH_AHEAD");
-  const bool ahead = small_steps && sizeof(T) == 8 && !mixed && !spectral && !op->sp && !ozaki &&
+  const bool ahead = Nb <= kAheadMaxN && sizeof(T) == 8 && !mixed && !spectral && !op->sp && !ozaki &&
                      !ctx->timer.enabled && !(no_ahead && no_ahead[0] == '1');
   constexpr int kAheadChunk = 8;
   int* gate = ahead ? static_cast<int*>(ctx->ws.get("krylov_gate", sizeof(int))) : nullptr;
-  auto inner_step = [&](int j, cudaGraphConditionalHandle handle, bool scale_next, cudaStream_t q) {
+  auto inner_step = [&](int j, cudaGraphConditionalHandle handle, cudaStream_t q) {
     if constexpr (sizeof(T) == 8) {
       if (spectral)   // W = M(V_j) slice by slice: the scaling commutes with the per-slice operator
         apply_f64_spectral(ctx, op, reinterpret_cast<const double2*>(basis_ptr(V, Nb, j)),
@@ -205,18 +204,7 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
     } else {
       apply_basis(ctx, op, prec, basis_ptr(V, Nb, j), W, q);
     }
-    if (small_steps) {   // sweep, norm, Givens / Hessenberg update and V_{j+1} in one launch
-      arnoldi_small<T>(W, V, Nb, Nb, j, m, state, method, q, handle, stop_dev, ahead ? gate : nullptr);
-      return;
-    }
-    dot_partials<T>(basis_ptr(V, Nb, 0), W, Nb, Pp[0], q);
-    for (int i = 0; i <= j; ++i) {                                  // MGS sweep, fused with the next dot
-      const T* Vn = i < j ? basis_ptr(V, Nb, i + 1) : nullptr;
-      mgs_pass<T>(W, basis_ptr(V, Nb, i), Vn, Nb, Pp[i & 1], ks_H(state, m) + i + (size_t)(m + 1) * j,
-                  Pp[(i + 1) & 1], q);
-    }
-    ks_step(state, m, j, method, Pp[(j + 1) & 1], q, handle, stop_dev);
-    if (scale_next) scale_dev<T, T>(W, basis_ptr(V, Nb, j + 1), Nb, ks_est(state, m) + 1, q);   // V_{j+1}
+    arnoldi_step<T>(W, V, Nb, Nb, j, m, state, method, Pgs, q, handle, stop_dev, ahead ? gate : nullptr);
   };
   // V_1 = R / ||R|| (in the spectral basis: the scaled Fourier slices of R, over ||R||)
   auto init_v1 = [&](cudaStream_t q) {
@@ -261,7 +249,7 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
             });
           },
           [&](int j, cudaGraphConditionalHandle next, cudaStream_t q) {
-            return counted([&] { inner_step(j, next, j + 1 < m, q); });
+            return counted([&] { inner_step(j, next, q); });
           },
           [&](cudaStream_t) { return 0ll; }, cnt);
       cg->prologue_kernels = cnt.prologue;
@@ -327,7 +315,7 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
       int launched = 0;
       while (launched < m) {
         const int upto = std::min(m, launched + kAheadChunk);
-        for (int j = launched; j < upto; ++j) inner_step(j, 0, true, st);
+        for (int j = launched; j < upto; ++j) inner_step(j, 0, st);
         launched = upto;
         TS_CUDA(cudaMemcpyAsync(hest, ks_est(state, m), 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
         TS_CUDA(cudaStreamSynchronize(st));
@@ -345,7 +333,7 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
       ks_init(state, m, sc + 2, st);
       init_v1(st);
       for (int j = 0; j < m; ++j) {
-        inner_step(j, 0, false, st);
+        inner_step(j, 0, st);
         if (mixed) ++info.applies_low; else ++info.applies_fp64;
         TS_CUDA(cudaMemcpyAsync(hs + 8, ks_est(state, m), 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
         TS_CUDA(cudaStreamSynchronize(st));
@@ -358,7 +346,6 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
         const bool broke = ((int)flags & 1) != 0;
         const bool bad = ((int)flags & 6) != 0;
         if (bad || broke || est <= o.tol * normC || (mixed && est <= inner_tol * res)) break;
-        if (!small_steps) scale_dev<T, T>(W, basis_ptr(V, Nb, j + 1), Nb, ks_est(state, m) + 1, st);  // V_{j+1}
       }
     }
     ++info.cycles;
@@ -377,7 +364,7 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
       status = TS_ERR_NONFINITE;
       break;
     }
-    ks_solve(state, m, k, method, st);
+    ks_solve(state, m, k, st);
     if (spectral) {
       // X += V_k (*) y: combine the spectral basis, undo the slice scaling, back to real space
       double2* D = Rh;

@@ -1,13 +1,12 @@
 // Streaming kernels of the Arnoldi process (Algorithm 2) and of the solution update: inner
-// products and norms (Definition 2.3), the modified Gram-Schmidt sweep, scaling and the
-// (*) product of §3.1.  All are HBM-bound: grid-stride loops over packs of 4 elements (16- or
+// products and norms (Definition 2.3), scaling and the (*) product of §3.1.  All are HBM-bound: grid-stride loops over packs of 4 elements (16- or
 // 32-byte loads, two packs in flight per thread) when N is a multiple of 4 and the tensors are
 // 16-byte aligned, scalar loops otherwise; a fixed grid of kRedBlocks blocks wherever a sum is
 // formed; FP64 accumulation across packs whatever the storage type (an FP32 pack sums its own few
 // products in FP32 first, see pack.cuh).
 //
 // Reductions never use atomics: each block writes one partial sum, and whoever needs the total
-// (the next MGS pass, the Givens kernel) adds the kRedBlocks partials in a fixed order.  The
+// (a norm, a residual) adds the kRedBlocks partials in a fixed order.  The
 // results are therefore bitwise reproducible from run to run.  A short vector is reduced by fewer
 // blocks (red_blocks: one per 2048 elements, at most kRedBlocks), whose first block zeroes the
 // rest of the partial array, so consumers still add kRedBlocks entries: a small solve does not pay
@@ -68,80 +67,6 @@ __global__ void __launch_bounds__(kRedThreads) k_dot4(const T* __restrict__ x, c
   }
   const double tot = block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
-}
-
-// One modified Gram-Schmidt step fused with the inner product the next step needs:
-//   h = <V_i, W> (finalised from Pin);  W -= h V_i;  Pout = partials of <V_next, W> or <W, W>.
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_mgs(T* __restrict__ W, const T* __restrict__ Vi,
-                                                     const T* __restrict__ Vn, long long N,
-                                                     const double* __restrict__ Pin, double* __restrict__ h_out,
-                                                     double* __restrict__ Pout) {
-  const double h = finalize_partials(Pin);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *h_out = h;
-  zero_unused_partials(Pout);
-  const T hT = (T)h;
-  double acc = 0.0;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const T* __restrict__ other = Vn ? Vn : W;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < N; e += stride) {
-    const T w = W[e] - hT * Vi[e];
-    W[e] = w;
-    acc += (double)(Vn ? other[e] : w) * (double)w;
-  }
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) Pout[blockIdx.x] = tot;
-}
-
-// Packed form of k_mgs: N4 packs of 4.
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_mgs4(T* __restrict__ W, const T* __restrict__ Vi,
-                                                      const T* __restrict__ Vn, long long N4,
-                                                      const double* __restrict__ Pin, double* __restrict__ h_out,
-                                                      double* __restrict__ Pout) {
-  const double h = finalize_partials(Pin);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *h_out = h;
-  zero_unused_partials(Pout);
-  const T hT = (T)h;
-  double acc = 0.0;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < N4; e += 2 * stride) {
-    const long long e1 = e + stride;
-    const bool two = e1 < N4;
-    T w0[4], v0[4], o0[4], w1[4], v1[4], o1[4];
-    ld4(W, e, w0);
-    ld4(Vi, e, v0);
-    if (Vn) ld4(Vn, e, o0);
-    if (two) {
-      ld4(W, e1, w1);
-      ld4(Vi, e1, v1);
-      if (Vn) ld4(Vn, e1, o1);
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      w0[c] = w0[c] - hT * v0[c];
-      if (!Vn) o0[c] = w0[c];
-    }
-    st4(W, e, w0);
-    if (two) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        w1[c] = w1[c] - hT * v1[c];
-        if (!Vn) o1[c] = w1[c];
-      }
-      st4(W, e1, w1);
-    }
-    if constexpr (sizeof(T) == 4) {   // both packs summed in FP32, one FP64 add (pack.cuh)
-      float f = pack_dot(o0, w0);
-      if (two) f = pack_dot(o1, w1, f);
-      acc += (double)f;
-    } else {
-      acc_pack(acc, o0, w0);
-      if (two) acc_pack(acc, o1, w1);
-    }
-  }
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) Pout[blockIdx.x] = tot;
 }
 
 template <typename T, typename U>
@@ -271,17 +196,6 @@ void dot_partials(const T* x, const T* y, long long N, double* partials, cudaStr
   TS_CUDA(cudaGetLastError());
 }
 
-template <typename T>
-void mgs_pass(T* W, const T* Vi, const T* Vnext, long long N, const double* Pin, double* h_out, double* Pout,
-              cudaStream_t st) {
-  if (packable(N, {W, Vi, Vnext}))
-    k_mgs4<T><<<red_blocks(N), kRedThreads, 0, st>>>(W, Vi, Vnext, N / 4, Pin, h_out, Pout);
-  else
-    k_mgs<T><<<red_blocks(N), kRedThreads, 0, st>>>(W, Vi, Vnext, N, Pin, h_out, Pout);
-  count_launch();
-  TS_CUDA(cudaGetLastError());
-}
-
 template <typename T, typename U>
 void scale_dev(const T* x, U* y, long long N, const double* scale, cudaStream_t st) {
   if (packable(N, {x, y})) k_scale4<T, U><<<grid_for(N / 4), 256, 0, st>>>(x, y, N / 4, scale);
@@ -327,13 +241,8 @@ void fill_zero(void* p, size_t bytes, cudaStream_t st) { TS_CUDA(cudaMemsetAsync
 
 template void dot_partials<double>(const double*, const double*, long long, double*, cudaStream_t);
 template void dot_partials<float>(const float*, const float*, long long, double*, cudaStream_t);
-template void mgs_pass<double>(double*, const double*, const double*, long long, const double*, double*, double*,
-                               cudaStream_t);
-template void mgs_pass<float>(float*, const float*, const float*, long long, const double*, double*, double*,
-                              cudaStream_t);
 template void scale_dev<double, double>(const double*, double*, long long, const double*, cudaStream_t);
 template void scale_dev<double, float>(const double*, float*, long long, const double*, cudaStream_t);
-template void scale_dev<float, float>(const float*, float*, long long, const double*, cudaStream_t);
 template void multi_axpy<double, double>(double*, const double*, long long, long long, const double*, int, double,
                                          const double*, cudaStream_t);
 template void multi_axpy<float, double>(double*, const float*, long long, long long, const double*, int, double,
