@@ -83,13 +83,10 @@ __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
     else *d = make_double2(0.0, 0.0);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
-  for (int r = t; r < p; r += kSmThreads) {
-    double sv, cv;
-    sincospi(2.0 * r / p, &sv, &cv);
-    tc[r] = cv;
-    tsn[r] = sv;
+  if constexpr (!POW2) {
+    for (int r = t; r < p; r += kSmThreads) direct_twiddle(r, p, tc[r], tsn[r]);
+    __syncthreads();
   }
-  __syncthreads();
 
   // Tubes: the TN columns of X (Xc[k][l][j]), then its 4 rows (Xr[k][l][i]).
   const int ncol = TN * n;
@@ -112,7 +109,7 @@ __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
     const double* src = a.X + (long long)col * n + row;
     if constexpr (POW2) {
       rfft_reg<double, P>([&](int u) { return in ? src[u * T] : 0.0; },
-                          [&](int k, double re, double im) { dst[k * step] = make_double2(re, im); }, tc, tsn);
+                          [&](int k, double re, double im) { dst[k * step] = make_double2(re, im); });
     } else {
       double x[P];
 #pragma unroll
@@ -132,6 +129,12 @@ __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
         }
         dst[k * step] = make_double2(re, im);
       }
+    }
+  }
+  if constexpr (POW2) {   // for the inverse
+    for (int r = t; r < p; r += kSmThreads) {
+      tc[r] = cos32(r * (32 / P));
+      tsn[r] = sin32(r * (32 / P));
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");

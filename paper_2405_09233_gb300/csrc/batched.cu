@@ -233,13 +233,10 @@ __global__ void __launch_bounds__(kTubes) k_b_rfft(BDev d, const Real* __restric
   const BInst& ins = d.inst[i];
   const int p = ins.p;
   __shared__ Real tc[64], tsn[64];
-  for (int r = threadIdx.x; r < p; r += blockDim.x) {
-    double sv, cv;
-    sincospi(2.0 * r / p, &sv, &cv);
-    tc[r] = (Real)cv;
-    tsn[r] = (Real)sv;
+  if (p > 32 || (p & (p - 1)) != 0 || p == 1) {   // the direct sums' table (uniform over the block)
+    for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, tc[r], tsn[r]);
+    __syncthreads();
   }
-  __syncthreads();
   const long long e = d.tb_off[blockIdx.x] + threadIdx.x;
   if (e >= ins.T) return;
   const Real* src = SRC == 0 ? in + ins.offN : reinterpret_cast<const Real*>(ins.X);
@@ -253,11 +250,11 @@ __global__ void __launch_bounds__(kTubes) k_b_rfft(BDev d, const Real* __restric
     dst[k * T + e] = v;
   };
   switch (p) {
-    case 2: rfft_reg<Real, 2>(ld, stv, tc, tsn); break;
-    case 4: rfft_reg<Real, 4>(ld, stv, tc, tsn); break;
-    case 8: rfft_reg<Real, 8>(ld, stv, tc, tsn); break;
-    case 16: rfft_reg<Real, 16>(ld, stv, tc, tsn); break;
-    case 32: rfft_reg<Real, 32>(ld, stv, tc, tsn); break;
+    case 2: rfft_reg<Real, 2>(ld, stv); break;
+    case 4: rfft_reg<Real, 4>(ld, stv); break;
+    case 8: rfft_reg<Real, 8>(ld, stv); break;
+    case 16: rfft_reg<Real, 16>(ld, stv); break;
+    case 32: rfft_reg<Real, 32>(ld, stv); break;
     default: {
       const int K = p / 2 + 1;
       for (int k = 0; k < K; ++k) {
@@ -286,20 +283,18 @@ __global__ void __launch_bounds__(kTubes) k_b_irfft(BDev d, const Cplx* __restri
   const BInst& ins = d.inst[i];
   const int p = ins.p;
   __shared__ Real tc[64], tsn[64];
-  for (int r = threadIdx.x; r < p; r += blockDim.x) {
-    double sv, cv;
-    sincospi(2.0 * r / p, &sv, &cv);
-    tc[r] = (Real)cv;
-    tsn[r] = (Real)sv;
+  if (p > 32 || (p & (p - 1)) != 0 || p == 1) {   // the direct sums' table (uniform over the block)
+    for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, tc[r], tsn[r]);
+    __syncthreads();
   }
-  __syncthreads();
   const long long e = d.tb_off[blockIdx.x] + threadIdx.x;
   double local = 0.0;
   if (e < ins.T) {
     const Cplx* src = in + ins.offS;
     Real* dst = out + ins.offN;
     const long long T = ins.T;
-    const Real invp = Real(1) / Real(p);
+    // (a register FFT in FP64 has applied the scale)
+    const Real invp = sizeof(Real) == 8 && p <= 32 && (p & (p - 1)) == 0 && p > 1 ? Real(1) : Real(1) / Real(p);
     auto ld = [&](int k, Real& re, Real& im) {
       const Cplx c = src[k * T + e];
       re = c.x;
@@ -314,11 +309,11 @@ __global__ void __launch_bounds__(kTubes) k_b_irfft(BDev d, const Cplx* __restri
       dst[t * T + e] = v;
     };
     switch (p) {
-      case 2: irfft_reg<Real, 2>(ld, stv, tc, tsn); break;
-      case 4: irfft_reg<Real, 4>(ld, stv, tc, tsn); break;
-      case 8: irfft_reg<Real, 8>(ld, stv, tc, tsn); break;
-      case 16: irfft_reg<Real, 16>(ld, stv, tc, tsn); break;
-      case 32: irfft_reg<Real, 32>(ld, stv, tc, tsn); break;
+      case 2: irfft_reg<Real, 2>(ld, stv); break;
+      case 4: irfft_reg<Real, 4>(ld, stv); break;
+      case 8: irfft_reg<Real, 8>(ld, stv); break;
+      case 16: irfft_reg<Real, 16>(ld, stv); break;
+      case 32: irfft_reg<Real, 32>(ld, stv); break;
       default: {
         const int K = p / 2 + 1, nyq = (p % 2 == 0) ? p / 2 : -1;
         for (int t = 0; t < p; ++t) {

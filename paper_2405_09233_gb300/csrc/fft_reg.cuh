@@ -8,9 +8,15 @@
 // real FFT), about 40% fewer arithmetic instructions than a complex length-P FFT with zero
 // imaginary parts.  That matters for FP64 tubes, which GB300's FP64 rate makes instruction bound.
 //
-// Convention (MATLAB's fft): forward X_k = sum_t x_t e^{-2 pi i k t / P}; the inverse here is the
-// unnormalised sum with e^{+2 pi i k t / P} (the caller applies 1/P).  Twiddle table: tc[r] =
-// cos(2 pi r / P), ts[r] = sin(2 pi r / P), r < P, computed with sincospi.
+// Convention (MATLAB's fft): forward X_k = sum_t x_t e^{-2 pi i k t / P}; the inverse is the sum with
+// e^{+2 pi i k t / P}, times 1/P in FP64 and unnormalised in FP32 (the caller applies kIrfftScale).
+//
+// The twiddles are constants (cos and sin of multiples of pi/16).  As a table that every block computed with
+// sincospi they cost 1.3 us at the start of a block, in FP64 instructions of one warp, whatever the tube
+// type.  In FP64, whose instructions these kernels are bound by, the butterflies with twiddle (1 -+ i)/sqrt 2
+// multiply sums of the two parts (6 instructions instead of 8) and the scale 1/P rides on constants and
+// multiply-adds that are there anyway: 16 fewer instructions of ~115 for an inverse of 16 points.  FP64,
+// 1024 x 1024 x 16: forward 208 -> 185 us, inverse 233 -> 186; 64 uneven instances: FP32 49 -> 31 and 48 -> 26.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -23,55 +29,102 @@ __host__ __device__ constexpr int bitrevc(int x, int bits) {
   return r;
 }
 
+// cos(2 pi r / 32) and sin(2 pi r / 32), correctly rounded; 32 r / P for the P-th roots of unity.
+__host__ __device__ constexpr double cos32(int r) {
+  const double t[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                       0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                       0.19509032201612826785, 0.0};
+  r &= 31;
+  if (r > 16) r = 32 - r;
+  return r > 8 ? -t[16 - r] : t[r];
+}
+__host__ __device__ constexpr double sin32(int r) { return cos32(r + 24); }
+template <typename Real, int P>
+__host__ __device__ constexpr Real kIrfftScale() { return sizeof(Real) == 8 ? Real(1) : Real(1) / Real(P); }
+// The P-th roots for a direct sum over any p: cos and sin of 2 pi r / p.
+template <typename Real>
+__device__ __forceinline__ void direct_twiddle(int r, int p, Real& c, Real& s) {
+  double sv, cv;
+  sincospi(2.0 * r / p, &sv, &cv);
+  c = (Real)cv;
+  s = (Real)sv;
+}
+
+// a b + c d and a b - c d with the rounding written out: the second product is rounded, the first is not.
+// Left to the compiler the choice changes with what it knows about the constants, and an FP32 transform that
+// feeds BF16 operands has to give the same bits everywhere.
+template <typename Real>
+__device__ __forceinline__ Real mul2_add(Real a, Real b, Real c, Real d) {
+  if constexpr (sizeof(Real) == 8) return __fma_rn(a, b, __dmul_rn(c, d));
+  else return __fmaf_rn(a, b, __fmul_rn(c, d));
+}
+template <typename Real>
+__device__ __forceinline__ Real mul2_sub(Real a, Real b, Real c, Real d) {
+  if constexpr (sizeof(Real) == 8) return __fma_rn(a, b, -__dmul_rn(c, d));
+  else return __fmaf_rn(a, b, -__fmul_rn(c, d));
+}
+
 // One radix-2 stage of span LEN, then the next; LEN is a template argument so that every register
 // index is a compile-time constant (a runtime stage loop leaves the arrays in local memory).
-// TSTR: stride into the twiddle table (2 when a length-P/2 FFT uses the table of length P).
+// TSTR: stride into the roots of unity (2 when a length-P/2 FFT uses those of length P).
 template <typename Real, int P, bool INVERSE, int LEN, int TSTR = 1>
 struct FftStages {
-  static __device__ __forceinline__ void run(Real (&xr)[P], Real (&xi)[P], const Real* __restrict__ tc,
-                                             const Real* __restrict__ ts) {
-    constexpr int half = LEN / 2, stride = TSTR * (P / LEN);
-#pragma unroll
-    for (int start = 0; start < P; start += LEN) {
-#pragma unroll
-      for (int q = 0; q < half; ++q) {
-        const int a = start + q, b = start + q + half;
-        Real vr, vi;
-        if (q == 0) {                       // twiddle 1
-          vr = xr[b];
-          vi = xi[b];
-        } else if (4 * q == LEN) {          // twiddle -+i
-          vr = INVERSE ? -xi[b] : xi[b];
-          vi = INVERSE ? xr[b] : -xr[b];
-        } else {
-          const Real wr = tc[q * stride];
-          const Real wi = INVERSE ? ts[q * stride] : -ts[q * stride];
-          vr = xr[b] * wr - xi[b] * wi;
-          vi = xr[b] * wi + xi[b] * wr;
-        }
-        xr[b] = xr[a] - vr;
-        xi[b] = xi[a] - vi;
-        xr[a] = xr[a] + vr;
-        xi[a] = xi[a] + vi;
-      }
+  template <int Q, int START>
+  static __device__ __forceinline__ void butterfly(Real (&xr)[P], Real (&xi)[P]) {
+    constexpr int half = LEN / 2, a = START + Q, b = START + Q + half, root = Q * (32 / LEN);
+    Real vr, vi;
+    if constexpr (Q == 0) {                       // twiddle 1
+      vr = xr[b];
+      vi = xi[b];
+    } else if constexpr (4 * Q == LEN) {          // twiddle -+i
+      vr = INVERSE ? -xi[b] : xi[b];
+      vi = INVERSE ? xr[b] : -xr[b];
+    } else if constexpr (sizeof(Real) == 8 && (8 * Q == LEN || 8 * Q == 3 * LEN)) {   // (+-1 -+ i) / sqrt 2
+      // forward: v = h (sum, dif), then h (dif, -sum); inverse: h (dif, sum), then h (-sum, dif)
+      constexpr bool q1 = 8 * Q == LEN;
+      constexpr Real h = Real(cos32(4)), cr = INVERSE && !q1 ? -h : h, ci = !INVERSE && !q1 ? -h : h;
+      const Real sum = xr[b] + xi[b], dif = INVERSE ? xr[b] - xi[b] : xi[b] - xr[b];
+      const Real pr = q1 != INVERSE ? sum : dif, pi = q1 != INVERSE ? dif : sum;
+      xr[b] = fma(-cr, pr, xr[a]);
+      xi[b] = fma(-ci, pi, xi[a]);
+      xr[a] = fma(cr, pr, xr[a]);
+      xi[a] = fma(ci, pi, xi[a]);
+      return;
+    } else {
+      constexpr Real wr = Real(cos32(root)), si = Real(sin32(root));
+      vr = INVERSE ? mul2_sub(xr[b], wr, xi[b], si) : mul2_add(xr[b], wr, xi[b], si);
+      vi = INVERSE ? mul2_add(xr[b], si, xi[b], wr) : mul2_sub(xi[b], wr, xr[b], si);
     }
-    FftStages<Real, P, INVERSE, 2 * LEN, TSTR>::run(xr, xi, tc, ts);
+    xr[b] = xr[a] - vr;
+    xi[b] = xi[a] - vi;
+    xr[a] = xr[a] + vr;
+    xi[a] = xi[a] + vi;
+  }
+  template <int I>   // butterflies I .. P/2 - 1: group by group
+  static __device__ __forceinline__ void all(Real (&xr)[P], Real (&xi)[P]) {
+    if constexpr (I < P / 2) {
+      butterfly<I % (LEN / 2), (I / (LEN / 2)) * LEN>(xr, xi);
+      all<I + 1>(xr, xi);
+    }
+  }
+  static __device__ __forceinline__ void run(Real (&xr)[P], Real (&xi)[P]) {
+    all<0>(xr, xi);
+    FftStages<Real, P, INVERSE, 2 * LEN, TSTR>::run(xr, xi);
   }
 };
 template <typename Real, int P, bool INVERSE, int TSTR>
 struct FftStages<Real, P, INVERSE, 2 * P, TSTR> {
-  static __device__ __forceinline__ void run(Real (&)[P], Real (&)[P], const Real*, const Real*) {}
+  static __device__ __forceinline__ void run(Real (&)[P], Real (&)[P]) {}
 };
 
 // In-place decimation-in-time FFT; the inputs must already sit in bit-reversed order.
 template <typename Real, int P, bool INVERSE>
-__device__ __forceinline__ void fft_bitrev_inplace(Real (&xr)[P], Real (&xi)[P], const Real* __restrict__ tc,
-                                                   const Real* __restrict__ ts) {
-  FftStages<Real, P, INVERSE, 2>::run(xr, xi, tc, ts);
+__device__ __forceinline__ void fft_bitrev_inplace(Real (&xr)[P], Real (&xi)[P]) {
+  FftStages<Real, P, INVERSE, 2>::run(xr, xi);
 }
 
 // Forward transform of P real samples read by `load(t)`; writes the P/2+1 non-redundant outputs
-// through `store(k, re, im)`.  Twiddle table of length P.
+// through `store(k, re, im)`.
 //
 // Two-for-one (P >= 4): z_t = x_2t + i x_2t+1, Z = DFT_M(z).  With E_k, O_k the length-M DFTs of the
 // even and odd samples, Z_k = E_k + i O_k and conj(Z_M-k) = E_k - i O_k, so
@@ -79,7 +132,7 @@ __device__ __forceinline__ void fft_bitrev_inplace(Real (&xr)[P], Real (&xi)[P],
 // X_M-k = conj(E_k) - conj(w^k O_k), w = e^{-2 pi i/P}; X_0 = Re Z_0 + Im Z_0, X_M = Re Z_0 - Im Z_0
 // and X_M/2 = conj Z_M/2.
 template <typename Real, int P, typename Load, typename Store>
-__device__ __forceinline__ void rfft_reg(Load load, Store store, const Real* tc, const Real* ts) {
+__device__ __forceinline__ void rfft_reg(Load load, Store store) {
   if constexpr (P < 4) {
     constexpr int LB = ilog2c(P);
     Real xr[P], xi[P];
@@ -88,7 +141,7 @@ __device__ __forceinline__ void rfft_reg(Load load, Store store, const Real* tc,
       xr[bitrevc(t, LB)] = load(t);
       xi[bitrevc(t, LB)] = Real(0);
     }
-    fft_bitrev_inplace<Real, P, false>(xr, xi, tc, ts);
+    fft_bitrev_inplace<Real, P, false>(xr, xi);
 #pragma unroll
     for (int k = 0; k <= P / 2; ++k) store(k, xr[k], (k == 0 || k == P / 2) ? Real(0) : xi[k]);
   } else {
@@ -99,7 +152,7 @@ __device__ __forceinline__ void rfft_reg(Load load, Store store, const Real* tc,
       zr[bitrevc(t, LB)] = load(2 * t);
       zi[bitrevc(t, LB)] = load(2 * t + 1);
     }
-    FftStages<Real, M, false, 2, 2>::run(zr, zi, tc, ts);
+    FftStages<Real, M, false, 2, 2>::run(zr, zi);
     store(0, zr[0] + zi[0], Real(0));
     store(M, zr[0] - zi[0], Real(0));
 #pragma unroll
@@ -109,8 +162,8 @@ __device__ __forceinline__ void rfft_reg(Load load, Store store, const Real* tc,
       } else {
         const Real s1 = zr[k] + zr[M - k], s2 = zi[k] - zi[M - k];
         const Real s3 = zi[k] + zi[M - k], s4 = zr[M - k] - zr[k];
-        const Real hc = Real(0.5) * tc[k], hs = Real(0.5) * ts[k];
-        const Real u = hc * s3 + hs * s4, v = hc * s4 - hs * s3;
+        const Real hc = Real(0.5) * Real(cos32(k * (32 / P))), hs = Real(0.5) * Real(sin32(k * (32 / P)));
+        const Real u = mul2_add(hc, s3, hs, s4), v = mul2_sub(hc, s4, hs, s3);
         store(k, Real(0.5) * s1 + u, Real(0.5) * s2 + v);
         store(M - k, Real(0.5) * s1 - u, v - Real(0.5) * s2);
       }
@@ -119,14 +172,15 @@ __device__ __forceinline__ void rfft_reg(Load load, Store store, const Real* tc,
 }
 
 // Inverse of a Hermitian half spectrum c_0..c_{P/2} read by `load(k, re, im)`: writes the P real
-// samples times P (unnormalised) through `store(t, value)`.  Imaginary parts of c_0 and c_{P/2}
+// samples (FP32: times P) through `store(t, value)`.  Imaginary parts of c_0 and c_{P/2}
 // are ignored (they are zero for the spectrum of a real tensor).
 //
 // Two-for-one (P >= 4), the forward steps reversed: Z'_k = (c_k + conj c_M-k) +
 // i (c_k - conj c_M-k) w^-k (= 2 Z_k), and the unnormalised inverse DFT_M of Z' is P z, so
 // x_2t = Re and x_2t+1 = Im of its entry t.
 template <typename Real, int P, typename Load, typename Store>
-__device__ __forceinline__ void irfft_reg(Load load, Store store, const Real* tc, const Real* ts) {
+__device__ __forceinline__ void irfft_reg(Load load, Store store) {
+  constexpr Real scale = Real(1) / (kIrfftScale<Real, P>() * Real(P));   // FP64: 1/P; FP32: 1
   if constexpr (P < 4) {
     constexpr int LB = ilog2c(P);
     Real xr[P], xi[P];
@@ -142,9 +196,9 @@ __device__ __forceinline__ void irfft_reg(Load load, Store store, const Real* tc
         xi[bitrevc(P - k, LB)] = -im;
       }
     }
-    fft_bitrev_inplace<Real, P, true>(xr, xi, tc, ts);
+    fft_bitrev_inplace<Real, P, true>(xr, xi);
 #pragma unroll
-    for (int t = 0; t < P; ++t) store(t, xr[t]);
+    for (int t = 0; t < P; ++t) store(t, sizeof(Real) == 8 ? scale * xr[t] : xr[t]);
   } else {
     constexpr int M = P / 2, LB = ilog2c(M);
     Real zr[M], zi[M];
@@ -154,27 +208,38 @@ __device__ __forceinline__ void irfft_reg(Load load, Store store, const Real* tc
       load(M, c, d);
       zr[0] = a + c;
       zi[0] = a - c;
+      if (sizeof(Real) == 8) {
+        zr[0] *= scale;
+        zi[0] *= scale;
+      }
     }
 #pragma unroll
     for (int k = 1; 2 * k <= M; ++k) {
       Real a, b;
       load(k, a, b);
       if (2 * k == M) {
-        zr[bitrevc(k, LB)] = Real(2) * a;
-        zi[bitrevc(k, LB)] = Real(-2) * b;
+        zr[bitrevc(k, LB)] = Real(2) * scale * a;
+        zi[bitrevc(k, LB)] = Real(-2) * scale * b;
       } else {
         Real c, d;
         load(M - k, c, d);
         const Real s1 = a + c, s2 = b - d, s3 = b + d, s4 = c - a;
-        const Real co = tc[k], si = ts[k];
-        const Real pp = -(s4 * co + s3 * si), qq = s3 * co - s4 * si;
-        zr[bitrevc(k, LB)] = s1 - qq;
-        zi[bitrevc(k, LB)] = s2 + pp;
-        zr[bitrevc(M - k, LB)] = s1 + qq;
-        zi[bitrevc(M - k, LB)] = pp - s2;
+        const Real co = scale * Real(cos32(k * (32 / P))), si = scale * Real(sin32(k * (32 / P)));
+        const Real pp = -mul2_add(s4, co, s3, si), qq = mul2_sub(s3, co, s4, si);
+        if constexpr (sizeof(Real) == 8) {
+          zr[bitrevc(k, LB)] = fma(scale, s1, -qq);
+          zi[bitrevc(k, LB)] = fma(scale, s2, pp);
+          zr[bitrevc(M - k, LB)] = fma(scale, s1, qq);
+          zi[bitrevc(M - k, LB)] = fma(-scale, s2, pp);
+        } else {
+          zr[bitrevc(k, LB)] = s1 - qq;
+          zi[bitrevc(k, LB)] = s2 + pp;
+          zr[bitrevc(M - k, LB)] = s1 + qq;
+          zi[bitrevc(M - k, LB)] = pp - s2;
+        }
       }
     }
-    FftStages<Real, M, true, 2, 2>::run(zr, zi, tc, ts);
+    FftStages<Real, M, true, 2, 2>::run(zr, zi);
 #pragma unroll
     for (int t = 0; t < M; ++t) {
       store(2 * t, zr[t]);

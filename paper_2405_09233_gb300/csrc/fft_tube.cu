@@ -20,12 +20,7 @@ template <> struct Vec2<float> { using T = float2; };
 
 template <typename Real>
 __device__ __forceinline__ void load_twiddles(Real* c, Real* s, int p) {
-  for (int r = threadIdx.x; r < p; r += blockDim.x) {
-    double sv, cv;
-    sincospi(2.0 * r / p, &sv, &cv);
-    c[r] = (Real)cv;
-    s[r] = (Real)sv;
-  }
+  for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, c[r], s[r]);
   __syncthreads();
 }
 
@@ -69,8 +64,6 @@ template <typename Real, typename Cplx, int P>
 __global__ void __launch_bounds__(256) k_rfft_pow2(const Real* __restrict__ in, Cplx* __restrict__ out, long long T,
                                                    const int* __restrict__ gate) {
   if (gate && *gate == 0) return;   // a cycle that already ended (launched ahead)
-  __shared__ Real tc[P], tsn[P];
-  load_twiddles(tc, tsn, P);
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < T;
        e += (long long)gridDim.x * blockDim.x) {
     rfft_reg<Real, P>([&](int t) { return in[t * T + e]; },
@@ -79,8 +72,7 @@ __global__ void __launch_bounds__(256) k_rfft_pow2(const Real* __restrict__ in, 
                         v.x = re;
                         v.y = im;
                         out[k * T + e] = v;
-                      },
-                      tc, tsn);
+                      });
   }
 }
 
@@ -89,9 +81,6 @@ __global__ void __launch_bounds__(256) k_irfft_pow2(const Cplx* __restrict__ in,
                                                     const Real* __restrict__ C, double* __restrict__ partials,
                                                     const int* __restrict__ gate) {
   if (gate && *gate == 0) return;   // a cycle that already ended (launched ahead)
-  __shared__ Real tc[P], tsn[P];
-  load_twiddles(tc, tsn, P);
-  const Real invp = Real(1) / Real(P);
   double local = 0.0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < T;
        e += (long long)gridDim.x * blockDim.x) {
@@ -102,14 +91,13 @@ __global__ void __launch_bounds__(256) k_irfft_pow2(const Cplx* __restrict__ in,
           im = c.y;
         },
         [&](int t, Real v) {
-          v *= invp;
+          v *= kIrfftScale<Real, P>();
           if (MODE == IRFFT_RESIDUAL) {
             v = C[t * T + e] - v;
             local += (double)v * (double)v;
           }
           out[t * T + e] = v;
-        },
-        tc, tsn);
+        });
   }
   if (MODE == IRFFT_RESIDUAL) {
     const double tot = block_sum(local);

@@ -559,12 +559,7 @@ __global__ void __launch_bounds__(256) k_rfft_planar(const float* __restrict__ X
                                                      OpT* __restrict__ im, int n, int s, int p, int ldn,
                                                      float* __restrict__ re_lo, float* __restrict__ im_lo) {
   __shared__ float tc[PMAX], tsn[PMAX];
-  for (int r = threadIdx.x; r < p; r += blockDim.x) {
-    double sv, cv;
-    sincospi(2.0 * r / p, &sv, &cv);
-    tc[r] = (float)cv;
-    tsn[r] = (float)sv;
-  }
+  for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, tc[r], tsn[r]);
   __syncthreads();
   const int K = p / 2 + 1;
   const long long T = (long long)n * s;
@@ -619,14 +614,6 @@ __global__ void __launch_bounds__(256) k_rfft_planar_fused(const float* __restri
   OpT* tim = tre + K * TJ * 33;
   float* tlr = reinterpret_cast<float*>(tim + K * TJ * 33);   // split: low parts, same shape
   float* tli = tlr + (SPLIT ? K * TJ * 33 : 0);
-  __shared__ float tc[P], tsn[P];
-  for (int r = threadIdx.y * 32 + threadIdx.x; r < P; r += 256) {
-    double sv, cv;
-    sincospi(2.0 * r / P, &sv, &cv);
-    tc[r] = (float)cv;
-    tsn[r] = (float)sv;
-  }
-  __syncthreads();
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * TJ;
   const long long T = (long long)n * s;
@@ -657,8 +644,7 @@ __global__ void __launch_bounds__(256) k_rfft_planar_fused(const float* __restri
                              cim_lo[o] = lb;
                            }
                          }
-                       },
-                       tc, tsn);
+                       });
   }
   __syncthreads();
   // row-major planes: rows i0 + r (r < 32), columns j0 + c (c < TJ), all K slices
