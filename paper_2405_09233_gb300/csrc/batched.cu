@@ -29,6 +29,7 @@
 #include "reduce.cuh"
 #include "pack.cuh"
 #include "fft_reg.cuh"
+#include "gs_sweep.cuh"
 #include "gemm_tile.cuh"
 #include "cycle_graph.cuh"
 
@@ -38,7 +39,9 @@ void ensure_f32_operator(ts_op* op, cudaStream_t st);  // lowprec.cu
 
 namespace {
 
-constexpr int kChunk = 4096;      // unknowns per streaming block (256 threads x 16)
+// Unknowns per streaming block of 256 threads, a multiple of 4: large batches take longer ones, since every
+// block of a sweep adds up its instance's partial sums and reduces its own, in FP64.
+long long stream_chunk(long long totN) { return totN >= 4ll * 152 * 8192 ? 8192 : 4096; }
 constexpr int kTubes = 256;       // tubes per DFT block (one per thread)
 
 struct BInst {
@@ -73,12 +76,13 @@ struct BDev {
   double* sc;
   double* state;
   long long stride;
+  long long chunk;   // unknowns per streaming block
   double inner_tol;
   int mixed;
 };
 
 // Per-instance Krylov state: H and its rotated copy R ((m+1) x m each), the rotations cs, sn (m),
-// the rotated right-hand side g (m+1) and the solution y (m).
+// the rotated right-hand side g (m+1), the solution y (m) and the basis's Gram rows (m+1 of kGB).
 struct StLayout {
   int m;
   __host__ __device__ long long H() const { return 0; }
@@ -87,7 +91,8 @@ struct StLayout {
   __host__ __device__ long long sn() const { return cs() + m; }
   __host__ __device__ long long g() const { return sn() + m; }
   __host__ __device__ long long y() const { return g() + m + 1; }
-  __host__ __device__ long long end() const { return y() + m; }
+  __host__ __device__ long long gram() const { return y() + m; }   // as the single solver's (gs_sweep.cuh)
+  __host__ __device__ long long end() const { return gram() + (long long)(m + 1) * kGB; }
 };
 long long state_stride(int m) { return StLayout{m}.end(); }
 
@@ -111,85 +116,48 @@ __global__ void __launch_bounds__(256) k_b_scale_R(BDev d, const double* __restr
   const BInst& in = d.inst[i];
   const double sc = d.sc[16 * i + SC_INVRES];
   const long long e0 = in.offN + d.nb_off[blockIdx.x];
-  const long long e1 = min(in.offN + in.N, e0 + kChunk);
+  const long long e1 = min(in.offN + in.N, e0 + d.chunk);
   for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) V0[e] = (T)(R[e] * sc);
 }
 
-// Instance offsets are multiples of 4 and chunks are kChunk long, so a block's range starts
+// Instance offsets and chunks are multiples of 4, so a block's range starts
 // 16-byte aligned: the streaming kernels below move packs of 4 and finish a ragged instance tail
 // element by element.
-template <typename T>
-__global__ void __launch_bounds__(256) k_b_dot(BDev d, const T* __restrict__ x, const T* __restrict__ y,
-                                               double* __restrict__ P) {
-  const int i = d.nb_inst[blockIdx.x];
-  if (!d.act[i]) return;
-  const BInst& in = d.inst[i];
-  const long long e0 = in.offN + d.nb_off[blockIdx.x];
-  const long long e1 = min(in.offN + in.N, e0 + kChunk);
-  const long long n4 = (e1 - e0) / 4, p0 = e0 / 4;
-  double acc = 0.0;
-#pragma unroll 4
-  for (long long q = threadIdx.x; q < n4; q += blockDim.x) {
-    T a[4], c[4];
-    ld4(x, p0 + q, a);
-    ld4(y, p0 + q, c);
-    acc_pack(acc, a, c);   // an FP32 pack is summed in FP32 first (pack.cuh)
-  }
-  for (long long e = e0 + 4 * n4 + threadIdx.x; e < e1; e += blockDim.x) acc += (double)x[e] * (double)y[e];
-  const double t = block_sum(acc);
-  if (threadIdx.x == 0) P[blockIdx.x] = t;
-}
-
 // ||C_i||^2 partials (C read through the instance pointer).
 __global__ void __launch_bounds__(256) k_b_normC(BDev d, double* __restrict__ P) {
   const int i = d.nb_inst[blockIdx.x];
   const BInst& in = d.inst[i];
   const long long l0 = d.nb_off[blockIdx.x];
-  const long long l1 = min(in.N, l0 + kChunk);
+  const long long l1 = min(in.N, l0 + d.chunk);
   double acc = 0.0;
   for (long long e = l0 + threadIdx.x; e < l1; e += blockDim.x) acc += in.C[e] * in.C[e];
   const double t = block_sum(acc);
   if (threadIdx.x == 0) P[blockIdx.x] = t;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_b_mgs(BDev d, T* __restrict__ W, const T* __restrict__ Vi,
-                                               const T* __restrict__ Vn, const double* __restrict__ Pin,
-                                               double* __restrict__ Pout, int irow, int jcol) {
+// Pass b of step j's sweep (gs_sweep.cuh), P[sum][block]: one basis vector per launch, each reading W, V_i and
+// V_i+1 and writing W, took 54 us (35 for the first product) where the batch's vectors have 12M FP32 entries;
+// a pass takes 58 us there for up to four vectors, 75 for up to eight.
+template <typename T, int VB>
+__global__ void __launch_bounds__(256) k_b_gs_pass(BDev d, T* __restrict__ W, const T* __restrict__ V, int j, int b,
+                                                   const double* __restrict__ Pin, double* __restrict__ Pout) {
   const int i = d.nb_inst[blockIdx.x];
   if (!d.act[i]) return;
   const BInst& in = d.inst[i];
-  const double h = inst_sum(Pin, in.nb0, in.nb1);
-  if (blockIdx.x == in.nb0 && threadIdx.x == 0) {
-    StLayout L{d.m};
-    d.state[i * d.stride + L.H() + irow + (long long)(d.m + 1) * jcol] = h;
-  }
-  const T hT = (T)h;
+  const GsPass g(j, b);
+  StLayout L{d.m};
+  double* st = d.state + i * d.stride;
+  T h[VB];
+  gs_coefficients<T, VB>(g, Pin, gridDim.x, in.nb0, in.nb1, st + L.gram(), st + L.H() + (long long)(d.m + 1) * j,
+                         blockIdx.x == in.nb0, h);
   const long long e0 = in.offN + d.nb_off[blockIdx.x];
-  const long long e1 = min(in.offN + in.N, e0 + kChunk);
-  const long long n4 = (e1 - e0) / 4, p0 = e0 / 4;
-  double acc = 0.0;
-#pragma unroll 4
-  for (long long q = threadIdx.x; q < n4; q += blockDim.x) {
-    T w[4], v[4], o[4];
-    ld4(W, p0 + q, w);
-    ld4(Vi, p0 + q, v);
-    if (Vn) ld4(Vn, p0 + q, o);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      w[t] = w[t] - hT * v[t];
-      if (!Vn) o[t] = w[t];
-    }
-    st4(W, p0 + q, w);
-    acc_pack(acc, o, w);
-  }
-  for (long long e = e0 + 4 * n4 + threadIdx.x; e < e1; e += blockDim.x) {
-    const T w = W[e] - hT * Vi[e];
-    W[e] = w;
-    acc += (double)(Vn ? Vn[e] : w) * (double)w;
-  }
-  const double t = block_sum(acc);
-  if (threadIdx.x == 0) Pout[blockIdx.x] = t;
+  const long long e1 = min(in.offN + in.N, e0 + d.chunk);
+  constexpr int PK = 16 / sizeof(T);
+  const long long np = (e1 - e0) / PK, tail = e0 + np * PK;
+  GsSums<T, VB> sums;
+  gs_stream<T, PK, VB>(g, W + e0, V + e0, d.totN, threadIdx.x, np, blockDim.x, h, sums);
+  if (tail < e1) gs_stream<T, 1, VB>(g, W + tail, V + tail, d.totN, threadIdx.x, e1 - tail, blockDim.x, h, sums);
+  gs_store<T, VB>(g, sums, Pout, gridDim.x, blockIdx.x);
 }
 
 template <typename T>
@@ -199,7 +167,7 @@ __global__ void __launch_bounds__(256) k_b_scale_W(BDev d, const T* __restrict__
   const BInst& in = d.inst[i];
   const T sc = (T)d.sc[16 * i + SC_INVH];
   const long long e0 = in.offN + d.nb_off[blockIdx.x];
-  const long long e1 = min(in.offN + in.N, e0 + kChunk);
+  const long long e1 = min(in.offN + in.N, e0 + d.chunk);
   for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) Vn[e] = W[e] * sc;
 }
 
@@ -216,7 +184,7 @@ __global__ void __launch_bounds__(256) k_b_axpy(BDev d, const T* __restrict__ V)
   for (int q = threadIdx.x; q < k; q += blockDim.x) ys[q] = (T)d.state[i * d.stride + L.y() + q];
   __syncthreads();
   const long long l0 = d.nb_off[blockIdx.x];
-  const long long l1 = min(in.N, l0 + kChunk);
+  const long long l1 = min(in.N, l0 + d.chunk);
   for (long long l = l0 + threadIdx.x; l < l1; l += blockDim.x) {
     T acc = 0;
     for (int q = 0; q < k; ++q) acc = fma_t(ys[q], V[(long long)q * d.totN + in.offN + l], acc);
@@ -536,8 +504,7 @@ void preload_cycle_kernels() {
       (const void*)k_b_ks_init, (const void*)k_b_scale_R<T>, (const void*)k_b_rfft<T, Real2, 0, 0>,
       (const void*)k_b_gemm<T, 0, 0>, (const void*)k_b_gemm<T, 0, 64>, (const void*)k_b_gemm<T, 0, 32>,
       (const void*)k_b_gemm<T, 0, 16>, (const void*)k_b_irfft<T, Real2, 0>,
-      (const void*)k_b_dot<T>,
-      (const void*)k_b_mgs<T>, (const void*)k_b_givens, (const void*)k_b_scale_W<T>, (const void*)k_b_solve_y,
+      (const void*)k_b_gs_pass<T, 4>, (const void*)k_b_gs_pass<T, 8>, (const void*)k_b_givens, (const void*)k_b_scale_W<T>, (const void*)k_b_solve_y,
       (const void*)k_b_axpy<T>, (const void*)k_b_rfft<double, double2, 1, 1>, (const void*)k_b_gemm<double, 1, 0>,
       (const void*)k_b_gemm<double, 1, 64>, (const void*)k_b_gemm<double, 1, 32>, (const void*)k_b_gemm<double, 1, 16>,
       (const void*)k_b_irfft<double, double2, 1>, (const void*)k_b_finalize_norm, (const void*)k_b_any_active};
@@ -549,7 +516,7 @@ struct BatchPlan {
   std::vector<int> nb_inst, tb_inst;
   std::vector<long long> nb_off, tb_off;
   bool tiny = false;   // CUDA-core products on 8 x 4 tiles (gemm_tiny_tile) instead of 64 x BN
-  long long totN = 0, totS = 0;
+  long long totN = 0, totS = 0, chunk = 0;
 };
 
 // The pieces of one restart cycle, each recorded on `st` and returning the kernels it launched:
@@ -595,13 +562,14 @@ struct CycleRecorder {
     kernels += inner_products(st);
     if (ev) TS_CUDA(cudaEventRecordWithFlags(ev[2 * j + 1], st, cudaEventRecordExternal));
     k_b_irfft<Real, Real2, 0><<<ntb, kTubes, 0, st>>>(d, Yh, W, nullptr);
-    k_b_dot<T><<<nbs, 256, 0, st>>>(d, basis(V, d.totN, 0), W, Pp[0]);
-    for (int i = 0; i <= j; ++i)
-      k_b_mgs<T><<<nbs, 256, 0, st>>>(d, W, basis(V, d.totN, i), i < j ? basis(V, d.totN, i + 1) : nullptr,
-                                      Pp[i & 1], Pp[(i + 1) & 1], i, j);
-    k_b_givens<<<d.count, 256, 0, st>>>(d, Pp[(j + 1) & 1], j);
+    const int nblk = j / kGB + 1;
+    for (int b = -1; b < nblk; ++b) {
+      if (j < 4) k_b_gs_pass<T, 4><<<nbs, 256, 0, st>>>(d, W, V, j, b, Pp[(b + 2) & 1], Pp[(b + 1) & 1]);
+      else k_b_gs_pass<T, 8><<<nbs, 256, 0, st>>>(d, W, V, j, b, Pp[(b + 2) & 1], Pp[(b + 1) & 1]);
+    }
+    k_b_givens<<<d.count, 256, 0, st>>>(d, Pp[nblk & 1], j);
     k_b_scale_W<T><<<nbs, 256, 0, st>>>(d, W, basis(V, d.totN, j + 1));
-    kernels += 5 + j + 1;
+    kernels += 5 + nblk;
     if (next) {
       k_b_any_active<<<1, 256, 0, st>>>(d, next);
       ++kernels;
@@ -656,6 +624,10 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   const int m = o.restart;
   BatchPlan plan;
   plan.inst.resize(count);
+  long long unknowns = 0;
+  for (int i = 0; i < count; ++i)
+    if (insts[i].op) unknowns += (long long)insts[i].op->n * insts[i].op->s * insts[i].op->p;
+  plan.chunk = stream_chunk(unknowns);
   for (int i = 0; i < count; ++i) {
     const ts_instance& u = insts[i];
     TS_REQUIRE(u.op && u.C && u.X, "ts_batched_solve: instance with a null pointer");
@@ -684,7 +656,7 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
     plan.totS += (long long)b.K * b.T;
     b.tol = u.tol > 0 ? u.tol : o.tol;
     b.nb0 = (int)plan.nb_inst.size();
-    for (long long l = 0; l < b.N; l += kChunk) {
+    for (long long l = 0; l < b.N; l += plan.chunk) {
       plan.nb_inst.push_back(i);
       plan.nb_off.push_back(l);
     }
@@ -782,8 +754,9 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   double2* Xh64 = mixed ? (double2*)get("b_Xh64", sizeof(double2) * (size_t)plan.totS) : (double2*)Xh;
   double2* Yh64 = mixed ? (double2*)get("b_Yh64", sizeof(double2) * (size_t)plan.totS) : (double2*)Yh;
   const size_t np = std::max(plan.nb_inst.size(), plan.tb_inst.size());
-  double* P0 = (double*)get("b_P0", sizeof(double) * np);
-  double* P1 = (double*)get("b_P1", sizeof(double) * np);
+  // P0, P1: the sums of a sweep's passes, [sum][streaming block]; P0 also holds plain partial sums
+  double* P0 = (double*)get("b_P0", sizeof(double) * std::max(np, kGsSums * plan.nb_inst.size()));
+  double* P1 = (double*)get("b_P1", sizeof(double) * std::max(np, kGsSums * plan.nb_inst.size()));
   double* Pt = (double*)get("b_Pt", sizeof(double) * np);
   double* sc = (double*)get("b_sc", sizeof(double) * 16 * count);
   int* flags = (int*)get("b_flags", sizeof(int) * 2 * count);
@@ -845,6 +818,7 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   d.count = count;
   d.m = m;
   d.totN = plan.totN;
+  d.chunk = plan.chunk;
   d.totS = plan.totS;
   d.nb_inst = d_nb_inst;
   d.nb_off = d_nb_off;

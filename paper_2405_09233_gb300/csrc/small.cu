@@ -9,22 +9,14 @@
 // matrix only needs a choice between rows c and c+1 at column c), also one column at a time: the
 // eliminations of the columns before k - 1 do not depend on k, and the last column has none; the estimate
 // is h_{k+1,k} |y_k| (Proposition 3.3), y_k = (right-hand side)_k / (last pivot).
-//
-// The Gram-Schmidt sweep takes kGB basis vectors at a time.  Modified Gram-Schmidt's coefficients against
-// V_b .. V_b+7 solve (I + L) h = d, d_i = <V_i, W> and L the strictly lower part of the block's Gram matrix
-// <V_i, V_l>: h_i = <V_i, W - sum_{l<i} h_l V_l> written out.  So one reduction gives eight coefficients where
-// a sweep vector by vector waits for eight, each behind the other; the Gram row of V_j (at most 7 more inner
-// products) is formed once, in step j, whose last block it completes.  The result is modified Gram-Schmidt's
-// up to rounding: against FP64 MGS, orthogonality and residuals are the same (see the tests).
 #include <algorithm>
 #include "internal.cuh"
 #include "reduce.cuh"
-#include "pack.cuh"
+#include "gs_sweep.cuh"
 
 namespace ts {
 namespace {
 
-constexpr int kGB = 8;         // basis vectors per block of the sweep
 constexpr int kMaxM = 256;     // longest restart
 
 // tFOM keeps its eliminated columns in R, the multipliers and row choices in cs and sn, its right-hand side in g.
@@ -206,16 +198,6 @@ __device__ __forceinline__ void ks_finish(const KsStage& S, double* st, int m, i
       if (end.gate) *end.gate = 0;
     }
   }
-}
-
-// One warp: lane r < nb holds d_r on entry and h_r on return; row is the lane's Gram row (l < its own r).
-__device__ __forceinline__ double gs_forward(double d, const double (&row)[kGB - 1], int nb, int lane) {
-#pragma unroll
-  for (int l = 0; l < kGB - 1; ++l) {
-    const double hl = __shfl_sync(0xffffffffu, d, l);
-    if (l + 1 < nb && lane > l && lane < nb) d = fma(-row[l], hl, d);
-  }
-  return d;
 }
 
 // Everything of inner step j after W = M(V_j), for vectors of at most kArnMaxN entries, in one launch of a
@@ -429,222 +411,22 @@ __global__ void __launch_bounds__(kArnThreads, 1)
 // V_i+1, writing W) above 65536 entries and one cluster launch per step below: FP64, 61440 entries 1877 ->
 // 542 us, 262144 1534 -> 745, 4.2M 8474 -> 5556; FP32, 1.05M 1944 -> 888, 16.8M 10303 -> 6427.  The line to
 // the cluster form lies where both take the same time (FP64, 8000 entries in the cluster 457 us, 8200 here 451).
-constexpr int kGsBlocks = 152, kGsSums = 2 * kGB;
+constexpr int kGsBlocks = 152;
 
-// v[0..NV-1] summed over the warp: lane's result is sum lane / (32 / NV); NV 4, 8 or 16.
-template <int NV>
-__device__ __forceinline__ double warp_reduce_scatter(double (&v)[NV], int lane) {
-  constexpr int LG = NV == 16 ? 4 : (NV == 8 ? 3 : 2);
-#pragma unroll
-  for (int r = 0; r < LG; ++r) {
-    const bool up = (lane & (16 >> r)) != 0;
-#pragma unroll
-    for (int i = 0; i < NV / 2; ++i) {
-      if (i < (NV >> (r + 1))) {
-        const int o = NV >> (r + 1);
-        const double send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16 >> r);
-      }
-    }
-  }
-  double x = v[0];
-#pragma unroll
-  for (int mask = 16 >> LG; mask > 0; mask >>= 1) x += __shfl_xor_sync(0xffffffffu, x, mask);
-  return x;
-}
-
-// One pack of a vector: four FP32 or two FP64 entries (one 16-byte access), or one entry.
-template <typename T, int PK>
-__device__ __forceinline__ void ld_pack(const T* p, long long e, T (&v)[PK]) {
-  if constexpr (PK == 1) v[0] = p[e];
-  else if constexpr (sizeof(T) == 4) {
-    const float4 q = reinterpret_cast<const float4*>(p)[e];
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-  } else {
-    const double2 q = reinterpret_cast<const double2*>(p)[e];
-    v[0] = q.x; v[1] = q.y;
-  }
-}
-template <typename T, int PK>
-__device__ __forceinline__ void st_pack(T* p, long long e, const T (&v)[PK]) {
-  if constexpr (PK == 1) p[e] = v[0];
-  else if constexpr (sizeof(T) == 4) reinterpret_cast<float4*>(p)[e] = make_float4(v[0], v[1], v[2], v[3]);
-  else reinterpret_cast<double2*>(p)[e] = make_double2(v[0], v[1]);
-}
-
-// VB: the most vectors of a block, 4 (the first steps; twice the packs in flight) or 8.
 template <typename T, int PK, int VB>
 __global__ void __launch_bounds__(512, 1)
     k_gs_pass(T* __restrict__ W, const T* __restrict__ V, long long ldv, long long NP, int j, int b,
               const double* __restrict__ Pin, double* __restrict__ Pout, double* st, int m, const int* gate) {
   if (gate && *gate == 0) return;
-  __shared__ double sd[kGsSums], sh[kGB], red[16][kGsSums];
-  const int t = threadIdx.x, lane = t & 31, wp = t >> 5, nw = blockDim.x >> 5;
-  const int nblk = j / kGB + 1;
-  const int nu = b >= 0 ? min(kGB, j + 1 - kGB * b) : 0;              // vectors subtracted
-  const int nd = b + 1 < nblk ? min(kGB, j + 1 - kGB * (b + 1)) : 0;  // vectors multiplied
-  const bool lastu = b + 1 == nblk, lastd = b + 2 == nblk;
+  const GsPass g(j, b);
+  Layout L{m};
   T h[VB];
-  if (nu) {
-    Layout L{m};
-    double* G = st + L.gram() + (size_t)(kGB * b) * kGB;
-    double row[kGB - 1];
-    if (wp == 0) {
-#pragma unroll
-      for (int l = 0; l < kGB - 1; ++l)   // rows of earlier steps; V_j's is among the sums
-        row[l] = lane < nu && l < lane && kGB * b + lane < j ? G[lane * kGB + l] : 0.0;
-    }
-    for (int q = wp; q < kGsSums; q += nw) {
-      if (!(q < kGB ? q < nu : (lastu && q - kGB < nu - 1))) continue;
-      double x = 0.0;
-      for (int c = lane; c < (int)gridDim.x; c += 32) x += Pin[q * kGsBlocks + c];
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
-      if (lane == 0) sd[q] = x;
-    }
-    __syncthreads();
-    if (wp == 0) {
-      double x = lane < nu ? sd[lane] : 0.0;
-      if (lastu && lane == nu - 1) {
-#pragma unroll
-        for (int l = 0; l < kGB - 1; ++l) row[l] = l < lane ? sd[kGB + l] : 0.0;
-        if (blockIdx.x == 0) {
-#pragma unroll
-          for (int l = 0; l < kGB - 1; ++l)
-            if (l < lane) G[lane * kGB + l] = row[l];
-        }
-      }
-      x = gs_forward(x, row, nu, lane);
-      if (lane < nu) {
-        sh[lane] = x;
-        if (blockIdx.x == 0) st[L.H() + kGB * b + lane + (size_t)(m + 1) * j] = x;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < VB; ++q) h[q] = q < nu ? (T)sh[q] : T(0);
-  }
-  const T *Vu = V + (long long)(kGB * max(b, 0)) * ldv, *Vd = V + (long long)(kGB * (b + 1)) * ldv;
-  // FP32 vectors: two packs (eight products) are summed in FP32 (pack.cuh), and such sums in pairs of FP32
-  // numbers with the rounding error of every addition kept (Knuth's two-sum), as exact as an FP64 sum here; a
-  // conversion and an FP64 addition per eight products took half of this kernel's time.
-  constexpr int UN = sizeof(T) == 4 ? 2 : 1, GR = VB == 4 ? 2 * UN : 1, NI = VB == 4 ? GR : UN;
-  double acc[2 * VB];
-  float hi[2 * VB], lo[2 * VB], f[2 * VB];
-#pragma unroll
-  for (int q = 0; q < 2 * VB; ++q) {
-    acc[q] = 0.0;
-    hi[q] = lo[q] = f[q] = 0.f;
-  }
-  const auto used = [&](int q) { return q < VB ? q < nd : (lastd && q - VB < nd - 1); };
-  const auto add_dot = [&](const T (&x)[PK], const T (&y)[PK], int q) {
-#pragma unroll
-    for (int c = 0; c < PK; ++c) {
-      if constexpr (sizeof(T) == 8) acc[q] = fma(x[c], y[c], acc[q]);
-      else f[q] = fmaf(x[c], y[c], f[q]);
-    }
-  };
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long p0 = (long long)blockIdx.x * blockDim.x + t; p0 < NP; p0 += NI * stride) {
-#pragma unroll
-    for (int u0 = 0; u0 < NI; u0 += GR) {
-      T w[GR][PK], v[VB][GR][PK];
-      bool in[GR];
-#pragma unroll
-      for (int u = 0; u < GR; ++u) {
-        in[u] = p0 + (u0 + u) * stride < NP;
-#pragma unroll
-        for (int c = 0; c < PK; ++c) w[u][c] = T(0);
-        if (in[u]) ld_pack<T, PK>(W, p0 + (u0 + u) * stride, w[u]);
-      }
-      const auto load = [&](const T* base, int count) {
-#pragma unroll
-        for (int q = 0; q < VB; ++q)
-#pragma unroll
-          for (int u = 0; u < GR; ++u) {
-#pragma unroll
-            for (int c = 0; c < PK; ++c) v[q][u][c] = T(0);
-            if (q < count && in[u]) ld_pack<T, PK>(base + q * ldv, p0 + (u0 + u) * stride, v[q][u]);
-          }
-      };
-      if (nu) {
-        load(Vu, nu);
-#pragma unroll
-        for (int u = 0; u < GR; ++u) {
-#pragma unroll
-          for (int q = 0; q < VB; ++q)
-            if (q < nu) {
-#pragma unroll
-              for (int c = 0; c < PK; ++c) w[u][c] = w[u][c] - h[q] * v[q][u][c];
-            }
-          if (in[u]) st_pack<T, PK>(W, p0 + (u0 + u) * stride, w[u]);
-        }
-      }
-      if (nd) load(Vd, nd);
-#pragma unroll
-      for (int u = 0; u < GR; ++u) {
-        if (nd) {
-          T vj[PK];   // V_j where the block holds it, for its Gram row (again, from L1)
-#pragma unroll
-          for (int c = 0; c < PK; ++c) vj[c] = T(0);
-          if (lastd && nd > 1 && in[u])
-            ld_pack<T, PK>(Vd + (long long)(nd - 1) * ldv, p0 + (u0 + u) * stride, vj);
-#pragma unroll
-          for (int q = 0; q < VB; ++q)
-            if (q < nd) add_dot(v[q][u], w[u], q);
-          if (lastd) {
-#pragma unroll
-            for (int q = 0; q < VB - 1; ++q)
-              if (q < nd - 1) add_dot(v[q][u], vj, VB + q);
-          }
-        } else {
-          add_dot(w[u], w[u], 0);
-        }
-        if constexpr (sizeof(T) == 4) {
-          if ((u0 + u) % UN == UN - 1) {
-            if (nd) {
-#pragma unroll
-              for (int q = 0; q < 2 * VB; ++q)
-                if (used(q)) {
-                  const float sum = hi[q] + f[q], g = sum - hi[q];
-                  lo[q] += (hi[q] - (sum - g)) + (f[q] - g);
-                  hi[q] = sum;
-                  f[q] = 0.f;
-                }
-            } else {
-              acc[0] += (double)f[0];   // no sum of squares beyond FP32's range
-              f[0] = 0.f;
-            }
-          }
-        }
-      }
-    }
-  }
-  if constexpr (sizeof(T) == 4) {
-#pragma unroll
-    for (int q = 0; q < 2 * VB; ++q) acc[q] += (double)hi[q] + (double)lo[q];
-  }
-  if (!nd) {
-    const double tot = block_sum(acc[0]);
-    if (t == 0) Pout[blockIdx.x] = tot;
-    return;
-  }
-  if (lastd) {
-    const double x = warp_reduce_scatter<2 * VB>(acc, lane);
-    if (lane % (16 / VB) == 0) red[wp][lane / (16 / VB)] = x;
-  } else {
-    double a[VB];
-#pragma unroll
-    for (int q = 0; q < VB; ++q) a[q] = acc[q];
-    const double x = warp_reduce_scatter<VB>(a, lane);
-    if (lane % (32 / VB) == 0) red[wp][lane / (32 / VB)] = x;
-  }
-  __syncthreads();
-  if (t < (lastd ? 2 * VB : VB)) {
-    double x = 0.0;
-    for (int q = 0; q < nw; ++q) x += red[q][t];
-    Pout[(t < VB ? t : kGB + t - VB) * kGsBlocks + blockIdx.x] = x;
-  }
+  gs_coefficients<T, VB>(g, Pin, kGsBlocks, 0, gridDim.x, st + L.gram(), st + L.H() + (size_t)(m + 1) * j,
+                         blockIdx.x == 0, h);
+  GsSums<T, VB> sums;
+  gs_stream<T, PK, VB>(g, W, V, ldv, (long long)blockIdx.x * blockDim.x + threadIdx.x, NP,
+                       (long long)gridDim.x * blockDim.x, h, sums);
+  gs_store<T, VB>(g, sums, Pout, kGsBlocks, blockIdx.x);
 }
 
 // h_{j+1,j} from the last pass's sums, V_{j+1} = W / h_{j+1,j}, and the column update (the last CTA).
