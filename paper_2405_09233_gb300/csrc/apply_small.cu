@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
   if constexpr (!POW2) {
-    for (int r = t; r < p; r += kSmThreads) direct_twiddle(r, p, tc[r], tsn[r]);
+    fill_roots(tc, tsn, p, t, kSmThreads);
     __syncthreads();
   }
 
@@ -111,24 +111,9 @@ __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
       rfft_reg<double, P>([&](int u) { return in ? src[u * T] : 0.0; },
                           [&](int k, double re, double im) { dst[k * step] = make_double2(re, im); });
     } else {
-      double x[P];
-#pragma unroll
-      for (int u = 0; u < P; ++u) x[u] = (in && u < p) ? src[u * T] : 0.0;
-#pragma unroll 1
-      for (int k = 0; k < K; ++k) {
-        double re = 0.0, im = 0.0;
-        int r = 0;
-#pragma unroll
-        for (int u = 0; u < P; ++u) {
-          if (u < p) {
-            re = fma(x[u], tc[r], re);
-            im = fma(-x[u], tsn[r], im);
-            r += k;
-            if (r >= p) r -= p;
-          }
-        }
-        dst[k * step] = make_double2(re, im);
-      }
+      rfft_direct<double, P>([&](int u) { return in ? src[u * T] : 0.0; },
+                             [&](int k, double re, double im) { dst[k * step] = make_double2(re, im); }, p, 0, 1,
+                             [&](int r) { return tc[r]; }, [&](int r) { return tsn[r]; });
     }
   }
   if constexpr (POW2) {   // for the inverse
@@ -217,7 +202,7 @@ __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
 double tube_ops(int p) {
   if (p <= 1) return 1.0;
   if ((p & (p - 1)) == 0) return p == 2 ? 2.0 : 2.5 * p * std::max(1.0, std::log2(p / 2.0)) - 1.0 * p;
-  return 2.0 * p * (p / 2 + 1);
+  return 2.0 * ((p - 1) / 2) * (p / 2 + 1) + p;
 }
 
 // Clocks of the busiest SM: its four sub-partitions issue an FP64 instruction of a warp in 64 clocks each.

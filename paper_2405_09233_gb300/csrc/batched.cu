@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kTubes) k_b_rfft(BDev d, const Real* __restric
   const int p = ins.p;
   __shared__ Real tc[64], tsn[64];
   if (p > 32 || (p & (p - 1)) != 0 || p == 1) {   // the direct sums' table (uniform over the block)
-    for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, tc[r], tsn[r]);
+    fill_roots(tc, tsn, p, threadIdx.x, blockDim.x);
     __syncthreads();
   }
   const long long e = d.tb_off[blockIdx.x] + threadIdx.x;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kTubes) k_b_irfft(BDev d, const Cplx* __restri
   const int p = ins.p;
   __shared__ Real tc[64], tsn[64];
   if (p > 32 || (p & (p - 1)) != 0 || p == 1) {   // the direct sums' table (uniform over the block)
-    for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, tc[r], tsn[r]);
+    fill_roots(tc, tsn, p, threadIdx.x, blockDim.x);
     __syncthreads();
   }
   const long long e = d.tb_off[blockIdx.x] + threadIdx.x;

@@ -41,13 +41,15 @@ __host__ __device__ constexpr double cos32(int r) {
 __host__ __device__ constexpr double sin32(int r) { return cos32(r + 24); }
 template <typename Real, int P>
 __host__ __device__ constexpr Real kIrfftScale() { return sizeof(Real) == 8 ? Real(1) : Real(1) / Real(P); }
-// The P-th roots for a direct sum over any p: cos and sin of 2 pi r / p.
+// Roots of unity for direct sums, cos and sin of 2 pi r / p for r < p, by threads t < nt of a block (a multiple
+// of 64).  Even warps take the cosines and odd ones the sines: one warp's sincospi is twice the chain of FP64
+// instructions (64 clocks each), and every block waits for it.
 template <typename Real>
-__device__ __forceinline__ void direct_twiddle(int r, int p, Real& c, Real& s) {
-  double sv, cv;
-  sincospi(2.0 * r / p, &sv, &cv);
-  c = (Real)cv;
-  s = (Real)sv;
+__device__ __forceinline__ void fill_roots(Real* c, Real* s, int p, int t, int nt) {
+  for (int r = (t >> 6) * 32 + (t & 31); r < p; r += nt / 2) {
+    if (t & 32) s[r] = (Real)sinpi(2.0 * r / p);
+    else c[r] = (Real)cospi(2.0 * r / p);
+  }
 }
 
 // a b + c d and a b - c d with the rounding written out: the second product is rounded, the first is not.
@@ -244,6 +246,81 @@ __device__ __forceinline__ void irfft_reg(Load load, Store store) {
     for (int t = 0; t < M; ++t) {
       store(2 * t, zr[t]);
       store(2 * t + 1, zi[t]);
+    }
+  }
+}
+
+// Direct DFT of p <= PMAX real samples, p any: the outputs k0, k0 + ks, ... of the p/2+1 non-redundant ones.
+// x_t and x_p-t meet the same cosine and opposite sines, so their sum and difference are formed once and a
+// multiply-add serves both: half of a term-by-term sum's.  c(r), s(r): cos and sin of 2 pi r / p.
+template <typename Real, int PMAX, typename Load, typename Store, typename Cos, typename Sin>
+__device__ __forceinline__ void rfft_direct(Load load, Store store, int p, int k0, int ks, Cos c, Sin s) {
+  constexpr int H = PMAX / 2;
+  const int K = p / 2 + 1, h = (p - 1) / 2;
+  Real sum[H + 1], dif[H + 1];
+  const Real x0 = load(0), xm = p % 2 == 0 ? load(p / 2) : Real(0);
+#pragma unroll
+  for (int t = 1; t <= H; ++t) {
+    const Real a = t <= h ? load(t) : Real(0), b = t <= h ? load(p - t) : Real(0);
+    sum[t] = a + b;
+    dif[t] = b - a;
+  }
+#pragma unroll 1
+  for (int k = k0; k < K; k += ks) {
+    Real re = k & 1 ? x0 - xm : x0 + xm, im = 0;
+    int r = 0;
+#pragma unroll
+    for (int t = 1; t <= H; ++t) {
+      if (t <= h) {
+        r += k;
+        if (r >= p) r -= p;
+        re = fma(sum[t], c(r), re);
+        im = fma(dif[t], s(r), im);
+      }
+    }
+    store(k, re, im);
+  }
+}
+
+// The inverse from p/2+1 coefficients, times p: the outputs t and p - t of t0 <= t < t0 + NO, t <= p/2.
+template <typename Real, int NO, typename Load, typename Store, typename Cos, typename Sin>
+__device__ __forceinline__ void irfft_direct(Load load, Store store, int p, int t0, Cos c, Sin s) {
+  const int K = p / 2 + 1, nyq = p % 2 == 0 ? p / 2 : -1;
+  Real a[NO], b[NO];
+#pragma unroll
+  for (int u = 0; u < NO; ++u) a[u] = b[u] = Real(0);
+  Real next_re, next_im;
+  load(0, next_re, next_im);
+  int r0 = 0;   // k t0 mod p
+#pragma unroll 1
+  for (int k = 0; k < K; ++k) {
+    const Real re = next_re, im = next_im;
+    if (k + 1 < K) load(k + 1, next_re, next_im);   // one coefficient ahead
+    const bool real = k == 0 || k == nyq;
+    const Real cr = real ? re : Real(2) * re, ci = real ? Real(0) : Real(2) * im;
+    int r = r0;
+#pragma unroll
+    for (int u = 0; u < NO; ++u) {
+      if (t0 + u < K) {
+        a[u] = fma(cr, c(r), a[u]);
+        b[u] = fma(ci, s(r), b[u]);
+        r += k;
+        if (r >= p) r -= p;
+      }
+    }
+    r0 += t0;
+    if (r0 >= p) r0 -= p;
+  }
+#pragma unroll
+  for (int u = 0; u < NO; ++u) {
+    const int t = t0 + u;
+    if (t < K) {
+      if (t == 0 || 2 * t == p) {
+        store(t, a[u]);
+      } else {
+        store(t, a[u] - b[u]);
+        store(p - t, a[u] + b[u]);
+      }
     }
   }
 }

@@ -553,146 +553,123 @@ __global__ void k_prep_B(const double2* __restrict__ Bh, OpT* __restrict__ re, O
   }
 }
 
-// Planar DFT along mode 3 of an FP32 tensor: X (n x s x p) -> planes [k][j][ldn] (column-major X_k).
-template <typename OpT, int PMAX>
-__global__ void __launch_bounds__(256) k_rfft_planar(const float* __restrict__ X, OpT* __restrict__ re,
-                                                     OpT* __restrict__ im, int n, int s, int p, int ldn,
-                                                     float* __restrict__ re_lo, float* __restrict__ im_lo) {
-  __shared__ float tc[PMAX], tsn[PMAX];
-  for (int r = threadIdx.x; r < p; r += blockDim.x) direct_twiddle(r, p, tc[r], tsn[r]);
-  __syncthreads();
-  const int K = p / 2 + 1;
-  const long long T = (long long)n * s;
-  const long long Tp = (long long)ldn * s;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < Tp; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e % ldn);
-    const long long j = e / ldn;
-    float x[PMAX];
-#pragma unroll
-    for (int t = 0; t < PMAX; ++t) x[t] = (t < p && i < n) ? X[t * T + j * n + i] : 0.f;
-#pragma unroll 1
-    for (int kk = 0; kk < K; ++kk) {
-      float a = 0.f, b = 0.f;
-      int r = 0;
-#pragma unroll
-      for (int t = 0; t < PMAX; ++t) {
-        if (t < p) {
-          a = fmaf(x[t], tc[r], a);
-          b = fmaf(-x[t], tsn[r], b);
-          r += kk;
-          if (r >= p) r -= p;
-        }
-      }
-      re[kk * Tp + e] = to_op<OpT>(a);
-      im[kk * Tp + e] = to_op<OpT>(b);
-      if (re_lo) {
-        re_lo[kk * Tp + e] = tf32_lo(a);
-        im_lo[kk * Tp + e] = tf32_lo(b);
-      }
-    }
-  }
-}
-
-// planes [k][j][ldn] (column-major X_k) -> planes [k][i][lds] (row-major X_k).
-// Power-of-two p: both planar layouts in one pass.  A CTA of 32 x 8 threads owns a tile of 32 rows
-// (i) x TJ columns (j) of tubes (TJ = 32, or 16 with the split-TF32 low parts); each thread runs
-// the register FFT of TJ / 8 tubes, writes the column-major planes [k][j][ldn] directly (coalesced
-// along i) and keeps the tile in shared memory, from which the row-major planes [k][i][lds] are
-// written coalesced along j.  Entries outside n x s are written as zeros in both layouts.  The
-// separate transpose re-read the column-major planes from memory (a third of the traffic of the
-// pair) and moved 64-byte rows.
-template <typename OpT, int P, bool SPLIT>
+// Planar DFT along mode 3 of an FP32 tensor X (n x s x p) into column-major planes [k][j][ldn] and row-major
+// planes [k][i][lds] of Re and Im, and with SPLIT the low parts v - tf32(v) of both, in one pass.  A CTA of
+// 32 x 8 threads owns a tile of 32 rows (i) x TJ columns (j) of tubes (TJ = 32, or 16 with low parts); each
+// thread transforms TJ / 8 tubes, writes the column-major planes directly (coalesced along i) and keeps the
+// tile in shared memory, from which the row-major planes are written coalesced along j.  Entries outside
+// n x s are written as zeros in both layouts.  A separate transpose re-reads the column-major planes from
+// memory (a third of the traffic of the pair) and moves 64-byte rows.
+// P is the tube length (register FFT, POW2) or a bound on p: then the sums run term by term, and where the
+// tiles are few the slices are shared out, slice k by the CTA with blockIdx.z = k mod gridDim.z.  Against a
+// transform and a transpose: 220 x 64 x 31 BF16 32.5 -> 11.3 us, 800 x 300 x 6 14.4 -> 9.1, 1000 x 300 x 12
+// 30.9 -> 23.1.
+template <typename OpT, int P, bool POW2, bool SPLIT>
 __global__ void __launch_bounds__(256) k_rfft_planar_fused(const float* __restrict__ X, OpT* __restrict__ cre,
                                                            OpT* __restrict__ cim, OpT* __restrict__ rre,
                                                            OpT* __restrict__ rim, float* __restrict__ cre_lo,
                                                            float* __restrict__ cim_lo, float* __restrict__ rre_lo,
-                                                           float* __restrict__ rim_lo, int n, int s, int ldn,
+                                                           float* __restrict__ rim_lo, int n, int s, int p, int ldn,
                                                            int lds) {
-  constexpr int K = P / 2 + 1, TJ = SPLIT ? 16 : 32, NQ = TJ / 8;
+  constexpr int TJ = SPLIT ? 16 : 32, NQ = TJ / 8;
+  const int K = (POW2 ? P : p) / 2 + 1, zs = POW2 ? 1 : gridDim.z, z = POW2 ? 0 : blockIdx.z;
+  const int Kz = POW2 ? K : (K - z + zs - 1) / zs;            // slices of this CTA: z + zs m, m < Kz
   extern __shared__ uint8_t pf_smem[];
-  OpT* tre = reinterpret_cast<OpT*>(pf_smem);             // [K][TJ][33]
-  OpT* tim = tre + K * TJ * 33;
-  float* tlr = reinterpret_cast<float*>(tim + K * TJ * 33);   // split: low parts, same shape
-  float* tli = tlr + (SPLIT ? K * TJ * 33 : 0);
+  OpT* tre = reinterpret_cast<OpT*>(pf_smem);             // [Kz][TJ][33]
+  OpT* tim = tre + Kz * TJ * 33;
+  float* tlr = reinterpret_cast<float*>(tim + Kz * TJ * 33);   // split: low parts, same shape
+  float* tli = tlr + (SPLIT ? Kz * TJ * 33 : 0);
+  __shared__ float2 tw[POW2 ? 1 : P];
+  if constexpr (!POW2) {
+    __shared__ float tc[P], tsn[P];
+    const int t = threadIdx.y * 32 + threadIdx.x;
+    fill_roots(tc, tsn, p, t, 256);
+    __syncthreads();
+    if (t < p) tw[t] = make_float2(tc[t], tsn[t]);
+    __syncthreads();
+  }
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * TJ;
   const long long T = (long long)n * s;
   const long long Tc = (long long)ldn * s, Tr = (long long)n * lds;
   const int i = i0 + tx;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const int jj = ty + 8 * q, j = j0 + jj;
-    const bool live = i < n && j < s;
-    rfft_reg<float, P>([&](int t) { return live ? X[t * T + (long long)j * n + i] : 0.f; },
-                       [&](int kk, float a, float b) {
-                         const OpT ha = to_op<OpT>(a), hb = to_op<OpT>(b);
-                         tre[(kk * TJ + jj) * 33 + tx] = ha;
-                         tim[(kk * TJ + jj) * 33 + tx] = hb;
-                         float la = 0.f, lb = 0.f;
-                         if constexpr (SPLIT) {
-                           la = tf32_lo(a);
-                           lb = tf32_lo(b);
-                           tlr[(kk * TJ + jj) * 33 + tx] = la;
-                           tli[(kk * TJ + jj) * 33 + tx] = lb;
-                         }
-                         if (j < s && i < ldn) {
-                           const long long o = kk * Tc + (long long)j * ldn + i;
-                           cre[o] = ha;
-                           cim[o] = hb;
-                           if constexpr (SPLIT) {
-                             cre_lo[o] = la;
-                             cim_lo[o] = lb;
-                           }
-                         }
-                       });
-  }
-  __syncthreads();
-  // row-major planes: rows i0 + r (r < 32), columns j0 + c (c < TJ), all K slices
-  for (int e = ty * 32 + tx; e < K * 32 * TJ; e += 256) {
-    const int c = e % TJ, r = (e / TJ) % 32, kk = e / (TJ * 32);
-    const int ir = i0 + r, jc = j0 + c;
-    if (ir < n && jc < lds) {
-      const long long o = kk * Tr + (long long)ir * lds + jc;
-      rre[o] = tre[(kk * TJ + c) * 33 + r];
-      rim[o] = tim[(kk * TJ + c) * 33 + r];
+  const auto load = [&](int jj, int t) {
+    const int j = j0 + jj;
+    return i < n && j < s ? X[t * T + (long long)j * n + i] : 0.f;
+  };
+  const auto store = [&](int jj, int m, float a, float b) {
+    const int j = j0 + jj;
+    const OpT ha = to_op<OpT>(a), hb = to_op<OpT>(b);
+    tre[(m * TJ + jj) * 33 + tx] = ha;
+    tim[(m * TJ + jj) * 33 + tx] = hb;
+    float la = 0.f, lb = 0.f;
+    if constexpr (SPLIT) {
+      la = tf32_lo(a);
+      lb = tf32_lo(b);
+      tlr[(m * TJ + jj) * 33 + tx] = la;
+      tli[(m * TJ + jj) * 33 + tx] = lb;
+    }
+    if (j < s && i < ldn) {
+      const long long o = (z + (long long)m * zs) * Tc + (long long)j * ldn + i;
+      cre[o] = ha;
+      cim[o] = hb;
       if constexpr (SPLIT) {
-        rre_lo[o] = tlr[(kk * TJ + c) * 33 + r];
-        rim_lo[o] = tli[(kk * TJ + c) * 33 + r];
+        cre_lo[o] = la;
+        cim_lo[o] = lb;
+      }
+    }
+  };
+  if constexpr (POW2) {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int jj = ty + 8 * q;
+      rfft_reg<float, P>([&](int t) { return load(jj, t); }, [&](int m, float a, float b) { store(jj, m, a, b); });
+    }
+  } else {
+#pragma unroll 1
+    for (int q = 0; q < NQ; q += 2) {   // two tubes per twiddle read
+      const int jj = ty + 8 * q;
+      float x[P], y[P];
+#pragma unroll
+      for (int t = 0; t < P; ++t) {
+        x[t] = t < p ? load(jj, t) : 0.f;
+        y[t] = t < p ? load(jj + 8, t) : 0.f;
+      }
+#pragma unroll 1
+      for (int m = 0; m < Kz; ++m) {
+        const int kk = z + zs * m;
+        float a = 0.f, b = 0.f, c = 0.f, d = 0.f;
+        int r = 0;
+#pragma unroll
+        for (int t = 0; t < P; ++t) {
+          if (t < p) {
+            const float2 w = tw[r];
+            a = fmaf(x[t], w.x, a);
+            b = fmaf(-x[t], w.y, b);
+            c = fmaf(y[t], w.x, c);
+            d = fmaf(-y[t], w.y, d);
+            r += kk;
+            if (r >= p) r -= p;
+          }
+        }
+        store(jj, m, a, b);
+        store(jj + 8, m, c, d);
       }
     }
   }
-}
-
-template <typename OpT, int P, bool SPLIT>
-constexpr int planar_fused_smem() {
-  constexpr int K = P / 2 + 1, TJ = SPLIT ? 16 : 32;
-  return K * TJ * 33 * (2 * (int)sizeof(OpT) + (SPLIT ? 8 : 0));
-}
-
-template <typename OpT>
-__global__ void k_transpose_planes(const OpT* __restrict__ cre, const OpT* __restrict__ cim, OpT* __restrict__ rre,
-                                   OpT* __restrict__ rim, int n, int s, int ldn, int lds) {
-  __shared__ OpT tr[32][33], ti[32][33];
-  const int k = blockIdx.z, i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-  const OpT* cr = cre + (long long)k * s * ldn;
-  const OpT* ci = cim + (long long)k * s * ldn;
-  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
-    const int j = j0 + q, i = i0 + threadIdx.x;
-    OpT a = to_op<OpT>(0.f), b = to_op<OpT>(0.f);
-    if (j < s && i < n) {
-      a = cr[(long long)j * ldn + i];
-      b = ci[(long long)j * ldn + i];
-    }
-    tr[q][threadIdx.x] = a;
-    ti[q][threadIdx.x] = b;
-  }
   __syncthreads();
-  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
-    const int i = i0 + q, j = j0 + threadIdx.x;
-    if (i < n && j < lds) {
-      const long long o = (long long)k * n * lds + (long long)i * lds + j;
-      rre[o] = j < s ? tr[threadIdx.x][q] : to_op<OpT>(0.f);
-      rim[o] = j < s ? ti[threadIdx.x][q] : to_op<OpT>(0.f);
+  // row-major planes: rows i0 + r (r < 32), columns j0 + c (c < TJ), this CTA's slices
+  for (int e = ty * 32 + tx; e < Kz * 32 * TJ; e += 256) {
+    const int c = e % TJ, r = (e / TJ) % 32, m = e / (TJ * 32);
+    const int ir = i0 + r, jc = j0 + c;
+    if (ir < n && jc < lds) {
+      const long long o = (z + (long long)m * zs) * Tr + (long long)ir * lds + jc;
+      rre[o] = tre[(m * TJ + c) * 33 + r];
+      rim[o] = tim[(m * TJ + c) * 33 + r];
+      if constexpr (SPLIT) {
+        rre_lo[o] = tlr[(m * TJ + c) * 33 + r];
+        rim_lo[o] = tli[(m * TJ + c) * 33 + r];
+      }
     }
   }
 }
@@ -730,57 +707,39 @@ void prepare_operator(ts_op* op, TcOperands& t, cudaStream_t st) {
   TS_CUDA(cudaGetLastError());
 }
 
-template <typename OpT, int P, bool SPLIT>
-void planar_fused_p(const float* X, TcWork& w, int n, int s, int ldn, int lds, cudaStream_t st) {
-  constexpr int smem = planar_fused_smem<OpT, P, SPLIT>(), TJ = SPLIT ? 16 : 32;
-  set_max_dynamic_smem((const void*)k_rfft_planar_fused<OpT, P, SPLIT>, smem);
-  const dim3 grid((unsigned)((std::max(n, ldn) + 31) / 32), (unsigned)((std::max(s, lds) + TJ - 1) / TJ), 1);
-  k_rfft_planar_fused<OpT, P, SPLIT><<<grid, dim3(32, 8), smem, st>>>(
+template <typename OpT, int P, bool POW2, bool SPLIT>
+void planar_fused_p(const float* X, TcWork& w, int n, int s, int p, int ldn, int lds, cudaStream_t st) {
+  constexpr int TJ = SPLIT ? 16 : 32;
+  const unsigned gx = (unsigned)((std::max(n, ldn) + 31) / 32), gy = (unsigned)((std::max(s, lds) + TJ - 1) / TJ);
+  // direct sums: two CTAs per SM while there are slices to share out
+  const int K = p / 2 + 1, zs = POW2 ? 1 : (int)std::max(1ull, std::min<unsigned long long>(K, 304ull / ((unsigned long long)gx * gy)));
+  const int per = TJ * 33 * (2 * (int)sizeof(OpT) + (SPLIT ? 8 : 0));
+  set_max_dynamic_smem((const void*)k_rfft_planar_fused<OpT, P, POW2, SPLIT>, (P / 2 + 1) * per);
+  k_rfft_planar_fused<OpT, P, POW2, SPLIT><<<dim3(gx, gy, zs), dim3(32, 8), (K + zs - 1) / zs * per, st>>>(
       X, (OpT*)w.xc_re, (OpT*)w.xc_im, (OpT*)w.xr_re, (OpT*)w.xr_im, (float*)w.xc_re_lo, (float*)w.xc_im_lo,
-      (float*)w.xr_re_lo, (float*)w.xr_im_lo, n, s, ldn, lds);
+      (float*)w.xr_re_lo, (float*)w.xr_im_lo, n, s, p, ldn, lds);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }
 
 template <typename OpT, bool SPLIT>
 void planar_fused(const float* X, TcWork& w, int n, int s, int p, int ldn, int lds, cudaStream_t st) {
-  if (p == 2) planar_fused_p<OpT, 2, SPLIT>(X, w, n, s, ldn, lds, st);
-  else if (p == 4) planar_fused_p<OpT, 4, SPLIT>(X, w, n, s, ldn, lds, st);
-  else if (p == 8) planar_fused_p<OpT, 8, SPLIT>(X, w, n, s, ldn, lds, st);
-  else if (p == 16) planar_fused_p<OpT, 16, SPLIT>(X, w, n, s, ldn, lds, st);
-  else planar_fused_p<OpT, 32, SPLIT>(X, w, n, s, ldn, lds, st);
+  if (p == 2) planar_fused_p<OpT, 2, true, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p == 4) planar_fused_p<OpT, 4, true, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p == 8) planar_fused_p<OpT, 8, true, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p == 16) planar_fused_p<OpT, 16, true, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p == 32) planar_fused_p<OpT, 32, true, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p <= 4) planar_fused_p<OpT, 4, false, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p <= 8) planar_fused_p<OpT, 8, false, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p <= 16) planar_fused_p<OpT, 16, false, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else if (p <= 32) planar_fused_p<OpT, 32, false, SPLIT>(X, w, n, s, p, ldn, lds, st);
+  else throw Error{TS_ERR_UNSUPPORTED, "tensor-core path supports p <= 32"};
 }
 
 template <typename OpT>
 void planar_dft(const float* X, TcWork& w, int n, int s, int p, int ldn, int lds, cudaStream_t st) {
-  const long long Tp = (long long)ldn * s;
-  int g = (int)((Tp + 255) / 256);
-  if (g > 152 * 16) g = 152 * 16;
-  OpT* cre = (OpT*)w.xc_re; OpT* cim = (OpT*)w.xc_im;
-  float* lre = (float*)w.xc_re_lo; float* lim = (float*)w.xc_im_lo;
-  if (p == 2 || p == 4 || p == 8 || p == 16 || p == 32) {   // both layouts in one pass
-    if (lre) planar_fused<OpT, true>(X, w, n, s, p, ldn, lds, st);
-    else planar_fused<OpT, false>(X, w, n, s, p, ldn, lds, st);
-    return;
-  }
-  if (p <= 4) k_rfft_planar<OpT, 4><<<g, 256, 0, st>>>(X, cre, cim, n, s, p, ldn, lre, lim);
-  else if (p <= 8) k_rfft_planar<OpT, 8><<<g, 256, 0, st>>>(X, cre, cim, n, s, p, ldn, lre, lim);
-  else if (p <= 16) k_rfft_planar<OpT, 16><<<g, 256, 0, st>>>(X, cre, cim, n, s, p, ldn, lre, lim);
-  else if (p <= 32) k_rfft_planar<OpT, 32><<<g, 256, 0, st>>>(X, cre, cim, n, s, p, ldn, lre, lim);
-  else throw Error{TS_ERR_UNSUPPORTED, "tensor-core path supports p <= 32"};
-  count_launch();
-  TS_CUDA(cudaGetLastError());
-  const int K = p / 2 + 1;
-  const dim3 tg((n + 31) / 32, (lds + 31) / 32, K);
-  k_transpose_planes<OpT><<<tg, dim3(32, 8), 0, st>>>(cre, cim, (OpT*)w.xr_re, (OpT*)w.xr_im, n, s, ldn, lds);
-  count_launch();
-  TS_CUDA(cudaGetLastError());
-  if (lre) {
-    k_transpose_planes<float><<<tg, dim3(32, 8), 0, st>>>(lre, lim, (float*)w.xr_re_lo, (float*)w.xr_im_lo, n, s,
-                                                            ldn, lds);
-    count_launch();
-    TS_CUDA(cudaGetLastError());
-  }
+  if (w.xc_re_lo) planar_fused<OpT, true>(X, w, n, s, p, ldn, lds, st);
+  else planar_fused<OpT, false>(X, w, n, s, p, ldn, lds, st);
 }
 
 template <int PARTS>
