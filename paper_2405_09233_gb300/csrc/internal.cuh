@@ -240,6 +240,7 @@ void ks_solve(void* state, int m, int k, cudaStream_t st);
 // <= stop[1]); gate (device, may be null): the kernels do nothing when *gate == 0, and *gate is set to 0
 // under the same conditions (stop must then be given).
 size_t arnoldi_scratch_bytes();
+template <typename T> void arnoldi_load();   // before a capture: loads the kernels of every step
 template <typename T>
 void arnoldi_step(T* W, T* V, long long ldv, long long N, int j, int m, void* state, int method, double* scratch,
                   cudaStream_t st, cudaGraphConditionalHandle handle = 0, const double* stop = nullptr,

@@ -567,6 +567,20 @@ void launch_gs(T* W, T* V, long long ldv, long long NP, int j, int m, double* s,
   count_launch();
 }
 
+// Every kernel a step of any j may launch is loaded: a capture cannot load one on its first launch.
+template <typename T>
+void arnoldi_load() {
+  cudaFuncAttributes fa;
+  constexpr int PK = 16 / sizeof(T);
+  const void* fns[] = {(const void*)k_arnoldi_cluster<T>,  (const void*)k_gs_pass<T, PK, 4>,
+                       (const void*)k_gs_pass<T, PK, 8>,   (const void*)k_gs_pass<T, 1, 4>,
+                       (const void*)k_gs_pass<T, 1, 8>,    (const void*)k_gs_finish<T, PK>,
+                       (const void*)k_gs_finish<T, 1>};
+  for (const void* f : fns) TS_CUDA(cudaFuncGetAttributes(&fa, f));
+}
+template void arnoldi_load<double>();
+template void arnoldi_load<float>();
+
 size_t arnoldi_scratch_bytes() { return sizeof(double) * 2 * kGsSums * kGsBlocks; }
 
 template <typename T>
@@ -591,7 +605,8 @@ template void arnoldi_step<float>(float*, float*, long long, long long, int, int
                                   cudaGraphConditionalHandle, const double*, int*);
 
 void ks_solve(void* state, int m, int k, cudaStream_t st) {
-  TS_REQUIRE(k >= 1 && k <= kMaxM, "ks_solve: bad size");
+  TS_REQUIRE(k <= kMaxM, "ks_solve: bad size");
+  if (k <= 0) return;
   k_ks_solve<<<1, (k + 31) / 32 * 32, 0, st>>>(static_cast<double*>(state), m, k);
   count_launch();
   TS_CUDA(cudaGetLastError());

@@ -229,6 +229,7 @@ ts_status krylov_solve(ts_ctx* ctx, ts_op* op, const double* C, double* X, const
     // legacy default stream), ordered after the caller's stream by an event
     if (!ctx->bstream) TS_CUDA(cudaStreamCreateWithFlags(&ctx->bstream, cudaStreamNonBlocking));
     TS_CUDA(cudaStreamSynchronize(st));
+    arnoldi_load<T>();   // steps beyond those of the first cycle may run kernels it did not
     cg.reset(new CycleGraph());
     const cudaStream_t gst = ctx->bstream;
     const long long launches0 = g_launches.load();
