@@ -131,7 +131,9 @@ def slice_flops(n, s, p, per_complex):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the dominant kernels at the
 # n = s = 1024, p = 16 workload, from one ncu capture each of the kernels as they stand; a roofline object
 # carries them only for that workload and, for the emulated product, only when every launch used 6 digits.
-TRAFFIC_N1024 = {"k_gemm_slices<double>": 502828800 + 137370112, "k_oz_sylv/6": 1566623488 + 140020736}
+# (k_gemm_slices<double> and k_oz_sylv/6 are the forms before these.)
+TRAFFIC_N1024 = {"k_gemm_f64": 484737024 + 139066624, "k_oz_sylv/6 resident": 1259727616 + 127081728,
+                 "k_gemm_slices<double>": 502828800 + 137370112, "k_oz_sylv/6": 1566623488 + 140020736}
 
 
 def traffic_for(kernel, workload):
@@ -170,7 +172,7 @@ def fp64_gemm_roofline(executed_per_launch, conventional_per_launch, avg_ms, sha
         note += f". cuBLAS DGEMM (8192^3, torch) in this run: {dgemm_tflops:.3f} TFLOP/s"
     note += probe_note(probe_tflops)
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": None, "kernel": "k_gemm_slices<double> (FP64 DFMA, 3-multiply complex)", "note": note,
+            "traffic": None, "kernel": "k_gemm_f64 (FP64 DFMA, 3-multiply complex)", "note": note,
             "peak_probe": probe_tflops}
 
 
@@ -194,7 +196,7 @@ def lowp_gemm_roofline(precision, flops_per_launch, avg_ms, sustained, share, sm
     if precision == "mixed_fp32":
         peak = ffma_peak_tflops(sms, mhz)
         return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "kernel": "k_gemm_slices<float> (FP32 FFMA)",
+                "traffic": None, "kernel": "k_gemm_f32 (FP32 FFMA)",
                 "note": f"peak derived: 2 FLOP x 128 lanes/SM x {sms} SMs x {mhz:.0f} MHz. Kernel share: {share:.3f}"}
     bf = pk["bf16_sustained"] if sustained else pk["bf16_burst"]
     tf32 = precision in ("mixed_tf32", "mixed_tf32x3")
@@ -224,13 +226,13 @@ def stats_rooflines(st, n, s, p, total_ms, sustained, precision, sms, mhz, workl
         r = fp64_gemm_roofline(executed, conv, st.gemm_ms / st.gemm_launches, st.gemm_ms / total_ms, sms, mhz, dgemm,
                                probe)
         if not batched:
-            r["traffic"] = traffic_for("k_gemm_slices<double>", workload)
+            r["traffic"] = traffic_for("k_gemm_f64", workload)
         out.append((st.gemm_ms, r))
     if st.oz_launches:
         r = ozaki_roofline(st.oz_flops / st.oz_launches, st.oz_pair_flops / st.oz_launches,
                            st.oz_ms / st.oz_launches, sustained, st.oz_ms / total_ms)
         if not batched and abs(st.oz_pair_flops - 21 * st.oz_flops) <= 1e-9 * st.oz_pair_flops:
-            r["traffic"] = traffic_for("k_oz_sylv/6", workload)
+            r["traffic"] = traffic_for("k_oz_sylv/6 resident", workload)
         out.append((st.oz_ms, r))
     if st.lowp_launches and precision != "fp64":
         r = lowp_gemm_roofline(precision, st.lowp_flops / st.lowp_launches, st.lowp_ms / st.lowp_launches,
