@@ -264,18 +264,44 @@ __global__ void __launch_bounds__(192, 1)
   tc_sylv_tile<BN, ESZ, PARTS>(maps[it.x], b.Y, b.n, b.s, b.nyq, it.y, it.z, it.w, err, 0, kWaitNs);
 }
 
-// Persistent batched form: gridDim.x CTAs (at most one per SM) walk the cost-sorted work list with
-// stride gridDim.x, skipping instances outside the current inner cycle.  Barriers are initialised
-// and tensor memory is allocated once per CTA; the TMA / MMA stage ring runs on from one item to the
-// next (one stage counter for the whole walk), and two accumulator sets in tensor memory let the
-// epilogue of item t drain while item t + 1 is multiplied (acc_full / acc_empty barriers per set).
-// Per item the MMAs and their order are those of k_b_tc, so both give bitwise the same products.
+// Persistent form: gridDim.x CTAs (at most one per SM) walk the work items with stride gridDim.x.  Barriers are
+// initialised and tensor memory is allocated once per CTA; the TMA / MMA stage ring runs on from one item to the
+// next (one stage counter for the whole walk), and two accumulator sets in tensor memory let the epilogue of item
+// t drain while item t + 1 is multiplied (acc_full / acc_empty barriers per set).  Per item the MMAs and their
+// order are those of tc_sylv_tile, so both give bitwise the same products.
 // Every wait is bounded; after an expired wait each role stops where it is, the producer waits for
 // the stages it loaded, the MMA warp for the MMAs it issued, and tensor memory is freed.
-template <int BN, int ESZ, int PARTS>
-__global__ void __launch_bounds__(192, 1)
-    k_b_tc_persist(const TcMaps* __restrict__ maps, const BTcInst* __restrict__ inst, const int* __restrict__ active,
-                   const int4* __restrict__ items, int nitems, int* err) {
+struct TcItem {
+  const TcMaps* m;   // null: nothing to do
+  float2* Y;
+  int n, s, nyq, k, i0, j0;
+};
+// A batch's cost-sorted list, without the instances outside the current inner cycle.
+struct BatchItems {
+  const TcMaps* maps;
+  const BTcInst* inst;
+  const int* active;
+  const int4* items;
+  __device__ __forceinline__ TcItem get(int q) const {
+    const int4 it = items[q];
+    const BTcInst& b = inst[it.x];
+    return TcItem{active[it.x] ? maps + it.x : nullptr, b.Y, b.n, b.s, b.nyq, it.y, it.z, it.w};
+  }
+};
+// One operator's tiles, column tiles fastest (they share the A tile in L2), the slices that cost a quarter last.
+template <int BN>
+struct GridItems {
+  const TcMaps* maps;
+  float2* Y;
+  int n, s, nyq, K, ni, nj;
+  __device__ __forceinline__ TcItem get(int q) const {
+    const int slice = q / (ni * nj), t = q - slice * (ni * nj), nc = K - 1 - (nyq > 0 ? 1 : 0);
+    const int k = slice < nc ? slice + 1 : (slice == nc ? 0 : nyq);
+    return TcItem{maps, Y, n, s, nyq, k, (t / nj) * kTileM, (t % nj) * BN};
+  }
+};
+template <int BN, int ESZ, int PARTS, typename Items>
+__device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* err) {
   using Cfg = TcCfg<BN, ESZ>;
   constexpr int kCols = 2 * Cfg::kTmemCols;   // two accumulator sets of (Re, Im)
   static_assert(kCols <= 512, "tensor memory");
@@ -312,7 +338,7 @@ __global__ void __launch_bounds__(192, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  auto iters_of = [&](const BTcInst& b) {
+  auto iters_of = [&](const TcItem& b) {
     return PARTS * ((b.n + Cfg::kElemsK - 1) / Cfg::kElemsK + (b.s + Cfg::kElemsK - 1) / Cfg::kElemsK);
   };
 
@@ -321,11 +347,10 @@ __global__ void __launch_bounds__(192, 1)
       long long g = 0, issued = 0;   // stages walked / whose loads were issued
       bool ok = true;
       for (int q = blockIdx.x; q < nitems && ok; q += gridDim.x) {
-        const int4 it = items[q];
-        if (!active[it.x]) continue;
-        const BTcInst& b = inst[it.x];
-        const TcMaps& m = maps[it.x];
-        const int k = it.y, i0 = it.z, j0 = it.w;
+        const TcItem b = src.get(q);
+        if (!b.m) continue;
+        const TcMaps& m = *b.m;
+        const int k = b.k, i0 = b.i0, j0 = b.j0;
         const bool real = (k == 0) || (k == b.nyq);
         const int it1 = (b.n + Cfg::kElemsK - 1) / Cfg::kElemsK, iters = iters_of(b);
         for (int u = 0; u < iters; ++u, ++g) {
@@ -373,10 +398,9 @@ __global__ void __launch_bounds__(192, 1)
     int t = 0;   // items multiplied by this CTA
     bool ok = true;
     for (int q = blockIdx.x; q < nitems && ok; q += gridDim.x) {
-      const int4 it = items[q];
-      if (!active[it.x]) continue;
-      const BTcInst& b = inst[it.x];
-      const bool real = (it.y == 0) || (it.y == b.nyq);
+      const TcItem b = src.get(q);
+      if (!b.m) continue;
+      const bool real = (b.k == 0) || (b.k == b.nyq);
       const int it1 = (b.n + Cfg::kElemsK - 1) / Cfg::kElemsK, iters = iters_of(b);
       const int set = t & 1;
       // the epilogue has drained this accumulator set's previous item (t - 2)
@@ -409,10 +433,9 @@ __global__ void __launch_bounds__(192, 1)
     // Epilogue: warp w reads TMEM lanes 32w..32w+31 (= output rows i0 + 32w + lane) of set t & 1.
     int t = 0;
     for (int q = blockIdx.x; q < nitems; q += gridDim.x) {
-      const int4 it = items[q];
-      if (!active[it.x]) continue;
-      const BTcInst& b = inst[it.x];
-      const int k = it.y, i0 = it.z, j0 = it.w;
+      const TcItem b = src.get(q);
+      if (!b.m) continue;
+      const int k = b.k, i0 = b.i0, j0 = b.j0;
       const bool real = (k == 0) || (k == b.nyq);
       const int set = t & 1;
       if (!mbar_wait(bar_accf + 8 * set, (uint32_t)(t >> 1) & 1u, err, 3)) break;
@@ -450,6 +473,19 @@ __global__ void __launch_bounds__(192, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
   }
+}
+
+template <int BN, int ESZ, int PARTS>
+__global__ void __launch_bounds__(192, 1)
+    k_b_tc_persist(const TcMaps* __restrict__ maps, const BTcInst* __restrict__ inst, const int* __restrict__ active,
+                   const int4* __restrict__ items, int nitems, int* err) {
+  tc_persist<BN, ESZ, PARTS>(BatchItems{maps, inst, active, items}, nitems, err);
+}
+template <int BN, int ESZ, int PARTS>
+__global__ void __launch_bounds__(192, 1)
+    k_tc_persist(const __grid_constant__ TcMaps maps, float2* __restrict__ Y, int n, int s, int K, int nyq, int ni,
+                 int nj, int* err) {
+  tc_persist<BN, ESZ, PARTS>(GridItems<BN>{&maps, Y, n, s, nyq, K, ni, nj}, ni * nj * K, err);
 }
 
 // Planar copies of the FP32 spectra of a batch: per (instance, slice, 32 x 32 tile) work item,
@@ -679,10 +715,36 @@ __global__ void __launch_bounds__(256) k_rfft_planar_fused(const float* __restri
 // ------------------------------------------------------------------------------------------------
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+int device_sms() {
+  static int cached[64] = {0};
+  int dev = 0;
+  TS_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return 152;
+  if (!cached[dev]) TS_CUDA(cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev));
+  return cached[dev];
+}
+
 template <int BN, int ESZ, int PARTS>
 void launch_tc(const TcMaps& maps, float2* Y, int n, int s, int K, int nyq, int* err, int stall,
                unsigned long long wait_ns, cudaStream_t st) {
   using Cfg = TcCfg<BN, ESZ>;
+  const long long ni = (n + kTileM - 1) / kTileM, nj = (s + BN - 1) / BN;
+  // More tiles than SMs: the persistent form, whose epilogues run under the next tile's products, while a tile is
+  // short enough for that to count: at n = s = 1024, p = 16 32 stages (BF16) 92.9 -> 80.8 us, 64 (TF32) 159.7 ->
+  // 146.9, 192 (split TF32) 413 -> 400; at n = 4096, s = 256, p = 32 136 (TF32) 653 / 655, 408 (split TF32)
+  // 1729 / 1789.  (BN = 256 leaves no tensor memory for a second accumulator set.)
+  const long long stages =
+      PARTS * ((n + Cfg::kElemsK - 1) / Cfg::kElemsK + (long long)(s + Cfg::kElemsK - 1) / Cfg::kElemsK);
+  if constexpr (BN <= 128) {
+    const int sms = device_sms();
+    if (!stall && stages <= 256 && ni * nj * K > sms && ni * nj * K <= INT32_MAX) {
+      set_max_dynamic_smem((const void*)k_tc_persist<BN, ESZ, PARTS>, Cfg::kSmem);
+      k_tc_persist<BN, ESZ, PARTS><<<sms, 192, Cfg::kSmem, st>>>(maps, Y, n, s, K, nyq, (int)ni, (int)nj, err);
+      count_launch();
+      TS_CUDA(cudaGetLastError());
+      return;
+    }
+  }
   set_max_dynamic_smem((const void*)k_tc_sylv<BN, ESZ, PARTS>, Cfg::kSmem);
   dim3 grid((s + BN - 1) / BN, (n + kTileM - 1) / kTileM, K);
   k_tc_sylv<BN, ESZ, PARTS><<<grid, 192, Cfg::kSmem, st>>>(maps, Y, n, s, nyq, err, stall, wait_ns);
@@ -907,15 +969,6 @@ void batch_preload_bn() {
   set_max_dynamic_smem((const void*)k_b_tc<BN, ESZ, PARTS>, Cfg::kSmem);
   TS_CUDA(cudaFuncGetAttributes(&fa, (const void*)k_b_tc_persist<BN, ESZ, PARTS>));
   set_max_dynamic_smem((const void*)k_b_tc_persist<BN, ESZ, PARTS>, Cfg::kSmem);
-}
-
-int device_sms() {
-  static int cached[64] = {0};
-  int dev = 0;
-  TS_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return 152;
-  if (!cached[dev]) TS_CUDA(cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev));
-  return cached[dev];
 }
 
 template <typename OpT, int ESZ, int PARTS, bool SPLIT>
