@@ -60,6 +60,7 @@ struct SmallLayout {
 // P: the tube length when POW2, else a bound on it (direct DFT of a.p <= P samples in registers).
 template <int P, bool POW2, int TN>
 __global__ void __launch_bounds__(kSmThreads) k_apply_small(SmallApply a) {
+  step_kernel_begin();
   if (a.gate && *a.gate == 0) return;   // a cycle that already ended (launched ahead)
   extern __shared__ double2 sm[];
   const int n = a.n, s = a.s, K = a.K, p = POW2 ? P : a.p;
@@ -233,7 +234,7 @@ void launch(const SmallApply& a, int tn, cudaStream_t st) {
   const unsigned tiles = (unsigned)a.mtiles * ((a.s + tn - 1) / tn);
   auto go = [&](auto kernel) {
     if (smem > 48 * 1024) set_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
-    kernel<<<tiles, kSmThreads, smem, st>>>(a);
+    launch_step_kernel(kernel, a.gate != nullptr, tiles, kSmThreads, smem, 0, st, a);
   };
   if (tn == 2) go(k_apply_small<P, POW2, 2>);
   else go(k_apply_small<P, POW2, 4>);

@@ -166,6 +166,41 @@ inline int num_slices(int p) { return p / 2 + 1; }
 // Memory-kind helper: true for device (or managed) memory of the current device, false for host
 // memory; throws TS_ERR_ARG for memory of another device, which a kernel here must not be given.
 bool is_device_ptr(const void* p);
+// Launched-ahead steps are chains of kernels of a few microseconds.  With `overlap` a kernel is brought up while
+// its predecessor in the stream still runs: its CTAs start and wait in step_kernel_begin until the predecessor
+// has completed and its writes are visible.  Every kernel launched so calls step_kernel_begin first (it does
+// nothing in a plain launch); it also lets the next kernel come up.  24 x 24 x 4, 18 steps of two kernels:
+// 668 -> 587 us.
+__device__ __forceinline__ void step_kernel_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... Params, typename... Args>
+void launch_step_kernel(void (*kernel)(Params...), bool overlap, unsigned grid, unsigned block, size_t smem, int cluster,
+                        cudaStream_t st, Args... args) {
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 0;
+  if (cluster > 0) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
+  if (overlap) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
+  }
+  TS_CUDA(cudaLaunchKernelEx(&cfg, kernel, Params(args)...));
+}
+
 // Raise a kernel's dynamic shared-memory limit to `bytes` on the current device (once per kernel and
 // device; thread-safe).
 void set_max_dynamic_smem(const void* func, int bytes);

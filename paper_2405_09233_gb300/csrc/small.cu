@@ -237,6 +237,7 @@ template <typename T>
 __global__ void __launch_bounds__(kArnThreads, 1)
     k_arnoldi_cluster(const T* __restrict__ W, T* __restrict__ V, long long ldv, int N, int j, int m, double* st,
                       int method, StepEnd end) {
+  step_kernel_begin();
   if (end.gate && *end.gate == 0) return;   // launched ahead of a cycle that has already ended (all CTAs alike)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double slots[2][kArnCL * 2 * kGB];
@@ -417,6 +418,7 @@ template <typename T, int PK, int VB>
 __global__ void __launch_bounds__(512, 1)
     k_gs_pass(T* __restrict__ W, const T* __restrict__ V, long long ldv, long long NP, int j, int b,
               const double* __restrict__ Pin, double* __restrict__ Pout, double* st, int m, const int* gate) {
+  step_kernel_begin();
   if (gate && *gate == 0) return;
   const GsPass g(j, b);
   Layout L{m};
@@ -434,6 +436,7 @@ template <typename T, int PK>
 __global__ void __launch_bounds__(512, 1)
     k_gs_finish(const T* __restrict__ W, T* __restrict__ Vn, long long NP, const double* __restrict__ Pin, int nparts,
                 int j, int m, double* st, int method, StepEnd end) {
+  step_kernel_begin();
   __shared__ double snorm[2];
   __shared__ double col[kMaxM];
   __shared__ KsStage S;
@@ -531,19 +534,8 @@ void launch_arnoldi_cluster(const T* W, T* V, long long ldv, int N, int j, int m
   const int cl = std::min(kArnCL, std::max(1, (N + 63) / 64));
   const int smem = (int)sizeof(T) * ((N + cl - 1) / cl) * (2 * kGB + 1);
   if (smem > 32 * 1024) set_max_dynamic_smem(reinterpret_cast<const void*>(&k_arnoldi_cluster<T>), smem);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cl, 1, 1);
-  cfg.blockDim = dim3(kArnThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cl;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  TS_CUDA(cudaLaunchKernelEx(&cfg, k_arnoldi_cluster<T>, W, V, ldv, N, j, m, s, method, end));
+  launch_step_kernel(k_arnoldi_cluster<T>, end.gate != nullptr, cl, kArnThreads, smem, cl, st, W, V, ldv, N, j, m, s,
+                     method, end);
   count_launch();
 }
 
@@ -557,13 +549,12 @@ void launch_gs(T* W, T* V, long long ldv, long long NP, int j, int m, double* s,
   double* Pb[2] = {P, P + (size_t)kGsSums * kGsBlocks};
   const int nblk = j / kGB + 1;
   for (int b = -1; b < nblk; ++b) {
-    if (j < 4)
-      k_gs_pass<T, PK, 4><<<nb, nt, 0, st>>>(W, V, ldv, NP, j, b, Pb[(b + 2) & 1], Pb[(b + 1) & 1], s, m, end.gate);
-    else
-      k_gs_pass<T, PK, 8><<<nb, nt, 0, st>>>(W, V, ldv, NP, j, b, Pb[(b + 2) & 1], Pb[(b + 1) & 1], s, m, end.gate);
+    launch_step_kernel(j < 4 ? k_gs_pass<T, PK, 4> : k_gs_pass<T, PK, 8>, end.gate != nullptr, nb, nt, 0, 0, st, W, V,
+                       ldv, NP, j, b, Pb[(b + 2) & 1], Pb[(b + 1) & 1], s, m, end.gate);
     count_launch();
   }
-  k_gs_finish<T, PK><<<nb + 1, nt, 0, st>>>(W, V + (long long)(j + 1) * ldv, NP, Pb[nblk & 1], nb, j, m, s, method, end);
+  launch_step_kernel(k_gs_finish<T, PK>, end.gate != nullptr, nb + 1, nt, 0, 0, st, W, V + (long long)(j + 1) * ldv, NP,
+                     Pb[nblk & 1], nb, j, m, s, method, end);
   count_launch();
 }
 

@@ -61,3 +61,18 @@ def test_fp32_basis(ctx, case):
     first = min(len(ref.history), len(res.history), m, 8)
     np.testing.assert_allclose(res.history[:first], ref.history[:first], rtol=0, atol=2e-5 * ref.normC)
     assert res.status == 0 and tp.norm(C - kr.sylv_apply(pr.A, pr.B, X)) <= 1e-10 * tp.norm(C)
+
+
+@pytest.mark.parametrize("method", ["gmres", "fom"])
+@pytest.mark.parametrize("case", [(24, 24, 4, 20), (91, 91, 1, 17), (60, 64, 16, 12)],
+                         ids=lambda c: "n%d_s%d_p%d_m%d" % c)
+def test_launched_ahead_gives_the_same_bits(ctx, monkeypatch, method, case):
+    """Steps launched ahead come up while their predecessors still run; step by step they do not."""
+    n, s, p, m = case
+    pr = inputs.dense_problem(n, s, p, seed=970 + n)
+    C = kr.sylv_apply(pr.A, pr.B, pr.Xstar)
+    runs = [solve(ctx, method, pr, C, m) for _ in range(5)]
+    monkeypatch.setenv("TSTAR_NO_LAUNCH_AHEAD", "1")
+    X, res = solve(ctx, method, pr, C, m)
+    for Xa, ra in runs:
+        assert np.array_equal(Xa, X) and np.array_equal(np.asarray(ra.history), np.asarray(res.history))
