@@ -42,15 +42,41 @@ __device__ __noinline__ void givens_safe(double2 a, double2 b, double& c, double
   }
   if (na == 0.0) {
     c = 0.0;
-    s = cscale(cconj(b), 1.0 / nb);   // G [0; b] = [s b; c b] = [|b|; 0]
+    s = make_double2(b.x / nb, -b.y / nb);   // G [0; b] = [s b; c b] = [|b|; 0]
     r = make_double2(nb, 0.0);
     return;
   }
+  // quotients, not reciprocals: the reciprocal of a subnormal modulus overflows
   const double nr = hypot(na, nb);
   c = na / nr;
-  const double2 ua = cscale(a, 1.0 / na);  // a / |a|
-  s = cscale(cmul(ua, cconj(b)), 1.0 / nr);
+  const double2 ua = make_double2(a.x / na, a.y / na);
+  s = cmul(ua, make_double2(b.x / nr, -b.y / nr));
   r = cscale(ua, nr);
+}
+
+// Principal square root of z with |z| = r > 0: the smaller component as Im z / (2 larger), no cancellation.
+__device__ __forceinline__ double2 principal_root(double2 z, double r) {
+  const double t = sqrt(0.5 * (r + fabs(z.x))), o = z.y / (2.0 * t);
+  return z.x >= 0.0 ? make_double2(t, o) : make_double2(fabs(o), z.y < 0.0 ? -t : t);
+}
+
+// The Wilkinson shift of [[a, b], [cc, d]] (see the sweep) when squares of its entries leave the FP64 range: the
+// block is scaled by a power of two first, moduli are taken by hypot and the quotient by Smith's division.
+__device__ __noinline__ double2 shift_safe(double2 a, double2 b, double2 cc, double2 d) {
+  double2 half = csub(a, d);
+  const double m = fmax(fmax(fmax(fabs(half.x), fabs(half.y)), fmax(fabs(b.x), fabs(b.y))),
+                        fmax(fabs(cc.x), fabs(cc.y)));
+  if (!(m > 0.0 && m <= DBL_MAX)) return d;
+  const int e = ilogb(m);
+  auto scaled = [](double2 z, int q) { return make_double2(scalbn(z.x, q), scalbn(z.y, q)); };
+  half = scaled(half, -e - 1);
+  const double2 bc = cmul(scaled(b, -e), scaled(cc, -e)), z = cadd(cmul(half, half), bc);
+  const double r = cabs2(z);
+  double2 sq = r > 0.0 ? principal_root(z, r) : make_double2(0.0, 0.0);
+  if (fma(half.y, sq.y, half.x * sq.x) < 0.0) sq = make_double2(-sq.x, -sq.y);
+  const double2 den = cadd(half, sq);
+  if (den.x == 0.0 && den.y == 0.0) return d;
+  return csub(d, scaled(cdiv(bc, den), e));
 }
 
 __device__ __forceinline__ double shfl_d(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -272,16 +298,15 @@ __global__ void __launch_bounds__(kSchurThreads)
         } else {
           const double2 half = cscale(csub(a, d), 0.5), bc = cmul(b, cc);
           const double2 z = cadd(cmul(half, half), bc);
-          const double r = sqrt(fma(z.y, z.y, z.x * z.x));
-          double2 sq = make_double2(0.0, 0.0);
-          if (r > 0.0) {   // principal square root: the smaller component as Im z / (2 larger), no cancellation
-            const double t = sqrt(0.5 * (r + fabs(z.x))), o = z.y / (2.0 * t);
-            sq = z.x >= 0.0 ? make_double2(t, o) : make_double2(fabs(o), z.y < 0.0 ? -t : t);
+          const double r2 = fma(z.y, z.y, z.x * z.x);
+          if (r2 >= 1e-280) {   // |sq| >= 1e-70, and |den| >= |sq|
+            double2 sq = principal_root(z, sqrt(r2));
+            if (fma(half.y, sq.y, half.x * sq.x) < 0.0) sq = make_double2(-sq.x, -sq.y);
+            const double2 den = cadd(half, sq);
+            mu = csub(d, cscale(cmul(bc, cconj(den)), 1.0 / fma(den.y, den.y, den.x * den.x)));
+          } else {
+            mu = shift_safe(a, b, cc, d);
           }
-          if (fma(half.y, sq.y, half.x * sq.x) < 0.0) sq = make_double2(-sq.x, -sq.y);
-          const double2 den = cadd(half, sq);
-          const double dn = fma(den.y, den.y, den.x * den.x);
-          mu = dn > 0.0 ? csub(d, cscale(cmul(bc, cconj(den)), 1.0 / dn)) : d;
         }
         const double2 x = csub(T[lo + lt * lo], mu), y = T[lo + 1 + lt * lo];
         const Rot q = make_rot(x, y, lane);
