@@ -45,6 +45,7 @@
 #include <cuda_bf16.h>
 #include <climits>
 #include <cfloat>
+#include <cstdlib>
 #include <algorithm>
 #include <vector>
 #include "internal.cuh"
@@ -86,6 +87,7 @@ struct OzOut {
   const unsigned long long* mx_op;
   const unsigned long long* mx_x;
   int n, s, K, nyq, S, F;
+  int stall;   // test aid: load the first k-block only, so the MMA warp's next wait expires
 };
 
 // Exponent of a slice from its maximum: max < 2^(E-1): ilogb(max) + 2 (0 for an all-zero slice); false when
@@ -191,7 +193,7 @@ __host__ __device__ constexpr int oz_sub(int S) { return 2 * S <= kOzSlots ? 2 :
 // KIND 0: complex slice, A X: D += Ar [Xr | Xi] + Ai [-Xi | Xr]   (B blocks [P; Q; R], Q-R then P-Q)
 //      1: complex slice, X B: D += -Xr [Br | Bi] + Xi [Bi | -Br]  (P-Q then Q-R)
 //      2, 3: real slice, A X and X B, 128 real columns: D += Ar [Xr], D += -Xr [Br]  (P-Q)
-// Returns false when a wait expired.
+// one: set in the lane that issues (elect_one).  Returns false when a wait expired.
 template <int S, int KIND>
 __device__ __forceinline__ bool oz_mma_block(uint32_t one, uint32_t bar_full, uint32_t bar_empty, uint32_t bar_acc, uint32_t bar_free,
                                              uint64_t desc0, uint32_t tmem, int first, int& q, int* err) {
@@ -244,12 +246,12 @@ __device__ __forceinline__ bool oz_mma_block(uint32_t one, uint32_t bar_full, ui
   return true;
 }
 template <int S>
-__device__ __noinline__ bool oz_mma_walk(uint32_t bars, uint32_t base, uint32_t tmem_, int real_, int kbA_, int kbs_,
-                                         int* err) {
+__device__ __noinline__ bool oz_mma_walk(uint32_t one, uint32_t bars, uint32_t base, uint32_t tmem_, int real_, int kbA_,
+                                         int kbs_, int* err) {
   const uint32_t bar_full = warp_uniform(bars), bar_empty = bar_full + 8 * kOzSlots;
   const uint32_t bar_acc = bar_empty + 8 * kOzSlots, bar_free = bar_acc + 8 * kOzAccs;
   const uint64_t desc0 = smem_desc_sw64(warp_uniform(base));
-  const uint32_t tmem = warp_uniform(tmem_), one = elect_one();
+  const uint32_t tmem = warp_uniform(tmem_);
   const bool real = warp_uniform(real_) != 0;
   const int kbA = (int)warp_uniform(kbA_), kbs = (int)warp_uniform(kbs_);
   int q = 0;   // unit
@@ -376,7 +378,7 @@ __device__ __noinline__ void oz_tile(const OzMaps* maps, const OzOut& o, int k, 
     if (lane == 0) {
       int it = 0, issued = 0;   // slots visited / slots whose loads were issued
       bool ok = true;
-      for (int kb = 0; kb < kbs && ok; ++kb) {
+      for (int kb = 0; kb < (o.stall ? 1 : kbs) && ok; ++kb) {
         const bool ax = kb < kbA;
         for (int i = 0; i < S * sub; ++i, ++it) {
           const int d = S - i / sub, l0 = (ax ? kb : kb - kbA) * depth + i % sub * kOzKB;
@@ -423,14 +425,15 @@ __device__ __noinline__ void oz_tile(const OzMaps* maps, const OzOut& o, int k, 
     }
   } else if (warp == kOzEpi + 1) {
     bool ok = true;
+    const uint32_t one = elect_one();
     switch (S) {
 #define TS_OZ_WALK(D) \
-  case D: ok = oz_mma_walk<D>(bar_full, base, tmem, real, kbA, kbs, err); break;
+  case D: ok = oz_mma_walk<D>(one, bar_full, base, tmem, real, kbA, kbs, err); break;
       TS_OZ_WALK(3) TS_OZ_WALK(4) TS_OZ_WALK(5) TS_OZ_WALK(6) TS_OZ_WALK(7) TS_OZ_WALK(8)
 #undef TS_OZ_WALK
     }
-    if (!ok && lane == 0) {   // after an error the MMAs already issued still complete before TMEM is freed
-      mma_commit(bar_done);
+    if (!ok) {   // after an error the MMAs already issued still complete before TMEM is freed
+      mma_commit_one(one, bar_done);   // by the lane that issued them: a commit covers its own thread's MMAs only
       mbar_wait(bar_done, 0u, err, 16);
     }
     __syncwarp();
@@ -701,7 +704,7 @@ void oz_maps(OzMaps* m, const ts_op* op, int S, const OzBuffers& b) {
 
 OzOut oz_out(const ts_op* op, double2* Yh, int S, const OzBuffers& b) {
   return OzOut{Yh, op->oz->mx, b.mx, op->n, op->s, op->K, nyquist_index(op->p), S,
-               oz_fixed_point(op->n, op->s, S)};
+               oz_fixed_point(op->n, op->s, S), 0};
 }
 
 }  // namespace
@@ -798,7 +801,12 @@ void oz_products(const ts_op* op, const double2* Xh, double2* Yh, int S, const O
   const long long mt = (n + kOzM - 1) / kOzM, kr = 1 + (nyq >= 0 ? 1 : 0);
   const long long blocks = mt * ((K - kr) * ((s + kOzN - 1) / kOzN) + kr * ((s + 2 * kOzN - 1) / (2 * kOzN)));
   TS_REQUIRE(blocks <= INT_MAX, "emulated product: grid too large");
-  k_oz_sylv<<<(unsigned)blocks, kOzThreads, kOzSmem, st>>>(maps, oz_out(op, Yh, S, b), nullptr, nullptr, nullptr, err);
+  OzOut out = oz_out(op, Yh, S, b);
+  // Test aid for the failure path (see tc_apply): with TSTAR_TEST_STALL_TMA=1 the producer stops after the first
+  // k-block, with that block's MMAs issued.
+  const char* stall_env = std::getenv("TSTAR_TEST_STALL_TMA");
+  out.stall = stall_env && stall_env[0] == '1';
+  k_oz_sylv<<<(unsigned)blocks, kOzThreads, kOzSmem, st>>>(maps, out, nullptr, nullptr, nullptr, err);
   count_launch();
   TS_CUDA(cudaGetLastError());
 }
