@@ -193,7 +193,8 @@ __host__ __device__ constexpr int oz_sub(int S) { return 2 * S <= kOzSlots ? 2 :
 // KIND 0: complex slice, A X: D += Ar [Xr | Xi] + Ai [-Xi | Xr]   (B blocks [P; Q; R], Q-R then P-Q)
 //      1: complex slice, X B: D += -Xr [Br | Bi] + Xi [Bi | -Br]  (P-Q then Q-R)
 //      2, 3: real slice, A X and X B, 128 real columns: D += Ar [Xr], D += -Xr [Br]  (P-Q)
-// one: set in the lane that issues (elect_one).  Returns false when a wait expired.
+// Returns false when a wait expired; oz_mma_walk has then committed the MMAs it issued to the `done` barrier (a
+// commit covers its own thread's MMAs only, and the elected lane is known here).
 template <int S, int KIND>
 __device__ __forceinline__ bool oz_mma_block(uint32_t one, uint32_t bar_full, uint32_t bar_empty, uint32_t bar_acc, uint32_t bar_free,
                                              uint64_t desc0, uint32_t tmem, int first, int& q, int* err) {
@@ -246,12 +247,12 @@ __device__ __forceinline__ bool oz_mma_block(uint32_t one, uint32_t bar_full, ui
   return true;
 }
 template <int S>
-__device__ __noinline__ bool oz_mma_walk(uint32_t one, uint32_t bars, uint32_t base, uint32_t tmem_, int real_, int kbA_,
-                                         int kbs_, int* err) {
+__device__ __noinline__ bool oz_mma_walk(uint32_t bars, uint32_t base, uint32_t tmem_, int real_, int kbA_, int kbs_,
+                                         int* err) {
   const uint32_t bar_full = warp_uniform(bars), bar_empty = bar_full + 8 * kOzSlots;
   const uint32_t bar_acc = bar_empty + 8 * kOzSlots, bar_free = bar_acc + 8 * kOzAccs;
   const uint64_t desc0 = smem_desc_sw64(warp_uniform(base));
-  const uint32_t tmem = warp_uniform(tmem_);
+  const uint32_t tmem = warp_uniform(tmem_), one = elect_one();
   const bool real = warp_uniform(real_) != 0;
   const int kbA = (int)warp_uniform(kbA_), kbs = (int)warp_uniform(kbs_);
   int q = 0;   // unit
@@ -264,7 +265,10 @@ __device__ __noinline__ bool oz_mma_walk(uint32_t one, uint32_t bars, uint32_t b
       ok = kb < kbA ? oz_mma_block<S, 0>(one, bar_full, bar_empty, bar_acc, bar_free, desc0, tmem, kb * S * oz_sub(S), q, err)
                     : oz_mma_block<S, 1>(one, bar_full, bar_empty, bar_acc, bar_free, desc0, tmem, kb * S * oz_sub(S), q, err);
     }
-    if (!ok) return false;
+    if (!ok) {
+      mma_commit_one(one, bar_free + 8 * kOzAccs);
+      return false;
+    }
   }
   return true;
 }
@@ -425,17 +429,14 @@ __device__ __noinline__ void oz_tile(const OzMaps* maps, const OzOut& o, int k, 
     }
   } else if (warp == kOzEpi + 1) {
     bool ok = true;
-    const uint32_t one = elect_one();
     switch (S) {
 #define TS_OZ_WALK(D) \
-  case D: ok = oz_mma_walk<D>(one, bar_full, base, tmem, real, kbA, kbs, err); break;
+  case D: ok = oz_mma_walk<D>(bar_full, base, tmem, real, kbA, kbs, err); break;
       TS_OZ_WALK(3) TS_OZ_WALK(4) TS_OZ_WALK(5) TS_OZ_WALK(6) TS_OZ_WALK(7) TS_OZ_WALK(8)
 #undef TS_OZ_WALK
     }
-    if (!ok) {   // after an error the MMAs already issued still complete before TMEM is freed
-      mma_commit_one(one, bar_done);   // by the lane that issued them: a commit covers its own thread's MMAs only
-      mbar_wait(bar_done, 0u, err, 16);
-    }
+    // after an error the MMAs already issued still complete before TMEM is freed
+    if (!ok) mbar_wait(bar_done, 0u, err, 16);
     __syncwarp();
   } else {
     oz_drain(o, tmem, bar_acc, bar_free, k, i0, j0, err);
