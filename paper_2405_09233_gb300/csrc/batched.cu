@@ -139,8 +139,9 @@ __global__ void __launch_bounds__(256) k_b_normC(BDev d, double* __restrict__ P)
 // V_i+1 and writing W, took 54 us (35 for the first product) where the batch's vectors have 12M FP32 entries;
 // a pass takes 58 us there for up to four vectors, 75 for up to eight.
 template <typename T, int VB>
-__global__ void __launch_bounds__(256) k_b_gs_pass(BDev d, T* __restrict__ W, const T* __restrict__ V, int j, int b,
-                                                   const double* __restrict__ Pin, double* __restrict__ Pout) {
+__global__ void __launch_bounds__(256, 2) k_b_gs_pass(BDev d, T* __restrict__ W, const T* __restrict__ V, int j,
+                                                      int b, const double* __restrict__ Pin,
+                                                      double* __restrict__ Pout) {
   const int i = d.nb_inst[blockIdx.x];
   if (!d.act[i]) return;
   const BInst& in = d.inst[i];

@@ -5,7 +5,7 @@
 // <V_i, V_l>: h_i = <V_i, W - sum_{l<i} h_l V_l> written out.  So one reduction gives eight coefficients where
 // a sweep vector by vector waits for eight, each behind the other; the Gram row of V_j (at most 7 more inner
 // products) is formed once, in step j, whose last block it completes.  The result is modified Gram-Schmidt's
-// up to rounding: against FP64 MGS, orthogonality and residuals are the same (see the tests).
+// up to rounding: the estimates of every step agree with FP64 MGS's to 1e-12 ||C|| in the tests.
 #pragma once
 #include <cuda_runtime.h>
 #include <type_traits>
@@ -27,22 +27,68 @@ __device__ __forceinline__ double gs_forward(double d, const double (&row)[kGB -
   return d;
 }
 
-// A sum kept as FP64, or as an unevaluated pair of FP32 numbers hi + lo to which every addition's rounding
-// error is added (Knuth's two-sum): as exact as FP64 here, without an FP64 instruction.
-struct Pair {
-  float hi, lo;
+// A sum kept as FP64, or as an unevaluated sum of three FP32 numbers.  Every addition's rounding error is added
+// to the next smaller part (Knuth's two-sum); what the smallest part rounds away is 2^-72 of the running sum per
+// addition, so n additions err by less than FP64's n 2^-53 up to n = 2^19, without an FP64 instruction.
+struct Triple {
+  float hi = 0.f, mid = 0.f, lo = 0.f;
 };
-__device__ __forceinline__ double add_sums(double a, double b) { return a + b; }
-__device__ __forceinline__ Pair add_sums(Pair a, Pair b) {
-  const float sum = a.hi + b.hi, g = sum - a.hi;
-  return Pair{sum, a.lo + b.lo + ((a.hi - (sum - g)) + (b.hi - g))};
+__host__ __device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float sum = a + b, g = sum - a;
+  err = (a - (sum - g)) + (b - g);
+  return sum;
+}
+__host__ __device__ __forceinline__ double add_sums(double a, double b) { return a + b; }
+__host__ __device__ __forceinline__ Triple add_sums(Triple a, Triple b) {
+  Triple s;
+  float e1, e2, e3;
+  s.hi = two_sum(a.hi, b.hi, e1);
+  s.mid = two_sum(a.mid, b.mid, e2);
+  s.mid = two_sum(s.mid, e1, e3);
+  s.lo = (a.lo + b.lo) + (e2 + e3);
+  return s;
+}
+__host__ __device__ __forceinline__ void add_to(Triple& s, float x) {
+  float e1, e2;
+  s.hi = two_sum(s.hi, x, e1);
+  s.mid = two_sum(s.mid, e1, e2);
+  s.lo += e2;
 }
 __device__ __forceinline__ double shfl_sum(double a, int mask) { return __shfl_xor_sync(0xffffffffu, a, mask); }
-__device__ __forceinline__ Pair shfl_sum(Pair a, int mask) {
-  return Pair{__shfl_xor_sync(0xffffffffu, a.hi, mask), __shfl_xor_sync(0xffffffffu, a.lo, mask)};
+__device__ __forceinline__ Triple shfl_sum(Triple a, int mask) {
+  Triple s;
+  s.hi = __shfl_xor_sync(0xffffffffu, a.hi, mask);
+  s.mid = __shfl_xor_sync(0xffffffffu, a.mid, mask);
+  s.lo = __shfl_xor_sync(0xffffffffu, a.lo, mask);
+  return s;
 }
-__device__ __forceinline__ double value_of(double a) { return a; }
-__device__ __forceinline__ double value_of(Pair a) { return (double)a.hi + (double)a.lo; }
+__host__ __device__ __forceinline__ double value_of(double a) { return a; }
+__host__ __device__ __forceinline__ double value_of(Triple a) {
+  return (double)a.hi + ((double)a.mid + (double)a.lo);
+}
+
+// s += <x, y>: term by term in FP64; of FP32 vectors a pack's products are summed in FP32 (pack.cuh), a single
+// product is added exactly.
+template <int PK>
+__host__ __device__ __forceinline__ void add_products(double& s, const double (&x)[PK], const double (&y)[PK]) {
+#pragma unroll
+  for (int c = 0; c < PK; ++c) s = fma(x[c], y[c], s);
+}
+template <int PK>
+__host__ __device__ __forceinline__ void add_products(Triple& s, const float (&x)[PK], const float (&y)[PK]) {
+  float f = x[0] * y[0];
+  if constexpr (PK == 1) {
+    const float e = fmaf(x[0], y[0], -f);
+    add_to(s, f);
+    float e2;
+    s.mid = two_sum(s.mid, e, e2);
+    s.lo += e2;
+  } else {
+#pragma unroll
+    for (int c = 1; c < PK; ++c) f = fmaf(x[c], y[c], f);
+    add_to(s, f);
+  }
+}
 
 // v[0..NV-1] summed over the warp: lane's result is sum lane / (32 / NV); NV 4, 8 or 16.
 template <int NV, typename Sum>
@@ -152,7 +198,7 @@ __device__ __forceinline__ void gs_coefficients(const GsPass& g, const double* _
 // A thread's sums of a pass.
 template <typename T, int VB>
 struct GsSums {
-  using Sum = typename std::conditional<sizeof(T) == 8, double, Pair>::type;
+  using Sum = typename std::conditional<sizeof(T) == 8, double, Triple>::type;
   Sum v[2 * VB];
   double norm = 0.0;
   __device__ __forceinline__ GsSums() {
@@ -162,9 +208,11 @@ struct GsSums {
 };
 
 // One thread's packs of W, first, first + stride, ... < NP, of a pass.
-// FP32 vectors: two packs (eight products) are summed in FP32 (pack.cuh) and such sums in Pairs; a conversion and
-// an FP64 addition per eight products took half of the pass's time, and reducing FP64 sums over the block most
-// of a batch's.  VB = 4 (the first steps) keeps twice the packs in flight.
+// FP32 vectors: a pack's four products are summed in FP32 and such sums in Triples; a conversion and an FP64
+// addition per eight products took half of the pass's time, and reducing FP64 sums over the block most of a
+// batch's.  (Two FP32 parts, rounding in the second one, and groups of eight held 48 bits: n = s = 1024, p = 16
+// BF16 solve 19.31 -> 19.36 ms, 64 uneven instances 20.43 -> 20.45; two sums to an f32x2 instruction 19.52 and
+// 20.91.)  VB = 4 (the first steps) keeps twice the packs in flight.
 template <typename T, int PK, int VB>
 __device__ __forceinline__ void gs_stream(const GsPass& g, T* __restrict__ W, const T* __restrict__ V, long long ldv,
                                           long long first, long long NP, long long stride, const T (&h)[VB],
@@ -172,19 +220,9 @@ __device__ __forceinline__ void gs_stream(const GsPass& g, T* __restrict__ W, co
   const int nu = g.nu, nd = g.nd;
   const bool lastd = g.lastd;
   const T *Vu = V + (long long)(kGB * max(g.b, 0)) * ldv, *Vd = V + (long long)(kGB * (g.b + 1)) * ldv;
+  // packs in flight of each vector, and per round of the loop
   constexpr int UN = sizeof(T) == 4 ? 2 : 1, GR = VB == 4 ? 2 * UN : 1, NI = VB == 4 ? GR : UN;
-  float f[2 * VB];
-#pragma unroll
-  for (int q = 0; q < 2 * VB; ++q) f[q] = 0.f;
-  const auto used = [&](int q) { return q < VB ? q < nd : (lastd && q - VB < nd - 1); };
-  const auto add_dot = [&](const T (&x)[PK], const T (&y)[PK], int q) {
-#pragma unroll
-    for (int c = 0; c < PK; ++c) {
-      if constexpr (sizeof(T) == 8) sums.v[q] = fma(x[c], y[c], sums.v[q]);
-      else f[q] = fmaf(x[c], y[c], f[q]);
-    }
-  };
-    for (long long p0 = first; p0 < NP; p0 += NI * stride) {
+  for (long long p0 = first; p0 < NP; p0 += NI * stride) {
 #pragma unroll
     for (int u0 = 0; u0 < NI; u0 += GR) {
       T w[GR][PK], v[VB][GR][PK];
@@ -230,29 +268,17 @@ __device__ __forceinline__ void gs_stream(const GsPass& g, T* __restrict__ W, co
             ld_pack<T, PK>(Vd + (long long)(nd - 1) * ldv, p0 + (u0 + u) * stride, vj);
 #pragma unroll
           for (int q = 0; q < VB; ++q)
-            if (q < nd) add_dot(v[q][u], w[u], q);
+            if (q < nd) add_products(sums.v[q], v[q][u], w[u]);
           if (lastd) {
 #pragma unroll
             for (int q = 0; q < VB - 1; ++q)
-              if (q < nd - 1) add_dot(v[q][u], vj, VB + q);
+              if (q < nd - 1) add_products(sums.v[VB + q], v[q][u], vj);
           }
-        } else {
-          add_dot(w[u], w[u], 0);
-        }
-        if constexpr (sizeof(T) == 4) {
-          if ((u0 + u) % UN == UN - 1) {
-            if (nd) {
+        } else if constexpr (sizeof(T) == 8 || PK == 1) {
 #pragma unroll
-              for (int q = 0; q < 2 * VB; ++q)
-                if (used(q)) {
-                  sums.v[q] = add_sums(sums.v[q], Pair{f[q], 0.f});
-                  f[q] = 0.f;
-                }
-            } else {
-              sums.norm += (double)f[0];   // no sum of squares beyond FP32's range
-              f[0] = 0.f;
-            }
-          }
+          for (int c = 0; c < PK; ++c) sums.norm = fma((double)w[u][c], (double)w[u][c], sums.norm);
+        } else {   // no sum of squares beyond FP32's range
+          sums.norm += (double)pack_dot(w[u], w[u]);
         }
       }
     }
@@ -266,9 +292,7 @@ __device__ __forceinline__ void gs_store(const GsPass& g, GsSums<T, VB>& sums, d
   __shared__ double red[16][kGsSums];
   const int t = threadIdx.x, lane = t & 31, wp = t >> 5, nw = blockDim.x >> 5;
   if (!g.nd) {
-    double own = sums.norm;
-    if constexpr (sizeof(T) == 8) own = sums.v[0];
-    const double tot = block_sum(own);
+    const double tot = block_sum(sums.norm);
     if (t == 0) Pout[at] = tot;
     return;
   }

@@ -302,19 +302,18 @@ __global__ void __launch_bounds__(kArnThreads, 1)
           if (gram) y = fma(v[q], vj[q], y);
         }
       } else {
-        for (int q0 = lane; q0 < cnt; q0 += 256) {   // eight products per FP64 addition (pack.cuh)
-          float f = 0.f, g = 0.f;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int q = q0 + 32 * u;
-            if (q < cnt) {
-              f = fmaf(v[q], w[q], f);
-              if (gram) g = fmaf(v[q], vj[q], g);
-            }
+        Triple f, g;
+        for (int q = lane; q < cnt; q += 64) {   // products summed in pairs, the pairs in Triples
+          const bool two = q + 32 < cnt;
+          const float v2[2] = {v[q], two ? v[q + 32] : 0.f}, w2[2] = {w[q], two ? w[q + 32] : 0.f};
+          add_products(f, v2, w2);
+          if (gram) {
+            const float j2[2] = {vj[q], two ? vj[q + 32] : 0.f};
+            add_products(g, v2, j2);
           }
-          x += (double)f;
-          if (gram) y += (double)g;
         }
+        x = value_of(f);
+        if (gram) y = value_of(g);
       }
       // lanes 0-15 end with the sum of x, lanes 16-31 with that of y
       const double o = __shfl_xor_sync(0xffffffffu, lane < 16 ? y : x, 16);
@@ -362,7 +361,7 @@ __global__ void __launch_bounds__(kArnThreads, 1)
             nrm = fma(x, x, nrm);
           } else {
             f = fmaf(x, x, f);
-            if ((u & 7) == 7) {
+            if ((u & 1) == 1) {
               nrm += (double)f;
               f = 0.f;
             }
