@@ -18,7 +18,7 @@
 //    g <= S + 1 are kept (the dropped ones are below the truncation error of the digits).  Each
 //    accumulator run ("unit": every pair of one g over one k-block of 32) is read from TMEM, converted to
 //    int32 and added into per-thread int64 accumulators at the common fixed point
-//    2^(E_op + E_x - F), F <= 63 - ceil(log2(2 (n + s))), which keeps every partial sum below 2^62.
+//    2^(E_op + E_x - F), F = 63 - ceil(log2(2 (n + s))), which keeps every partial sum below 2^62.
 //    Units with 8g > F are added with a rounded right shift.
 //  * Y = double(acc) 2^(E_op + E_x - F): one rounding.
 //
@@ -129,34 +129,56 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "memory");
 }
 
+// 32-deep blocks per unit: with few digits two fit the slots, and a unit of few MMAs would leave the epilogue
+// behind (4 pairs x 128 products of 2^14 stay below 2^24).
+__host__ __device__ constexpr int oz_sub(int S) { return 2 * S <= kOzSlots ? 2 : 1; }
+
 // Units are drained two at a time, g + 1 (values b) and g (values a), 256 apart in scale (an odd S leaves its
 // top unit alone, as a b without a): t = a' ca + b' in 32 bits, then acc += t m in one 32 x 32 + 64
 // multiply-add, so that the accumulators see half the updates.  a' is converted (2 clocks of the SM per
 // warp, on a pipe of its own); b' is read off the bit pattern of b + M, M = 1.5 2^(23 + e), which is that of M
 // plus round(b / 2^e) while |b| <= 2^(22 + e).  M's pattern goes into the accumulators with the value and
-// comes out at the end (arithmetic modulo 2^64).  Ranges: e = 0 needs at most 4 pairs (4 x 64 products of 2^14),
-// which g + 1 <= 5 has; g + 1 = S + 1 and 7 get e >= 1 from F <= 8 (S + 1) - 1 and F <= 55 (oz_fixed_point).
-// |t| < 2^31: the largest is M's pattern, 1.26e9, plus 256 times 3 x 2^20 plus 2^22.
+// comes out at the end (arithmetic modulo 2^64).  e = 0 needs at most 4 pairs (4 x 64 products of 2^14).  More occur
+// at e = 0 where F leaves all of the lowest units' bits: with 5 digits or fewer, and for n + s <= 64 (oz_forms's
+// conditions).  There b is converted like a (kOzConvert), and beyond a factor of 2^30 the sum is shifted instead of
+// multiplied more than twice (kOzShift).
+// |t| < 2^31: M's pattern, 1.26e9, plus 256 times 3 x 2^20 (e = 0) or 2^7 times 6 x 2^20 (e > 0), plus 2^23; without
+// M, 256 times 7 x 2^20 plus 2^23.
+// The epilogue sets the pace together with the MMAs, so it exists once per set of forms: with all of them in one,
+// n = s = 1024, p = 16 and 6 digits took 2.72 to 2.82 ms, not 2.69.
+// There, before the lowest bits were kept and now: 5 digits 2.40 / 2.48 ms, 4 digits 1.69 / 1.70, 3 digits 1.33 / 1.31.
 constexpr uint32_t kOzMagic = 0x4B400000u;   // pattern of 1.5 2^23; 2^e times it: + e 2^23
+enum { kOzPattern, kOzConvert, kOzShift };
+// The last form that some unit of a product takes.
+__device__ __forceinline__ int oz_forms(int F, int S) {
+  return F < 8 * (S + 1) && F <= 55 ? kOzPattern : (F <= 54 ? kOzConvert : kOzShift);
+}
 struct OzScale {
+  int mode;
   float M, fa;        // b' from b + M; a' = round(a fa)
   int ca, m, reps;    // acc += (a' ca + pattern) m, reps times
+  int sh;             // kOzShift: acc += (a' ca + b') << sh
   long long offset;   // what M's pattern adds
 };
-__device__ __forceinline__ OzScale oz_scale(int F, int gb, bool lone) {
+template <int FORMS>
+__device__ __forceinline__ OzScale oz_scale(int F, int S, int gb, bool lone) {
   const int sb = F - 8 * gb, sa = sb + 8;
   const uint32_t pat = kOzMagic + (sb < 0 ? (uint32_t)-sb << 23 : 0u);
   OzScale q;
+  if (FORMS == kOzPattern) q.mode = kOzPattern;
+  else if (FORMS == kOzShift && sb > 30) q.mode = kOzShift;
+  else q.mode = sb >= 0 && (gb - 1) * oz_sub(S) > 4 ? kOzConvert : kOzPattern;
   q.M = __uint_as_float(pat);
   q.fa = sa < 0 ? __uint_as_float((uint32_t)(127 + sa) << 23) : 1.f;
   q.ca = lone ? 0 : (sb >= 0 ? 256 : (sa > 0 ? 1 << sa : 1));
   q.m = sb <= 0 ? 1 : 1 << (sb > 30 ? 30 : sb);
   q.reps = sb > 30 ? 1 << (sb - 30) : 1;
-  q.offset = (long long)pat * q.m * q.reps;
+  q.sh = sb;
+  q.offset = q.mode == kOzPattern ? (long long)pat * q.m * q.reps : 0ll;
   return q;
 }
 // Columns C0 .. C0 + 7 of the units at ta (a) and tb (b).
-template <int C0>
+template <int MODE, int C0>
 __device__ __forceinline__ void acc_add8(long long (&acc)[kOzCols], uint32_t ta, uint32_t tb, const OzScale& q) {
   uint32_t va[8], vb[8];
   tmem_ld8(ta + C0, va);
@@ -164,27 +186,43 @@ __device__ __forceinline__ void acc_add8(long long (&acc)[kOzCols], uint32_t ta,
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const int t = __float2int_rn(__uint_as_float(va[c]) * q.fa) * q.ca + __float_as_int(__uint_as_float(vb[c]) + q.M);
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[C0 + c]) : "r"(t), "r"(q.m));
+    const float fb = __uint_as_float(vb[c]);
+    const int b = MODE == kOzPattern ? __float_as_int(fb + q.M) : __float2int_rn(fb);
+    const int t = __float2int_rn(__uint_as_float(va[c]) * q.fa) * q.ca + b;
+    if (MODE == kOzShift) acc[C0 + c] += (long long)t << q.sh;
+    else asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[C0 + c]) : "r"(t), "r"(q.m));
   }
 }
-template <int C0>
-__device__ __forceinline__ void acc_add(long long (&acc)[kOzCols], uint32_t ta, uint32_t tb, const OzScale& q) {
-  acc_add8<C0>(acc, ta, tb, q);
-  if constexpr (C0 + 8 < kOzCols) acc_add<C0 + 8>(acc, ta, tb, q);
+// The lone unit at tb.
+template <int MODE, int C0>
+__device__ __forceinline__ void acc_add8_lone(long long (&acc)[kOzCols], uint32_t tb, const OzScale& q) {
+  uint32_t vb[8];
+  tmem_ld8(tb + C0, vb);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const float fb = __uint_as_float(vb[c]);
+    const int t = MODE == kOzPattern ? __float_as_int(fb + q.M) : __float2int_rn(fb);
+    if (MODE == kOzShift) acc[C0 + c] += (long long)t << q.sh;
+    else asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[C0 + c]) : "r"(t), "r"(q.m));
+  }
 }
-// Fixed point 2^(E_op + E_x - F): |partial sums| < 2 (n + s) 2^(E_op + E_x - 2) <= 2^(E_op + E_x + 62 - F),
-// with the caps that acc_add8 needs; they bind for n + s <= 128 (S >= 6) or few digits, and leave F's unit at
-// 2^-56 or 2^-8 of the digits' own last unit.
-int oz_fixed_point(int n, int s, int S) {
+template <int MODE, int C0 = 0>
+__device__ __forceinline__ void acc_add(long long (&acc)[kOzCols], uint32_t ta, uint32_t tb, const OzScale& q) {
+  acc_add8<MODE, C0>(acc, ta, tb, q);
+  if constexpr (C0 + 8 < kOzCols) acc_add<MODE, C0 + 8>(acc, ta, tb, q);
+}
+template <int MODE, int C0 = 0>
+__device__ __forceinline__ void acc_add_lone(long long (&acc)[kOzCols], uint32_t tb, const OzScale& q) {
+  acc_add8_lone<MODE, C0>(acc, tb, q);
+  if constexpr (C0 + 8 < kOzCols) acc_add_lone<MODE, C0 + 8>(acc, tb, q);
+}
+// Fixed point 2^(E_op + E_x - F): |partial sums| < 2 (n + s) 2^(E_op + E_x - 2) <= 2^(E_op + E_x + 62 - F).
+int oz_fixed_point(int n, int s) {
   int lg = 0;
   while ((1ll << lg) < 2ll * ((long long)n + s)) ++lg;
-  return std::min(63 - lg, std::min(8 * (S + 1) - 1, 55));
+  return 63 - lg;
 }
-
-// 32-deep blocks per unit: with few digits two fit the slots, and a unit of few MMAs would leave the epilogue
-// behind (4 pairs x 128 products of 2^14 stay below 2^24, and in acc_add8's ranges).
-__host__ __device__ constexpr int oz_sub(int S) { return 2 * S <= kOzSlots ? 2 : 1; }
 
 // The MMA issuer's walk of a tile with S digits (one converged warp).  Everything but the slots is known at
 // compile time and the operands are uniform, so that between two MMAs (64 clocks) it executes a handful of
@@ -275,6 +313,7 @@ __device__ __noinline__ bool oz_mma_walk(uint32_t bars, uint32_t base, uint32_t 
 
 // The epilogue warps' part of a tile: every unit into the accumulators, then Y.  Out of line (as the issue
 // walks are), so that its registers are allocated for it alone.
+template <int FORMS>   // oz_forms(F, S)
 __device__ __noinline__ void oz_drain(const OzOut& o, uint32_t tmem, uint32_t bar_acc, uint32_t bar_free, int k, int i0,
                                       int j0, int* err) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -293,7 +332,7 @@ __device__ __noinline__ void oz_drain(const OzOut& o, uint32_t tmem, uint32_t ba
   for (int kb = 0; kb < kbs && ok; ++kb) {
     for (int g = S + 1; g >= 2;) {   // units g (b) and g - 1 (a)
       const bool lone = g == S + 1 && S % 2 != 0;
-      const OzScale sc = oz_scale(F, g, lone);
+      const OzScale sc = oz_scale<FORMS>(F, S, g, lone);
       const int qa = lone ? q : q + 1, bb = q % kOzAccs, ba = qa % kOzAccs;
       if (!mbar_wait(bar_acc + 8 * ba, (uint32_t)(qa / kOzAccs) & 1u, err, 14)) {   // then b is complete too
         ok = false;
@@ -301,9 +340,29 @@ __device__ __noinline__ void oz_drain(const OzOut& o, uint32_t tmem, uint32_t ba
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tb = lane_base + (uint32_t)(bb * 2 * kOzN), ta = lane_base + (uint32_t)(ba * 2 * kOzN);
-      for (int r = 0; r < sc.reps; ++r) {   // 8 columns at a time: little room beside the accumulators
-        acc_add<0>(ar, ta, tb, sc);
-        acc_add<0>(ai, ta + kOzN, tb + kOzN, sc);
+      // 8 columns at a time: little room beside the accumulators
+      if (FORMS == kOzPattern || (sc.mode == kOzPattern && !lone)) {
+        for (int r = 0; r < sc.reps; ++r) {
+          acc_add<kOzPattern>(ar, ta, tb, sc);
+          acc_add<kOzPattern>(ai, ta + kOzN, tb + kOzN, sc);
+        }
+      } else if (lone) {
+        if (sc.mode == kOzPattern) {
+          acc_add_lone<kOzPattern>(ar, tb, sc);
+          acc_add_lone<kOzPattern>(ai, tb + kOzN, sc);
+        } else if (FORMS == kOzConvert || sc.mode == kOzConvert) {
+          acc_add_lone<kOzConvert>(ar, tb, sc);
+          acc_add_lone<kOzConvert>(ai, tb + kOzN, sc);
+        } else {
+          acc_add_lone<kOzShift>(ar, tb, sc);
+          acc_add_lone<kOzShift>(ai, tb + kOzN, sc);
+        }
+      } else if (FORMS == kOzConvert || sc.mode == kOzConvert) {
+        acc_add<kOzConvert>(ar, ta, tb, sc);
+        acc_add<kOzConvert>(ai, ta + kOzN, tb + kOzN, sc);
+      } else {
+        acc_add<kOzShift>(ar, ta, tb, sc);
+        acc_add<kOzShift>(ai, ta + kOzN, tb + kOzN, sc);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -439,7 +498,10 @@ __device__ __noinline__ void oz_tile(const OzMaps* maps, const OzOut& o, int k, 
     if (!ok) mbar_wait(bar_done, 0u, err, 16);
     __syncwarp();
   } else {
-    oz_drain(o, tmem, bar_acc, bar_free, k, i0, j0, err);
+    const int forms = oz_forms(o.F, S);
+    if (forms == kOzPattern) oz_drain<kOzPattern>(o, tmem, bar_acc, bar_free, k, i0, j0, err);
+    else if (forms == kOzConvert) oz_drain<kOzConvert>(o, tmem, bar_acc, bar_free, k, i0, j0, err);
+    else oz_drain<kOzShift>(o, tmem, bar_acc, bar_free, k, i0, j0, err);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -705,7 +767,7 @@ void oz_maps(OzMaps* m, const ts_op* op, int S, const OzBuffers& b) {
 
 OzOut oz_out(const ts_op* op, double2* Yh, int S, const OzBuffers& b) {
   return OzOut{Yh, op->oz->mx, b.mx, op->n, op->s, op->K, nyquist_index(op->p), S,
-               oz_fixed_point(op->n, op->s, S), 0};
+               oz_fixed_point(op->n, op->s), 0};
 }
 
 }  // namespace
