@@ -217,6 +217,17 @@ SliceParts slice_parts(int K, int nyq, int n, int blocks, int min_rows) {
   return q;
 }
 
+// Blocks of an FP32 Gram: a block's rows are added up in FP32 (then in FP64 over the blocks), so a slice has at least
+// 2 x 152 / K of them, or one per 64 rows, the real slices too; with a third of a complex slice's blocks their
+// chains were 4.6 times as long (n = 16384, p = 8: 1261 rows instead of 274).
+SliceParts gram_parts_f32(int K, int nyq, int n, int sms) {
+  SliceParts q = slice_parts(K, nyq, n, sms, 32);
+  const int least = std::max(1, std::min(2 * sms / K, (n + 63) / 64));
+  q.nc = std::max(q.nc, least);
+  q.nr = std::max(q.nr, least);
+  return q;
+}
+
 // Partial Gram matrices G_k = V_k^H W_k over row chunks: partials[block * s*s + a + s*b].
 // Gauss's three-multiplication form: with u = conj(v), u w = (T1 - T3) + i (T1 + T2) where
 // T1 = sum w_re (u_re + u_im), T2 = sum u_re (w_im - w_re), T3 = sum u_im (w_re + w_im); the sums
@@ -229,8 +240,8 @@ SliceParts slice_parts(int K, int nyq, int n, int blocks, int min_rows) {
 // multiplied, staging is double buffered (one barrier per batch), columns are padded to a multiple of
 // 4 only, and blocks are dealt to the slices by their cost.
 // Measured (n = 16384, s = 32, p = 8): 546 -> 357 us, with V = W 214 us; s = 4: 205 -> 34 us.
-// C2 = float2: FP32 inputs and accumulation (the inner cycle of mixed-precision TBAS); the partial
-// Grams are written in FP64 either way.
+// C2 = float2: FP32 inputs and accumulation over a block's rows (the inner cycle of mixed-precision TBAS; see
+// gram_parts_f32); the partial Grams are written in FP64 either way.
 constexpr int kGramMaxElems = 4;     // staged elements per thread and operand
 struct GramShape {
   int sg, tiles, groups, rb;         // 4-wide column groups, 4 x 4 blocks, row groups, staged rows
@@ -733,7 +744,7 @@ struct TbaWork {
   double2* Rinv;            // K x s x s
   double2* R2;              // K x s x s
   double2* gram_part;       // partial Grams
-  SliceParts gram_parts, row_parts;   // blocks of the Gram and row products
+  SliceParts gram_parts, gram_parts32, row_parts;   // blocks of the Gram (FP64, FP32) and row products
   double2* LU;              // K x s x N x N
   int* piv;                 // K x s x N
   double2* Gp;              // K x N x s
@@ -895,17 +906,18 @@ double block_flops(const TbaWork& w) { return 8.0 * w.n * w.s * w.s * w.K; }
 template <typename C2>
 void gram(const TbaWork& w, const C2* V, const C2* W, double2* out, long long sOut, int ldo, cudaStream_t st) {
   w.tm->begin(st, 4, block_flops(w));
+  const SliceParts& parts = sizeof(C2) == 16 ? w.gram_parts : w.gram_parts32;
   auto run = [&](auto herm) {
     constexpr bool HERM = decltype(herm)::value;
     const GramShape g = gram_shape<typename RealOf<C2>::T>(w.s, HERM);
     set_max_dynamic_smem((const void*)k_gram<C2, HERM>, (int)g.smem);
-    k_gram<C2, HERM><<<w.gram_parts.blocks(), 256, g.smem, st>>>(V, W, w.n, w.s, w.gram_parts, g, w.gram_part);
+    k_gram<C2, HERM><<<parts.blocks(), 256, g.smem, st>>>(V, W, w.n, w.s, parts, g, w.gram_part);
   };
   if (V == W) run(std::true_type{});
   else run(std::false_type{});
   count_launch();
   TS_CUDA(cudaGetLastError());
-  k_gram_reduce<<<dim3((w.s * w.s + 63) / 64, w.K), 256, 0, st>>>(w.gram_part, w.gram_parts, w.s, out, sOut, ldo);
+  k_gram_reduce<<<dim3((w.s * w.s + 63) / 64, w.K), 256, 0, st>>>(w.gram_part, parts, w.s, out, sOut, ldo);
   count_launch();
   TS_CUDA(cudaGetLastError());
   w.tm->end(st);
@@ -1019,8 +1031,10 @@ TbaWork tba_work(ts_ctx* ctx, const ts_op* op, int m) {
   w.Rinv = (double2*)get("tba_Rinv", ss);
   const int nyq = nyquist_index(w.p);
   w.gram_parts = slice_parts(K, nyq, n, ctx->num_sms, 32);
+  w.gram_parts32 = gram_parts_f32(K, nyq, n, ctx->num_sms);
   w.row_parts = slice_parts(K, nyq, n, 2 * ctx->num_sms, 32);
-  w.gram_part = (double2*)get("tba_gram_part", sizeof(double2) * (size_t)w.gram_parts.blocks() * s * s);
+  w.gram_part = (double2*)get("tba_gram_part", sizeof(double2) * s * s *
+                                                   (size_t)std::max(w.gram_parts.blocks(), w.gram_parts32.blocks()));
   w.LU = (double2*)get("tba_LU", sizeof(double2) * (size_t)K * s * N * N);
   w.piv = (int*)get("tba_piv", sizeof(int) * (size_t)K * s * N);
   w.Gp = (double2*)get("tba_Gp", sizeof(double2) * (size_t)K * N * s);
