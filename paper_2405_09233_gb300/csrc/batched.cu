@@ -17,7 +17,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
-#include <numeric>
+#include <memory>
 #include <vector>
 #include <type_traits>
 #include <string>
@@ -680,12 +680,22 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   long long* d_nb_off = (long long*)(((uintptr_t)(d_nb_inst + plan.nb_inst.size()) + 15) & ~(uintptr_t)15);
   int* d_tb_inst = (int*)(d_nb_off + plan.nb_off.size());
   long long* d_tb_off = (long long*)(((uintptr_t)(d_tb_inst + plan.tb_inst.size()) + 15) & ~(uintptr_t)15);
-  // the tables are copied from pageable memory: synchronous, before anything is captured
-  TS_CUDA(cudaMemcpy(d_inst, plan.inst.data(), sizeof(BInst) * count, cudaMemcpyHostToDevice));
-  TS_CUDA(cudaMemcpy(d_nb_inst, plan.nb_inst.data(), sizeof(int) * plan.nb_inst.size(), cudaMemcpyHostToDevice));
-  TS_CUDA(cudaMemcpy(d_nb_off, plan.nb_off.data(), sizeof(long long) * plan.nb_off.size(), cudaMemcpyHostToDevice));
-  TS_CUDA(cudaMemcpy(d_tb_inst, plan.tb_inst.data(), sizeof(int) * plan.tb_inst.size(), cudaMemcpyHostToDevice));
-  TS_CUDA(cudaMemcpy(d_tb_off, plan.tb_off.data(), sizeof(long long) * plan.tb_off.size(), cudaMemcpyHostToDevice));
+  // Tables go to the device in stream order, on the caller's stream until the private stream is ordered after it and
+  // on that one from then on: a plain cudaMemcpy may return before its copy is done, and nothing orders its stream
+  // with the private one.  Their host memory lives until the call returns.
+  std::vector<std::shared_ptr<void>> host_tables;
+  auto upload = [&](void* dst, auto table, cudaStream_t q) {
+    using Table = decltype(table);
+    auto keep = std::make_shared<Table>(std::move(table));
+    TS_CUDA(cudaMemcpyAsync(dst, keep->data(), sizeof(typename Table::value_type) * keep->size(),
+                            cudaMemcpyHostToDevice, q));
+    host_tables.push_back(std::move(keep));
+  };
+  upload(d_inst, plan.inst, user);
+  upload(d_nb_inst, plan.nb_inst, user);
+  upload(d_nb_off, plan.nb_off, user);
+  upload(d_tb_inst, plan.tb_inst, user);
+  upload(d_tb_off, plan.tb_off, user);
   // CUDA-core slice products (FP64: the residuals on the DFMA engine and the whole cycle of a TS_FP64
   // batch on it; FP32: the inner products of TS_MIXED_FP32) run over a work list of (instance, slice,
   // row, column) tiles: warp-sized 8 x 4 tiles when every instance is tiny (a 64 x 64 tile of a
@@ -736,8 +746,8 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
       });
       TS_REQUIRE(items.size() < (size_t)INT32_MAX, "batch too large");
       int4* dev = (int4*)get(("b_items_" + std::to_string(bn)).c_str(), sizeof(int4) * items.size());
-      TS_CUDA(cudaMemcpy(dev, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
       simt.push_back(SimtList{bn, dev, (int)items.size()});
+      upload(dev, std::move(items), user);
     }
   }
   auto simt_list = [&](int bn) -> const SimtList& {
@@ -798,18 +808,16 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
     TS_REQUIRE(products.size() < (size_t)INT32_MAX && splits.size() < (size_t)INT32_MAX, "batch too large");
     char* tab = (char*)get("b_oz_tables", isz * count + sizeof(int4) * (products.size() + splits.size() + maxima.size()));
     int4* items = (int4*)(tab + isz * count);
-    TS_CUDA(cudaMemcpy(tab, table.data(), isz * count, cudaMemcpyHostToDevice));
-    TS_CUDA(cudaMemcpy(items, products.data(), sizeof(int4) * products.size(), cudaMemcpyHostToDevice));
-    oz_lists.products = items;
     oz_lists.n_products = (int)products.size();
-    items += products.size();
-    TS_CUDA(cudaMemcpy(items, splits.data(), sizeof(int4) * splits.size(), cudaMemcpyHostToDevice));
-    oz_lists.splits = items;
     oz_lists.n_splits = (int)splits.size();
-    items += splits.size();
-    TS_CUDA(cudaMemcpy(items, maxima.data(), sizeof(int4) * maxima.size(), cudaMemcpyHostToDevice));
-    oz_lists.maxima = items;
     oz_lists.n_maxima = (int)maxima.size();
+    oz_lists.products = items;
+    oz_lists.splits = items + products.size();
+    oz_lists.maxima = items + products.size() + splits.size();
+    upload(tab, std::move(table), user);
+    upload(items, std::move(products), user);
+    upload(items + oz_lists.n_products, std::move(splits), user);
+    upload(items + oz_lists.n_products + oz_lists.n_splits, std::move(maxima), user);
     oz_inst = tab;
     TS_CUDA(cudaMemsetAsync(tc_err, 0, sizeof(int) * 4, user));
   }
@@ -923,11 +931,6 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
       BTcInst* in_ = (BTcInst*)(((uintptr_t)(p_ + count) + 15) & ~(uintptr_t)15);
       int4* ti_ = (int4*)(((uintptr_t)(in_ + count) + 15) & ~(uintptr_t)15);
       int4* pi_ = ti_ + titems.size();
-      TS_CUDA(cudaMemcpy(m_, hmaps.data(), sizeof(TcMaps) * count, cudaMemcpyHostToDevice));
-      TS_CUDA(cudaMemcpy(p_, hplanes.data(), sizeof(BTcPlanes) * count, cudaMemcpyHostToDevice));
-      TS_CUDA(cudaMemcpy(in_, hinst.data(), sizeof(BTcInst) * count, cudaMemcpyHostToDevice));
-      TS_CUDA(cudaMemcpy(ti_, titems.data(), sizeof(int4) * titems.size(), cudaMemcpyHostToDevice));
-      TS_CUDA(cudaMemcpy(pi_, pitems.data(), sizeof(int4) * pitems.size(), cudaMemcpyHostToDevice));
       TcTables t;
       t.maps = m_;
       t.planes = p_;
@@ -936,6 +939,11 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
       t.pitems = pi_;
       t.n_titems = (int)titems.size();
       t.n_pitems = (int)pitems.size();
+      upload(m_, std::move(hmaps), st);
+      upload(p_, std::move(hplanes), st);
+      upload(in_, std::move(hinst), st);
+      upload(ti_, std::move(titems), st);
+      upload(pi_, std::move(pitems), st);
       return t;
     };
     tc_batch_preload(o.precision);   // shared-memory limits of the product kernels, before any launch

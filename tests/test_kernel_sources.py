@@ -23,3 +23,11 @@ def test_commits_come_from_the_issuing_lane():
             seen += 1
             assert text[:m.start()].endswith("@q "), (name, text[m.start():m.start() + 60])
     assert seen >= 3
+
+
+def test_host_tables_are_copied_in_stream_order():
+    """A plain cudaMemcpy from pageable memory may return before its copy is done, and its stream is not ordered with a
+    non-blocking one: whatever kernels read is copied by cudaMemcpyAsync on their stream or one they are ordered after."""
+    for name, text in SOURCES.items():
+        for m in re.finditer(r"cudaMemcpy\(([^;]*);", code(text)):
+            assert "cudaMemcpyHostToDevice" not in m.group(1), (name, m.group(0))
