@@ -216,7 +216,10 @@ typedef struct {
  * (TS_MIXED_FP32) or on the tcgen05 tensor cores (TS_MIXED_TF32, TS_MIXED_BF16, TS_MIXED_TF32X3);
  * the cycle's inner tolerance is opts->inner_tol (0: 1e-6 for FP32 and split TF32, 1e-3 TF32,
  * 1e-2 BF16).  opts->fp64_engine picks the engine of every FP64 product (the residuals, and the
- * whole cycle of a TS_FP64 batch): TS_ENGINE_DFMA or TS_ENGINE_OZAKI (opts->ozaki_digits).
+ * whole cycle of a TS_FP64 batch): TS_ENGINE_DFMA or TS_ENGINE_OZAKI (opts->ozaki_digits).  The
+ * emulated products' digits of X take up to 4 GiB of workspace (or one instance's, if that is more:
+ * 2 ozaki_digits (3 s round64(n) + 2 n round64(s)) (p / 2 + 1) bytes); larger batches go through
+ * them in groups.
  * The first call for a batch shape times the candidate launch shapes of its slice products (the
  * autotuner; see ts_tune_entries) before the cycle is captured; later calls reuse the choice.
  * opts->restart <= 128; dense operators with p <= 64.  infos / statuses (count entries each, may

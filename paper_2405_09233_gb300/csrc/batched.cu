@@ -43,6 +43,7 @@ namespace {
 // block of a sweep adds up its instance's partial sums and reduces its own, in FP64.
 long long stream_chunk(long long totN) { return totN >= 4ll * 152 * 8192 ? 8192 : 4096; }
 constexpr int kTubes = 256;       // tubes per DFT block (one per thread)
+constexpr size_t kOzBatchPlanes = 4ull << 30;   // bytes of the emulated products' digits of X
 
 struct BInst {
   double* X;
@@ -774,27 +775,51 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   const long long stride = state_stride(m);
   double* state = (double*)get("b_state", sizeof(double) * (size_t)stride * count);
   // Emulated FP64 products: digit planes of every operator, and the work lists of their three phases
-  // (maxima, digits of X, products), one launch each over all instances.  Everything is made before
+  // (maxima, digits of X, products), one launch each over a group of instances.  Everything is made before
   // anything is captured.  (A chain of five launches per instance on eight
   // side streams before: 64 instances, BF16 inner products, 29.7 -> 23.8 ms per solve.)
+  // A group's digits of X fit kOzBatchPlanes, so that they do not grow with the batch; where even that much memory
+  // is not to be had, they fit eight times the largest instance's.
   int* tc_err = (int*)get("tc_err", sizeof(int) * 4);
-  OzBatchLists oz_lists;
+  std::vector<OzBatchLists> oz_groups;
   const char* oz_inst = nullptr;
   unsigned long long* oz_mx = nullptr;
   size_t oz_mx_count = 0;
   if (ozaki) {
-    size_t plane_bytes = 0;
-    std::vector<size_t> poff(count), moff(count);
+    std::vector<size_t> poff(count), moff(count), bytes(count);
     std::vector<const ts_op*> cops(ops.begin(), ops.end());
+    size_t largest = 0;
     for (int i = 0; i < count; ++i) {
       oz_prepare(ops[i], oz_digits, user);
-      poff[i] = plane_bytes;
-      plane_bytes += oz_batch_plane_bytes(ops[i], oz_digits);
+      bytes[i] = oz_batch_plane_bytes(ops[i], oz_digits);
+      largest = std::max(largest, bytes[i]);
       moff[i] = oz_mx_count;
       oz_mx_count += ops[i]->K;
     }
     oz_preload();
-    char* planes = (char*)get("b_oz_planes", plane_bytes);
+    std::vector<int> ends;   // of the groups
+    auto make_groups = [&](size_t limit) {
+      size_t used = 0, most = 0;
+      ends.clear();
+      for (int i = 0; i < count; ++i) {
+        if (used > 0 && used + bytes[i] > limit) {
+          ends.push_back(i);
+          used = 0;
+        }
+        poff[i] = used;
+        used += bytes[i];
+        most = std::max(most, used);
+      }
+      ends.push_back(count);
+      return most;
+    };
+    char* planes = nullptr;
+    try {
+      planes = (char*)get("b_oz_planes", make_groups(kOzBatchPlanes));
+    } catch (const Error& e) {
+      if (e.status != TS_ERR_NOMEM) throw;
+      planes = (char*)get("b_oz_planes", make_groups(8 * largest));
+    }
     oz_mx = (unsigned long long*)get("b_oz_mx", sizeof(unsigned long long) * oz_mx_count);
     const size_t isz = oz_batch_instance_bytes();
     struct alignas(64) Line { char c[64]; };   // tensor maps are built 64-byte aligned
@@ -803,21 +828,36 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
     for (int i = 0; i < count; ++i)
       oz_batch_instance(ops[i], Xh64 + plan.inst[i].offS, Yh64 + plan.inst[i].offS, oz_digits, planes + poff[i],
                         oz_mx + moff[i], reinterpret_cast<char*>(table.data()) + isz * i);
-    std::vector<int4> products, splits, maxima;
-    oz_batch_items(cops, &products, &splits, &maxima);
-    TS_REQUIRE(products.size() < (size_t)INT32_MAX && splits.size() < (size_t)INT32_MAX, "batch too large");
-    char* tab = (char*)get("b_oz_tables", isz * count + sizeof(int4) * (products.size() + splits.size() + maxima.size()));
-    int4* items = (int4*)(tab + isz * count);
-    oz_lists.n_products = (int)products.size();
-    oz_lists.n_splits = (int)splits.size();
-    oz_lists.n_maxima = (int)maxima.size();
-    oz_lists.products = items;
-    oz_lists.splits = items + products.size();
-    oz_lists.maxima = items + products.size() + splits.size();
+    // one list of all groups' items, the three phases of a group one after the other
+    std::vector<int4> items;
+    std::vector<size_t> at;
+    int first = 0;
+    for (int end : ends) {
+      std::vector<int4> phase[3];
+      oz_batch_items(cops, first, end, &phase[0], &phase[1], &phase[2]);
+      for (const auto& q : phase) {
+        TS_REQUIRE(q.size() < (size_t)INT32_MAX, "batch too large");
+        at.push_back(items.size());
+        items.insert(items.end(), q.begin(), q.end());
+      }
+      first = end;
+    }
+    at.push_back(items.size());
+    char* tab = (char*)get("b_oz_tables", isz * count + sizeof(int4) * items.size());
+    int4* dev_items = (int4*)(tab + isz * count);
+    for (size_t g = 0; g < ends.size(); ++g) {
+      const size_t* a = at.data() + 3 * g;
+      OzBatchLists l;
+      l.products = dev_items + a[0];
+      l.splits = dev_items + a[1];
+      l.maxima = dev_items + a[2];
+      l.n_products = (int)(a[1] - a[0]);
+      l.n_splits = (int)(a[2] - a[1]);
+      l.n_maxima = (int)(a[3] - a[2]);
+      oz_groups.push_back(l);
+    }
     upload(tab, std::move(table), user);
-    upload(items, std::move(products), user);
-    upload(items + oz_lists.n_products, std::move(splits), user);
-    upload(items + oz_lists.n_products + oz_lists.n_splits, std::move(maxima), user);
+    upload(dev_items, std::move(items), user);
     oz_inst = tab;
     TS_CUDA(cudaMemsetAsync(tc_err, 0, sizeof(int) * 4, user));
   }
@@ -1000,8 +1040,8 @@ ts_status batched_entry(ts_ctx* ctx, int count, const ts_instance* insts, const 
   }
   // Emulated-FP64 slice products of every instance (Xh64 -> Yh64), each gated on the device by its flag.
   auto oz_all = [&](cudaStream_t s2, const int* gate) -> int {
-    oz_batch_products(oz_inst, oz_lists, oz_mx, oz_mx_count, oz_digits, gate, tc_err, s2);
-    return 3;
+    oz_batch_products(oz_inst, oz_groups, oz_mx, oz_mx_count, oz_digits, gate, tc_err, s2);
+    return 3 * (int)oz_groups.size();
   };
   auto inner_products = [&](cudaStream_t s2) -> int {
     // FP64 solve on the emulated engine: the Arnoldi products too (gated by the inner-cycle flag)

@@ -909,9 +909,10 @@ void oz_batch_instance(const ts_op* op, const double2* Xh, double2* Yh, int S, v
   o->lds = op->oz->lds;
 }
 
-void oz_batch_items(const std::vector<const ts_op*>& ops, std::vector<int4>* products, std::vector<int4>* splits,
-                    std::vector<int4>* maxima) {
-  for (int i = 0; i < (int)ops.size(); ++i) {
+void oz_batch_items(const std::vector<const ts_op*>& ops, int first, int end, std::vector<int4>* products,
+                    std::vector<int4>* splits, std::vector<int4>* maxima) {
+  const size_t sorted = products->size();
+  for (int i = first; i < end; ++i) {
     const int n = ops[i]->n, s = ops[i]->s, K = ops[i]->K, nyq = nyquist_index(ops[i]->p);
     for (int k = 0; k < K; ++k) {
       const int tn = oz_tile_cols(k, nyq);
@@ -924,7 +925,7 @@ void oz_batch_items(const std::vector<const ts_op*>& ops, std::vector<int4>* pro
     }
   }
   // largest first (a complex tile is twice a real one)
-  std::stable_sort(products->begin(), products->end(), [&](const int4& a, const int4& b) {
+  std::stable_sort(products->begin() + sorted, products->end(), [&](const int4& a, const int4& b) {
     auto cost = [&](const int4& q) {
       const ts_op* op = ops[q.x];
       return (oz_tile_cols(q.y, nyquist_index(op->p)) == kOzN ? 2.0 : 1.0) * (op->n + op->s);
@@ -933,14 +934,16 @@ void oz_batch_items(const std::vector<const ts_op*>& ops, std::vector<int4>* pro
   });
 }
 
-void oz_batch_products(const void* inst, const OzBatchLists& l, unsigned long long* mx, size_t mx_count, int S,
-                       const int* gate, int* err, cudaStream_t st) {
+void oz_batch_products(const void* inst, const std::vector<OzBatchLists>& groups, unsigned long long* mx,
+                       size_t mx_count, int S, const int* gate, int* err, cudaStream_t st) {
   const OzInstance* q = static_cast<const OzInstance*>(inst);
   TS_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * mx_count, st));
-  k_b_oz_maxabs<<<l.n_maxima, 256, 0, st>>>(q, l.maxima, gate);
-  k_b_oz_split<<<l.n_splits, kOzSplitThreads, oz_split_smem(S), st>>>(q, l.splits, gate);
-  k_oz_sylv<<<l.n_products, kOzThreads, kOzSmem, st>>>(OzMaps{}, OzOut{}, q, l.products, gate, err);
-  count_launch(3);
+  for (const OzBatchLists& l : groups) {
+    k_b_oz_maxabs<<<l.n_maxima, 256, 0, st>>>(q, l.maxima, gate);
+    k_b_oz_split<<<l.n_splits, kOzSplitThreads, oz_split_smem(S), st>>>(q, l.splits, gate);
+    k_oz_sylv<<<l.n_products, kOzThreads, kOzSmem, st>>>(OzMaps{}, OzOut{}, q, l.products, gate, err);
+    count_launch(3);
+  }
   TS_CUDA(cudaGetLastError());
 }
 

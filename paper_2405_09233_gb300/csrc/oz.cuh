@@ -43,10 +43,11 @@ void oz_preload();
 void oz_products(const ts_op* op, const double2* Xh, double2* Yh, int S, const OzBuffers& b, int* err,
                  cudaStream_t st);
 
-// Batches: the products of many instances in one launch per phase, each instance gated on the device by
-// its flag.  oz_batch_instance fills one entry (oz_batch_instance_bytes each, 64-byte aligned) of the
-// instance table in host memory: digit planes carved from `planes` (oz_batch_plane_bytes), maxima at mx (K
-// entries).  oz_batch_items lists the work of the three phases; the caller copies both to the device.
+// Batches: the products of many instances in one launch per phase and group of instances, each instance gated
+// on the device by its flag.  The groups share one buffer of digit planes, one after the other.  oz_batch_instance
+// fills one entry (oz_batch_instance_bytes each, 64-byte aligned) of the instance table in host memory: digit
+// planes carved from `planes` (oz_batch_plane_bytes), maxima at mx (K entries).  oz_batch_items appends the work of
+// the three phases of the instances first .. end - 1; the caller copies table and lists to the device.
 struct OzBatchLists {
   const int4* products = nullptr;
   const int4* splits = nullptr;
@@ -57,10 +58,10 @@ size_t oz_batch_instance_bytes();
 size_t oz_batch_plane_bytes(const ts_op* op, int S);
 void oz_batch_instance(const ts_op* op, const double2* Xh, double2* Yh, int S, void* planes, unsigned long long* mx,
                        void* out);
-void oz_batch_items(const std::vector<const ts_op*>& ops, std::vector<int4>* products, std::vector<int4>* splits,
-                    std::vector<int4>* maxima);
-void oz_batch_products(const void* inst, const OzBatchLists& l, unsigned long long* mx, size_t mx_count, int S,
-                       const int* gate, int* err, cudaStream_t st);
+void oz_batch_items(const std::vector<const ts_op*>& ops, int first, int end, std::vector<int4>* products,
+                    std::vector<int4>* splits, std::vector<int4>* maxima);
+void oz_batch_products(const void* inst, const std::vector<OzBatchLists>& groups, unsigned long long* mx,
+                       size_t mx_count, int S, const int* gate, int* err, cudaStream_t st);
 // Y = M(X) in FP64 through the emulated product (same contract as apply_f64), with S digits per
 // value; the operator's digit planes are prepared (once) with S_op >= S digits.
 void apply_f64_oz(ts_ctx* ctx, const ts_op* op, const double* X, double* Y, int mode, const double* C,
