@@ -301,7 +301,8 @@ struct GridItems {
   }
 };
 template <int BN, int ESZ, int PARTS, typename Items>
-__device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* err) {
+__device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* err, int stall,
+                                           unsigned long long wait_ns) {
   using Cfg = TcCfg<BN, ESZ>;
   constexpr int kCols = 2 * Cfg::kTmemCols;   // two accumulator sets of (Re, Im)
   static_assert(kCols <= 512, "tensor memory");
@@ -356,10 +357,11 @@ __device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* er
         for (int u = 0; u < iters; ++u, ++g) {
           const int slot = (int)(g % Cfg::kStages);
           const uint32_t phase = (uint32_t)(g / Cfg::kStages) & 1u;
-          if (!mbar_wait(bar_empty + 8 * slot, phase ^ 1u, err, 1)) {
+          if (!mbar_wait(bar_empty + 8 * slot, phase ^ 1u, err, 1, wait_ns)) {
             ok = false;
             break;
           }
+          if (stall) continue;   // test aid: arm no stage, so the MMA warp's wait expires
           const uint32_t full = bar_full + 8 * slot;
           mbar_expect_tx(full, real ? Cfg::kTileA + Cfg::kTileB : Cfg::kStage);
           const uint32_t sA = base + slot * Cfg::kStage;
@@ -387,7 +389,7 @@ __device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* er
         }
       }
       for (long long u = issued > Cfg::kStages ? issued - Cfg::kStages : 0; u < issued; ++u)
-        mbar_wait(bar_full + 8 * (int)(u % Cfg::kStages), (uint32_t)(u / Cfg::kStages) & 1u, err, 4);
+        mbar_wait(bar_full + 8 * (int)(u % Cfg::kStages), (uint32_t)(u / Cfg::kStages) & 1u, err, 4, wait_ns);
     }
   } else if (warp == 5) {
     constexpr int fmt = ESZ == 2 ? 1 : 2;
@@ -404,7 +406,7 @@ __device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* er
       const int it1 = (b.n + Cfg::kElemsK - 1) / Cfg::kElemsK, iters = iters_of(b);
       const int set = t & 1;
       // the epilogue has drained this accumulator set's previous item (t - 2)
-      if (t >= 2 && !mbar_wait_warp(bar_acce + 8 * set, (uint32_t)((t >> 1) + 1) & 1u, err, 6)) {
+      if (t >= 2 && !mbar_wait_warp(bar_acce + 8 * set, (uint32_t)((t >> 1) + 1) & 1u, err, 6, wait_ns)) {
         ok = false;
         break;
       }
@@ -413,7 +415,7 @@ __device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* er
       for (int u = 0; u < iters; ++u, ++g) {
         const int slot = (int)(g % Cfg::kStages);
         const uint32_t phase = (uint32_t)(g / Cfg::kStages) & 1u;
-        if (!mbar_wait_warp(bar_full + 8 * slot, phase, err, 2)) {
+        if (!mbar_wait_warp(bar_full + 8 * slot, phase, err, 2, wait_ns)) {
           ok = false;
           break;
         }
@@ -427,7 +429,7 @@ __device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* er
     }
     // every MMA issued (also on an error path) completes before tensor memory is freed
     mma_commit_one(one, bar_done);
-    mbar_wait(bar_done, 0u, err, 5);
+    mbar_wait(bar_done, 0u, err, 5, wait_ns);
     __syncwarp();
   } else {
     // Epilogue: warp w reads TMEM lanes 32w..32w+31 (= output rows i0 + 32w + lane) of set t & 1.
@@ -438,7 +440,7 @@ __device__ __forceinline__ void tc_persist(const Items& src, int nitems, int* er
       const int k = b.k, i0 = b.i0, j0 = b.j0;
       const bool real = (k == 0) || (k == b.nyq);
       const int set = t & 1;
-      if (!mbar_wait(bar_accf + 8 * set, (uint32_t)(t >> 1) & 1u, err, 3)) break;
+      if (!mbar_wait(bar_accf + 8 * set, (uint32_t)(t >> 1) & 1u, err, 3, wait_ns)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int row = i0 + warp * 32 + lane;
       float2* Yk = b.Y + (long long)k * b.n * b.s;
@@ -479,13 +481,13 @@ template <int BN, int ESZ, int PARTS>
 __global__ void __launch_bounds__(192, 1)
     k_b_tc_persist(const TcMaps* __restrict__ maps, const BTcInst* __restrict__ inst, const int* __restrict__ active,
                    const int4* __restrict__ items, int nitems, int* err) {
-  tc_persist<BN, ESZ, PARTS>(BatchItems{maps, inst, active, items}, nitems, err);
+  tc_persist<BN, ESZ, PARTS>(BatchItems{maps, inst, active, items}, nitems, err, 0, kWaitNs);
 }
 template <int BN, int ESZ, int PARTS>
 __global__ void __launch_bounds__(192, 1)
     k_tc_persist(const __grid_constant__ TcMaps maps, float2* __restrict__ Y, int n, int s, int K, int nyq, int ni,
-                 int nj, int* err) {
-  tc_persist<BN, ESZ, PARTS>(GridItems<BN>{&maps, Y, n, s, nyq, K, ni, nj}, ni * nj * K, err);
+                 int nj, int* err, int stall, unsigned long long wait_ns) {
+  tc_persist<BN, ESZ, PARTS>(GridItems<BN>{&maps, Y, n, s, nyq, K, ni, nj}, ni * nj * K, err, stall, wait_ns);
 }
 
 // Planar copies of the FP32 spectra of a batch: per (instance, slice, 32 x 32 tile) work item,
@@ -737,9 +739,10 @@ void launch_tc(const TcMaps& maps, float2* Y, int n, int s, int K, int nyq, int*
       PARTS * ((n + Cfg::kElemsK - 1) / Cfg::kElemsK + (long long)(s + Cfg::kElemsK - 1) / Cfg::kElemsK);
   if constexpr (BN <= 128) {
     const int sms = device_sms();
-    if (!stall && stages <= 256 && ni * nj * K > sms && ni * nj * K <= INT32_MAX) {
+    if (stages <= 256 && ni * nj * K > sms && ni * nj * K <= INT32_MAX) {
       set_max_dynamic_smem((const void*)k_tc_persist<BN, ESZ, PARTS>, Cfg::kSmem);
-      k_tc_persist<BN, ESZ, PARTS><<<sms, 192, Cfg::kSmem, st>>>(maps, Y, n, s, K, nyq, (int)ni, (int)nj, err);
+      k_tc_persist<BN, ESZ, PARTS><<<sms, 192, Cfg::kSmem, st>>>(maps, Y, n, s, K, nyq, (int)ni, (int)nj, err, stall,
+                                                                      wait_ns);
       count_launch();
       TS_CUDA(cudaGetLastError());
       return;
