@@ -290,9 +290,11 @@ ts_status ts_tune_entries(ts_ctx* ctx, char* buf, size_t cap, size_t* needed);
  * by CUDA events recorded on the launching stream around each timed launch. */
 typedef struct {
   long long launches;      /* libtstar kernels launched since the last ts_stats_reset */
-  long long gemm_launches; /* FP64 per-Fourier-slice GEMM launches timed while enabled */
+  long long gemm_launches; /* FP64 per-Fourier-slice GEMM launches timed while enabled.  A small operator's
+                              whole application is one launch: it counts here, its DFTs included */
   double gemm_ms;          /* their summed event durations */
-  double gemm_flops;       /* their algorithmic FLOPs: 8 per complex and 2 per real multiply-add */
+  double gemm_flops;       /* their algorithmic FLOPs: 8 per complex and 2 per real multiply-add (and
+                              2.5 p log2 p per tube and DFT of a whole application) */
   long long lowp_launches; /* low-precision slice GEMM launches (FP32 CUDA cores or tcgen05) */
   double lowp_ms;
   double lowp_flops;

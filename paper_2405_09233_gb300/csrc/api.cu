@@ -1,5 +1,6 @@
 // Context, workspace, operator setup and the operator-level entry points of libtstar:
 // ts_tstar (Definition 2.1 via Algorithm 1) and ts_sylv_apply (Eq. (2)).
+#include <cmath>
 #include <cstring>
 #include <cstdio>
 #include <algorithm>
@@ -390,10 +391,10 @@ void apply_f64(ts_ctx* ctx, const ts_op* op, const double* X, double* Y, int mod
     return;
   }
   KernelTimer& tm = ctx->timer;
-  // One launch where that is the cheaper form; an application in place needs X whole until it is transformed.
+  // One launch where that is the cheaper form; where X and Y overlap, X is needed whole until it is transformed.
   const int tn = X + T * p <= Y || Y + T * p <= X ? apply_small_tile(n, s, p) : 0;
-  if (tn) {
-    tm.begin(st, 0, gemm_flops(n, s, n, s, K, nyquist_index(p)));
+  if (tn) {   // booked whole, both transforms with the products
+    tm.begin(st, 0, gemm_flops(n, s, n, s, K, nyquist_index(p)) + 2.0 * T * 2.5 * p * std::log2((double)p));
     apply_small_f64(op, tn, X, Y, mode == IRFFT_RESIDUAL ? C : nullptr, partials, st, gate);
     tm.end(st);
     return;
