@@ -3,12 +3,12 @@
 //
 // All instances advance in lockstep through the restart cycle of Algorithm 3; every phase is ONE
 // launch over all instances:
-//   * streaming phases (scaling, inner products, MGS passes, X += V (*) y) run over a block table
-//     in which every block belongs to one instance (a chunk of its N = n s p unknowns), so each
-//     instance's inner product is the fixed-order sum of its own blocks' partials;
+//   * streaming phases (scaling, norms, passes of the Gram-Schmidt sweep, X += V (*) y) run over a
+//     block table in which every block belongs to one instance (a chunk of its N = n s p unknowns), so
+//     each instance's inner products are fixed-order sums of its own blocks' partials;
 //   * the mode-3 DFTs run over a tube-block table (one tube per thread, the instance's p);
-//   * the per-slice products run over a work list of (instance, Fourier slice, 64 x 64 tile)
-//     items, ordered by cost (largest first) so the tail of the launch stays short;
+//   * the per-slice products run over a work list of (instance, Fourier slice, tile) items, ordered
+//     by cost (largest first) so the tail of the launch stays short;
 //   * the Givens update is one block per instance.
 // Masks on the device (cycle participation, still iterating) let an instance stop its inner cycle
 // early or drop out of the batch without changing the launch sequence, so one restart cycle is
@@ -314,9 +314,9 @@ constexpr int kBatchSimtBM = 64;   // rows of a work-list tile of the CUDA-core 
 // --- per-slice products over the work list ---------------------------------------------------------
 // TILE 0: every instance has n, s <= kTinyL and the items are 8 x 4 tiles for kTinyThreads
 // (gemm_tiny_tile); otherwise 64 x TILE tiles (TILE = 64, 32 or 16 columns): 256 threads in FP64
-// (gemm_tile_f64), one per 8 x 4 block in FP32 (gemm_tile_f32).  Every TILE > 0 sums each output entry's products in the same order
-// (phase 1's reduction index, then phase 2's), so the column width, which the autotuner picks,
-// changes which CTA forms an entry and how much padding it computes, never the entry's value.
+// (gemm_tile_f64), one per 8 x 4 block in FP32 (gemm_tile_f32).  Every TILE > 0 sums each output entry's
+// products in the same order (phase 1's reduction index, then phase 2's), so the column width, which the
+// autotuner picks, changes which CTA forms an entry and how much padding it computes, never the entry's value.
 template <typename Real, int TILE>
 constexpr int b_gemm_threads() {
   return TILE == 0 ? kTinyThreads : (sizeof(Real) == 8 ? 256 : kBatchSimtBM * TILE / 32);
@@ -506,7 +506,8 @@ void preload_cycle_kernels() {
       (const void*)k_b_ks_init, (const void*)k_b_scale_R<T>, (const void*)k_b_rfft<T, Real2, 0, 0>,
       (const void*)k_b_gemm<T, 0, 0>, (const void*)k_b_gemm<T, 0, 64>, (const void*)k_b_gemm<T, 0, 32>,
       (const void*)k_b_gemm<T, 0, 16>, (const void*)k_b_irfft<T, Real2, 0>,
-      (const void*)k_b_gs_pass<T, 4>, (const void*)k_b_gs_pass<T, 8>, (const void*)k_b_givens, (const void*)k_b_scale_W<T>, (const void*)k_b_solve_y,
+      (const void*)k_b_gs_pass<T, 4>, (const void*)k_b_gs_pass<T, 8>, (const void*)k_b_givens,
+      (const void*)k_b_scale_W<T>, (const void*)k_b_solve_y,
       (const void*)k_b_axpy<T>, (const void*)k_b_rfft<double, double2, 1, 1>, (const void*)k_b_gemm<double, 1, 0>,
       (const void*)k_b_gemm<double, 1, 64>, (const void*)k_b_gemm<double, 1, 32>, (const void*)k_b_gemm<double, 1, 16>,
       (const void*)k_b_irfft<double, double2, 1>, (const void*)k_b_finalize_norm, (const void*)k_b_any_active};

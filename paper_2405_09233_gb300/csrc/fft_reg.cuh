@@ -68,8 +68,7 @@ __device__ __forceinline__ Real mul2_sub(Real a, Real b, Real c, Real d) {
 
 // One radix-2 stage of span LEN, then the next; LEN is a template argument so that every register
 // index is a compile-time constant (a runtime stage loop leaves the arrays in local memory).
-// TSTR: stride into the roots of unity (2 when a length-P/2 FFT uses those of length P).
-template <typename Real, int P, bool INVERSE, int LEN, int TSTR = 1>
+template <typename Real, int P, bool INVERSE, int LEN>
 struct FftStages {
   template <int Q, int START>
   static __device__ __forceinline__ void butterfly(Real (&xr)[P], Real (&xi)[P]) {
@@ -111,11 +110,11 @@ struct FftStages {
   }
   static __device__ __forceinline__ void run(Real (&xr)[P], Real (&xi)[P]) {
     all<0>(xr, xi);
-    FftStages<Real, P, INVERSE, 2 * LEN, TSTR>::run(xr, xi);
+    FftStages<Real, P, INVERSE, 2 * LEN>::run(xr, xi);
   }
 };
-template <typename Real, int P, bool INVERSE, int TSTR>
-struct FftStages<Real, P, INVERSE, 2 * P, TSTR> {
+template <typename Real, int P, bool INVERSE>
+struct FftStages<Real, P, INVERSE, 2 * P> {
   static __device__ __forceinline__ void run(Real (&)[P], Real (&)[P]) {}
 };
 
@@ -154,7 +153,7 @@ __device__ __forceinline__ void rfft_reg(Load load, Store store) {
       zr[bitrevc(t, LB)] = load(2 * t);
       zi[bitrevc(t, LB)] = load(2 * t + 1);
     }
-    FftStages<Real, M, false, 2, 2>::run(zr, zi);
+    FftStages<Real, M, false, 2>::run(zr, zi);
     store(0, zr[0] + zi[0], Real(0));
     store(M, zr[0] - zi[0], Real(0));
 #pragma unroll
@@ -241,7 +240,7 @@ __device__ __forceinline__ void irfft_reg(Load load, Store store) {
         }
       }
     }
-    FftStages<Real, M, true, 2, 2>::run(zr, zi);
+    FftStages<Real, M, true, 2>::run(zr, zi);
 #pragma unroll
     for (int t = 0; t < M; ++t) {
       store(2 * t, zr[t]);

@@ -2,9 +2,8 @@
 // it is the fused Y_k = A_k X_k - X_k B_k of Eq. (2) in the Fourier domain).
 //
 // GB300 runs FP64 at ~1 TFLOP/s on CUDA cores (DFMA and the m8n8k4 DMMA measure within 4% of
-// each other), so this kernel is FP64-pipe bound by a wide margin: a 64x64 output tile with
-// 16x16 threads of 4x4 outputs reuses every shared-memory operand 4 times, and the global
-// traffic is ~1/100 of what the pipe could hide.  The one lever that matters is the number of
+// each other), so the FP64 product is FP64-pipe bound by a wide margin and its tiles are free to
+// follow the problem's shape (gemm_tile.cuh; launch_cheapest picks them).  What matters is the number of
 // FP64 operations: the complex product uses three real products (Gauss):
 //   T1 = sum ar*br, T2 = sum ai*bi, T3 = sum (ar+ai)(br+bi);  re = T1 - T2, im = T3 - T1 - T2,
 // 3 DFMA per complex multiply-add instead of 4.  The sums ar+ai, br+bi are formed once per

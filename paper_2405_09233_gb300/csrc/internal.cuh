@@ -225,7 +225,7 @@ void spec_weight(const double2* in, double2* out, long long T, int p, bool inver
                  cudaStream_t st);
 
 // ---------------- per-slice complex GEMM on CUDA cores, FP64 / FP32 (gemm_simt.cu) ----------------
-// Y_k = A1_k B1_k + sgn2 * A2_k B2_k for k < K (phase 2 skipped when L2 == 0);
+// Y_k = A1_k B1_k + sgn2 * A2_k B2_k for k < K, sgn2 +1 or -1 (phase 2 skipped when L2 == 0);
 // slices k == 0 and k == nyq are treated as real (imaginary parts ignored, result imag = 0).
 template <typename Cplx>
 struct GemmArgs {
@@ -281,7 +281,6 @@ void arnoldi_step(T* W, T* V, long long ldv, long long N, int j, int m, void* st
                   cudaStream_t st, cudaGraphConditionalHandle handle = 0, const double* stop = nullptr,
                   int* gate = nullptr);
 // Device addresses inside the state block.
-double* ks_H(void* state, int m);          // column-major (m+1) x m, H[i + (m+1)*j]
 double* ks_y(void* state, int m);
 double* ks_est(void* state, int m);        // [0] = estimate, [1] = 1/h_{j+1,j}, [2] = h_{j+1,j}, [3] = flags,
                                            // [4] = steps taken in the cycle

@@ -54,7 +54,7 @@ __global__ void k_ks_init(double* st, int m, const double* beta_in) {
 }
 
 // est[0] = estimate, est[1] = 1/h_{j+1,j}, est[2] = h_{j+1,j}, est[3] = flags (1 breakdown,
-// 2 singular, 4 non-finite), est[4] = steps taken in this cycle (j + 1), est[8 + j] = estimate of
+// 2 singular, 4 non-finite), est[4] = steps taken in this cycle (j + 1); hist[j] = estimate of
 // step j.  In a graph-captured cycle, `handle` is the conditional handle of step j + 1 (0 for the
 // last step) and the update decides whether the cycle goes on: it sets that handle to 0 on breakdown,
 // a bad step, an estimate <= stop[0] (the tolerance times ||C||) or <= stop[1] (the inner tolerance
@@ -212,7 +212,7 @@ __device__ __forceinline__ void ks_finish(const KsStage& S, double* st, int m, i
 //
 // Bound by FP64 issue (64 clocks per warp instruction and sub-partition) and by the reduction's round trip.
 // The 20 steps of a cycle, vector by vector -> by blocks: 2304 FP64 entries 517 -> 260 us, 8000 FP64 931 ->
-// 448, 8000 FP32 861 -> 294.
+// 448, 8000 FP32 861 -> 294 (with FP64 sums over eight products; Triples over two take 2% less).
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -406,10 +406,11 @@ __global__ void __launch_bounds__(kArnThreads, 1)
 // two more.  Pass b = -1 forms the first block's inner products; pass b subtracts block b and forms those of
 // block b + 1, or ||W||^2 after the last.  A CTA writes its sums to P[sum][CTA]; the next launch adds them
 // up in every CTA (in the same order, so all have the same coefficients).
-// Bound by memory from about a million entries on (FP32: 16.8M entries, 20 steps move 37.6 GB in 6.4 ms), by
+// Bound by memory from about a million entries on (FP32: 16.8M entries, 20 steps move 37.6 GB in 6.6 ms), by
 // round trips below.  The sweeps of a 20-step cycle, against a launch per basis vector (reading W, V_i and
 // V_i+1, writing W) above 65536 entries and one cluster launch per step below: FP64, 61440 entries 1877 ->
-// 542 us, 262144 1534 -> 745, 4.2M 8474 -> 5556; FP32, 1.05M 1944 -> 888, 16.8M 10303 -> 6427.  The line to
+// 542 us, 262144 1534 -> 745, 4.2M 8474 -> 5556; FP32, 1.05M 1944 -> 888, 16.8M 10303 -> 6427 (sums in two
+// FP32 parts; in three, 3% more).  The line to
 // the cluster form lies where both take the same time (FP64, 8000 entries in the cluster 457 us, 8200 here 451).
 constexpr int kGsBlocks = 152;
 
@@ -513,7 +514,6 @@ __global__ void k_ks_solve(double* st, int m, int k) {
 }  // namespace
 
 size_t krylov_state_bytes(int m) { return Layout{m}.total() * sizeof(double); }
-double* ks_H(void* s, int m) { return static_cast<double*>(s) + Layout{m}.H(); }
 double* ks_y(void* s, int m) { return static_cast<double*>(s) + Layout{m}.y(); }
 double* ks_est(void* s, int m) { return static_cast<double*>(s) + Layout{m}.est(); }
 double* ks_beta(void* s, int m) { return static_cast<double*>(s) + Layout{m}.beta(); }
