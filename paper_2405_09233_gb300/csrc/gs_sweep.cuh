@@ -5,7 +5,9 @@
 // <V_i, V_l>: h_i = <V_i, W - sum_{l<i} h_l V_l> written out.  So one reduction gives eight coefficients where
 // a sweep vector by vector waits for eight, each behind the other; the Gram row of V_j (at most 7 more inner
 // products) is formed once, in step j, whose last block it completes.  The result is modified Gram-Schmidt's
-// up to rounding: the estimates of every step agree with FP64 MGS's to 1e-12 ||C|| in the tests.
+// up to rounding: the estimates of every step agree with FP64 MGS's to 1e-12 ||C|| in the tests, and the basis
+// loses orthogonality alike (||V^T V - I|| after 40 steps at n = 400, condition 1e4, the two sweeps written out in
+// numpy: FP64 1.9e-13 vector by vector, 2.5e-13 by blocks; FP32 5.9e-5 and 6.6e-5).
 #pragma once
 #include <cuda_runtime.h>
 #include <type_traits>
