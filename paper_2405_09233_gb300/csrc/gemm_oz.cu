@@ -146,7 +146,7 @@ __host__ __device__ constexpr int oz_sub(int S) { return 2 * S <= kOzSlots ? 2 :
 // M, 256 times 7 x 2^20 plus 2^23.
 // The epilogue sets the pace together with the MMAs, so it exists once per set of forms: with all of them in one,
 // n = s = 1024, p = 16 and 6 digits took 2.72 to 2.82 ms, not 2.69.
-// There, before the lowest bits were kept and now: 5 digits 2.40 / 2.48 ms, 4 digits 1.69 / 1.70, 3 digits 1.33 / 1.31.
+// There, before the lowest bits were kept and now: 5 digits 2.40 / 2.43 ms, 4 digits 1.69 / 1.69, 3 digits 1.33 / 1.32.
 constexpr uint32_t kOzMagic = 0x4B400000u;   // pattern of 1.5 2^23; 2^e times it: + e 2^23
 enum { kOzPattern, kOzConvert, kOzShift };
 // The last form that some unit of a product takes.
@@ -170,7 +170,7 @@ __device__ __forceinline__ OzScale oz_scale(int F, int S, int gb, bool lone) {
   else q.mode = sb >= 0 && (gb - 1) * oz_sub(S) > 4 ? kOzConvert : kOzPattern;
   q.M = __uint_as_float(pat);
   q.fa = sa < 0 ? __uint_as_float((uint32_t)(127 + sa) << 23) : 1.f;
-  q.ca = lone ? 0 : (sb >= 0 ? 256 : (sa > 0 ? 1 << sa : 1));
+  q.ca = FORMS == kOzPattern && lone ? 0 : (sb >= 0 ? 256 : (sa > 0 ? 1 << sa : 1));
   q.m = sb <= 0 ? 1 : 1 << (sb > 30 ? 30 : sb);
   q.reps = sb > 30 ? 1 << (sb - 30) : 1;
   q.sh = sb;
@@ -341,12 +341,7 @@ __device__ __noinline__ void oz_drain(const OzOut& o, uint32_t tmem, uint32_t ba
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tb = lane_base + (uint32_t)(bb * 2 * kOzN), ta = lane_base + (uint32_t)(ba * 2 * kOzN);
       // 8 columns at a time: little room beside the accumulators
-      if (FORMS == kOzPattern || (sc.mode == kOzPattern && !lone)) {
-        for (int r = 0; r < sc.reps; ++r) {
-          acc_add<kOzPattern>(ar, ta, tb, sc);
-          acc_add<kOzPattern>(ai, ta + kOzN, tb + kOzN, sc);
-        }
-      } else if (lone) {
+      if (FORMS != kOzPattern && lone) {
         if (sc.mode == kOzPattern) {
           acc_add_lone<kOzPattern>(ar, tb, sc);
           acc_add_lone<kOzPattern>(ai, tb + kOzN, sc);
@@ -356,6 +351,11 @@ __device__ __noinline__ void oz_drain(const OzOut& o, uint32_t tmem, uint32_t ba
         } else {
           acc_add_lone<kOzShift>(ar, tb, sc);
           acc_add_lone<kOzShift>(ai, tb + kOzN, sc);
+        }
+      } else if (FORMS == kOzPattern || sc.mode == kOzPattern) {
+        for (int r = 0; r < sc.reps; ++r) {
+          acc_add<kOzPattern>(ar, ta, tb, sc);
+          acc_add<kOzPattern>(ai, ta + kOzN, tb + kOzN, sc);
         }
       } else if (FORMS == kOzConvert || sc.mode == kOzConvert) {
         acc_add<kOzConvert>(ar, ta, tb, sc);
